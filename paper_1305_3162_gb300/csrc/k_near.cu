@@ -8,11 +8,19 @@
 //   EXPSUM:    (N - N_s)(r) = (1/r - sum_k w_k exp(-g_k r^2)) / (4 pi)  (r < eps,
 //              the exponential sum of Sec. 3.3).
 //
-// One warp per work item: lane t owns target tbegin + t; the warp walks the
-// item's source ranges 32 sources at a time, staging them in shared memory
-// and broadcasting each to all lanes.  Pair distances are formed from the
+// One warp per work item: lanes t and t + 16 own target tbegin + t; the warp
+// walks the item's source ranges 32 sources at a time, staging them in shared
+// memory and broadcasting each to the lanes of one half, the halves taking
+// sources in turn.  Pair distances are formed from the
 // integer cell difference plus the fractional offsets, so they keep full
 // precision however far the mesh sits from the origin.
+//
+// RADIAL plans (every FP32 plan and most FP64 ones) run k_near_radial32 and
+// k_near_radial64, which write the kernel as
+//   erfc(a r) / r = 1 / r - a E(a^2 r^2),  E(x) = erf(sqrt x) / sqrt x,
+// E being smooth on [0, (a eps)^2]: one polynomial in r^2 in FP32, a table of
+// short ones in FP64.  The general kernel k_near takes the other modes, and
+// RADIAL plans whose a eps lies outside the fits' range.
 #include "dev_common.cuh"
 
 namespace slp {
@@ -60,11 +68,12 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near(DevPlan p) {
     const int item = blockIdx.x * NEAR_WARPS + warp;
     if (item >= p.n_near) return;
     const NearItem it = p.near_items[item];
-    const bool active = lane < it.tcount;
+    const int half = lane / NEAR_TARGETS, tl = lane % NEAR_TARGETS;
+    const bool active = tl < it.tcount;
     int ctx = 0, cty = 0, ctz = 0;
     T ftx = T(0), fty = T(0), ftz = T(0);
     if (active) {
-        const T4 g = ((const T4 *)p.tgt_grid)[it.tbegin + lane];
+        const T4 g = ((const T4 *)p.tgt_grid)[it.tbegin + tl];
         unpack_cell(packed_cell(g.w), ctx, cty, ctz);
         ftx = g.x;
         fty = g.y;
@@ -73,6 +82,7 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near(DevPlan p) {
     const T hx = (T)p.h[0], hy = (T)p.h[1], hz = (T)p.h[2];
     const T eps2 = (T)p.eps2;
     const T a = (T)p.inv_s_sqrt2;
+    const T iLx = T(1) / T(p.L[0]), iLy = T(1) / T(p.L[1]), iLz = T(1) / T(p.L[2]);  // exact: powers of two
     const T4 *src = (const T4 *)p.src_grid;
     const T *qb = (const T *)p.qbuf;
     T acc = T(0);
@@ -86,7 +96,7 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near(DevPlan p) {
             }
             __syncwarp();
             const int cnt = min(32, rg.y - s0);
-            for (int j = 0; j < cnt; ++j) {
+            for (int j = half; j < cnt; j += 2) {
                 const T4 g = sg[warp][j];
                 int csx, csy, csz;
                 unpack_cell(packed_cell(g.w), csx, csy, csz);
@@ -105,9 +115,9 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near(DevPlan p) {
                                (near_rsqrt(r2) - expsum_value((const T *)p.es_w, (const T *)p.es_g, p.es_n, r2));
                 } else {
                     const T ri = near_rsqrt(r2);
-                    const T ux = (T(ctx - csx) + (ftx - g.x)) / T(p.L[0]);
-                    const T uy = (T(cty - csy) + (fty - g.y)) / T(p.L[1]);
-                    const T uz = (T(ctz - csz) + (ftz - g.z)) / T(p.L[2]);
+                    const T ux = (T(ctx - csx) + (ftx - g.x)) * iLx;
+                    const T uy = (T(cty - csy) + (fty - g.y)) * iLy;
+                    const T uz = (T(ctz - csz) + (ftz - g.z)) * iLz;
                     const T kn = sep_factor((const T *)p.sep_h[0], p.sep_nh[0], ux) *
                                  sep_factor((const T *)p.sep_h[1], p.sep_nh[1], uy) *
                                  sep_factor((const T *)p.sep_h[2], p.sep_nh[2], uz);
@@ -117,12 +127,240 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near(DevPlan p) {
             __syncwarp();
         }
     }
-    if (active) {
+    acc += __shfl_xor_sync(0xffffffffu, acc, NEAR_TARGETS);
+    if (lane < it.tcount) {
         const T v = acc * T(0.079577471545947667884);  // 1 / (4 pi)
         if (p.deterministic)
             ((T *)p.phi_near)[(int64_t)item * 32 + lane] = v;
         else
             atomicAdd((T *)p.phi_part + it.tbegin + lane, v);
+    }
+}
+
+// ---------------------------------------------------------------- RADIAL, fitted kernels
+// What bounds both: arithmetic (sources and targets are read once per item
+// and stay in L1/L2).  Both walk the sources of an item 32 at a time, one per
+// lane, and first drop those farther than eps from the box around the warp's
+// targets (the work list culls whole 2x2x2-cell bins only), so the inner loop
+// runs over the kept ones, packed by ballot.  Positions are relative to the
+// cell of the warp's first target: integer part and fraction separately in
+// FP32, whose differences are exact; their sum in FP64.
+
+// Keep this lane's source?  Distance from the targets' box, in cells of x, in
+// FP32 with a margin far above its rounding.
+__device__ __forceinline__ bool in_reach(const float (&lo)[3], const float (&hi)[3], float x, float y, float z,
+                                         float ry, float rz, float reach2) {
+    const float dx = fmaxf(0.f, fmaxf(lo[0] - x, x - hi[0]));
+    const float dy = fmaxf(0.f, fmaxf(lo[1] - y, y - hi[1])) * ry;
+    const float dz = fmaxf(0.f, fmaxf(lo[2] - z, z - hi[2])) * rz;
+    return dx * dx + dy * dy + dz * dz <= reach2;
+}
+__device__ __forceinline__ void warp_box(float v, float &lo, float &hi) {
+    lo = hi = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// FP32: a lane takes two sources per step in paired operations.  Per pair: 9 subtractions
+// (integer and fractional parts), 5 operations for r^2, one reciprocal square
+// root, the degree-13 polynomial of a E (14 multiply-adds, its argument's map
+// included), 2 for the sum: 30 lane operations where erfcf, the integer
+// conversions and the cell arithmetic per pair took about 180.  Level-5 sphere
+// at 128^3 (118M lane pairs after the cull, 73M inside eps): 670 -> 164 us.
+__global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial32(DevPlan p) {
+    __shared__ __align__(16) float2 st[NEAR_WARPS][16][10];  // per source pair: -H xyz, -f xyz, charge (80-byte
+                                                             // rows: stores 2-way instead of 8-way on the banks)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int item = blockIdx.x * NEAR_WARPS + warp;
+    pdl_wait();
+    pdl_trigger();
+    if (item >= p.n_near) return;
+    const NearItem it = p.near_items[item];
+    const int half = lane / NEAR_TARGETS;
+    const float4 tg = ((const float4 *)p.tgt_grid)[it.tbegin + min(lane % NEAR_TARGETS, it.tcount - 1)];
+    int cx, cy, cz;
+    unpack_cell(packed_cell(tg.w), cx, cy, cz);
+    const int c0x = __shfl_sync(0xffffffffu, cx, 0), c0y = __shfl_sync(0xffffffffu, cy, 0),
+              c0z = __shfl_sync(0xffffffffu, cz, 0);
+    const float Hx = (float)(cx - c0x), Hy = (float)(cy - c0y), Hz = (float)(cz - c0z);
+    float lo[3], hi[3];
+    warp_box(Hx + tg.x, lo[0], hi[0]);
+    warp_box(Hy + tg.y, lo[1], hi[1]);
+    warp_box(Hz + tg.z, lo[2], hi[2]);
+    // lengths in cells of x
+    const float ry = p.near_ryf, rz = p.near_rzf, eps2 = p.near_e2f, reach2 = eps2 * 1.001f;
+    const float2 k1 = make_float2(p.near_k1f, p.near_k1f), m1 = make_float2(-1.f, -1.f);
+    const float2 ry2 = make_float2(ry, ry), rz2 = make_float2(rz, rz);
+    const float2 Hx2 = make_float2(Hx, Hx), Hy2 = make_float2(Hy, Hy), Hz2 = make_float2(Hz, Hz);
+    const float2 fx2 = make_float2(tg.x, tg.x), fy2 = make_float2(tg.y, tg.y), fz2 = make_float2(tg.z, tg.z);
+    float2 c[NEAR_DEG32 + 1];  // coefficients of -a E
+#pragma unroll
+    for (int k = 0; k <= NEAR_DEG32; ++k) c[k] = make_float2(p.near_c32[k], p.near_c32[k]);
+    const float4 *src = (const float4 *)p.src_grid;
+    const float *qb = (const float *)p.qbuf;
+    float2 acc = make_float2(0.f, 0.f);
+    for (int r = it.rbegin; r < it.rend; ++r) {
+        const int2 rg = p.near_ranges[r];
+        for (int s0 = rg.x; s0 < rg.y; s0 += 32) {
+            const int s = min(s0 + lane, rg.y - 1);
+            const float4 g = src[s];
+            const float q = qb[s];
+            int sx, sy, sz;
+            unpack_cell(packed_cell(g.w), sx, sy, sz);
+            const float Sx = (float)(sx - c0x), Sy = (float)(sy - c0y), Sz = (float)(sz - c0z);
+            const bool keep = s0 + lane < rg.y && in_reach(lo, hi, Sx + g.x, Sy + g.y, Sz + g.z, ry, rz, reach2);
+            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+            if (kept == 0) continue;
+            const int cnt = __popc(kept);
+            const int at = __popc(kept & ((1u << lane) - 1u));
+            // a multiple of four: up to three lanes add their source once more, without charge
+            const int npad = -cnt & 3;
+            if (keep || lane < npad) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (e == 0 ? !keep : lane >= npad) continue;
+                    const int k = e == 0 ? at : cnt + lane;
+                    float *d = (float *)st[warp][k >> 1] + (k & 1);
+                    d[0] = -Sx;
+                    d[2] = -Sy;
+                    d[4] = -Sz;
+                    d[6] = -g.x;
+                    d[8] = -g.y;
+                    d[10] = -g.z;
+                    d[12] = e == 0 ? q : 0.f;
+                }
+            }
+            __syncwarp();
+            for (int j = half; 2 * j < cnt; j += 2) {
+                const float4 *v = (const float4 *)st[warp][j];
+                const float4 v0 = v[0], v1 = v[1], v2 = v[2];
+                const float2 qq = st[warp][j][6];
+                float2 dx = __fadd2_rn(__fadd2_rn(Hx2, make_float2(v0.x, v0.y)), __fadd2_rn(fx2, make_float2(v1.z, v1.w)));
+                float2 dy = __fadd2_rn(__fadd2_rn(Hy2, make_float2(v0.z, v0.w)), __fadd2_rn(fy2, make_float2(v2.x, v2.y)));
+                float2 dz = __fadd2_rn(__fadd2_rn(Hz2, make_float2(v1.x, v1.y)), __fadd2_rn(fz2, make_float2(v2.z, v2.w)));
+                dy = __fmul2_rn(dy, ry2);
+                dz = __fmul2_rn(dz, rz2);
+                const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                const float2 u = __ffma2_rn(r2, k1, m1);
+                float2 e = c[NEAR_DEG32];
+#pragma unroll
+                for (int k = NEAR_DEG32 - 1; k >= 0; --k) e = __ffma2_rn(e, u, c[k]);
+                float2 w = __fadd2_rn(make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y)), e);
+                w.x = r2.x < eps2 ? w.x : 0.f;
+                w.y = r2.y < eps2 ? w.y : 0.f;
+                acc = __ffma2_rn(qq, w, acc);
+            }
+            __syncwarp();
+        }
+    }
+    float sum = acc.x + acc.y;
+    sum += __shfl_xor_sync(0xffffffffu, sum, NEAR_TARGETS);
+    if (lane < it.tcount) {
+        const float v = sum * p.near_outf;
+        if (p.deterministic)
+            ((float *)p.phi_near)[(int64_t)item * 32 + lane] = v;
+        else
+            atomicAdd((float *)p.phi_part + it.tbegin + lane, v);
+    }
+}
+
+// 1 / sqrt(x) in FP64: the FP32 value and one third-order step of Householder's
+// iteration, y (1 + e/2 + 3 e^2 / 8) with e = 1 - x y^2 (e < 2^-21, so the
+// remainder is below 2^-63).  The FP32 seed needs x in FP32's range; here x is
+// a squared distance in grid cells.
+__device__ __forceinline__ double rsqrt_refined(double x) {
+    const double y = (double)rsqrt_approx((float)x);
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// FP64: this GPU's FP64 pipe (2 lanes per SM) bounds it, so everything that is
+// not the pair's own arithmetic is kept off it: about 27 FP64 operations per
+// pair (3 subtractions, 5 for r^2, 5 for the reciprocal square root, 3 for the
+// interval and its local coordinate, 9 of the degree-9 polynomial, 2 for the
+// sum) where rsqrt, erfc and the conversions of the cell differences took over
+// 100.  The interval is read off the low word of x / width + 1.5 2^52.
+// Level-4 sphere at 128^3 (63M pairs listed): 129 -> 3.6 ms, level-3 20.4 ->
+// 0.35 ms, both with the work list's full 16-target blocks.
+__global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial64(DevPlan p) {
+    __shared__ __align__(16) double4 st[NEAR_WARPS][32];  // position, charge
+    __shared__ double tab[(NEAR_DEG64 + 1) * NEAR_INT64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int item = blockIdx.x * NEAR_WARPS + warp;
+    const int ni = p.near_ni64;
+    for (int i = threadIdx.x; i < (NEAR_DEG64 + 1) * ni; i += blockDim.x) tab[i] = p.near_tab64[i];
+    pdl_wait();
+    pdl_trigger();
+    __syncthreads();
+    if (item >= p.n_near) return;
+    const NearItem it = p.near_items[item];
+    const int half = lane / NEAR_TARGETS;
+    const double4 tg = ((const double4 *)p.tgt_grid)[it.tbegin + min(lane % NEAR_TARGETS, it.tcount - 1)];
+    int cx, cy, cz;
+    unpack_cell(packed_cell(tg.w), cx, cy, cz);
+    const int c0x = __shfl_sync(0xffffffffu, cx, 0), c0y = __shfl_sync(0xffffffffu, cy, 0),
+              c0z = __shfl_sync(0xffffffffu, cz, 0);
+    const double tx = (cx - c0x) + tg.x, ty = (cy - c0y) + tg.y, tz = (cz - c0z) + tg.z;
+    float lo[3], hi[3];
+    warp_box((float)tx, lo[0], hi[0]);
+    warp_box((float)ty, lo[1], hi[1]);
+    warp_box((float)tz, lo[2], hi[2]);
+    const double ry = p.near_ry, rz = p.near_rz, iw = p.near_iw;
+    const float reach2 = p.near_e2f * 1.001f, ryf = p.near_ryf, rzf = p.near_rzf;
+    constexpr double MAGIC = 6755399441055744.0;  // 1.5 2^52
+    const double4 *src = (const double4 *)p.src_grid;
+    const double *qb = (const double *)p.qbuf;
+    double acc = 0.0;
+    for (int r = it.rbegin; r < it.rend; ++r) {
+        const int2 rg = p.near_ranges[r];
+        for (int s0 = rg.x; s0 < rg.y; s0 += 32) {
+            const int s = min(s0 + lane, rg.y - 1);
+            const double4 g = src[s];
+            const double q = qb[s];
+            int sx, sy, sz;
+            unpack_cell(packed_cell(g.w), sx, sy, sz);
+            const double x = (sx - c0x) + g.x, y = (sy - c0y) + g.y, z = (sz - c0z) + g.z;
+            const bool keep = s0 + lane < rg.y && in_reach(lo, hi, (float)x, (float)y, (float)z, ryf, rzf, reach2);
+            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+            if (kept == 0) continue;
+            if (keep) st[warp][__popc(kept & ((1u << lane) - 1u))] = make_double4(x, y, z, q);
+            __syncwarp();
+            const int cnt = __popc(kept);
+            for (int j = half; j < cnt; j += 2) {
+                const double4 v = st[warp][j];
+                const double dx = tx - v.x, dy = (ty - v.y) * ry, dz = (tz - v.z) * rz;
+                const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+                // interval i holds x / width in [i - 1/2, i + 1/2): a shift of 1/2 makes it [i, i + 1)
+                const double t = fma(r2, iw, -0.5);
+                const double tm = t + MAGIC;
+                const int i = __double2loint(tm);
+                const double u = t - (tm - MAGIC);  // in [-1/2, 1/2]
+                const bool in = (unsigned)i < (unsigned)ni;
+                const double *ct = tab + (in ? i : 0);
+                double e = ct[NEAR_DEG64 * ni];
+#pragma unroll
+                for (int k = NEAR_DEG64 - 1; k >= 0; --k) e = fma(e, u, ct[k * ni]);
+                const double w = rsqrt_refined(r2) + e;
+                acc = fma(in ? v.w : 0.0, w, acc);
+            }
+            __syncwarp();
+        }
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, NEAR_TARGETS);
+    if (lane < it.tcount) {
+        const double v = acc * p.near_out;
+        if (p.deterministic)
+            ((double *)p.phi_near)[(int64_t)item * 32 + lane] = v;
+        else
+            atomicAdd((double *)p.phi_part + it.tbegin + lane, v);
     }
 }
 
@@ -146,7 +384,9 @@ __global__ void k_near_reduce(DevPlan p, const int *__restrict__ blk_first, int 
 template <typename T> static cudaError_t near_t(const DevPlan &p, cudaStream_t s) {
     if (p.n_near == 0) return cudaSuccess;
     const int nb = (p.n_near + NEAR_WARPS - 1) / NEAR_WARPS;
-    if (p.kernel_mode == 2)
+    if (p.near_fit)
+        { const cudaError_t le = launch_k(sizeof(T) == 4 ? k_near_radial32 : k_near_radial64, nb, NEAR_WARPS * 32, 0, s, p); if (le != cudaSuccess) return le; }
+    else if (p.kernel_mode == 2)
         { const cudaError_t le = launch_k(k_near<T, 2>, nb, NEAR_WARPS * 32, 0, s, p); if (le != cudaSuccess) return le; }
     else if (p.kernel_mode == 3)
         { const cudaError_t le = launch_k(k_near<T, 3>, nb, NEAR_WARPS * 32, 0, s, p); if (le != cudaSuccess) return le; }

@@ -35,13 +35,32 @@ struct StatePtrs {
 // four items per SM; the gather kernel stages one item per block).
 constexpr int GATHER_CHUNK = 64;
 
-// Work item of the near-field kernel: up to 32 sorted targets
+// Work item of the near-field kernel: up to NEAR_TARGETS sorted targets
 // [tbegin, tbegin + tcount) and a slice [rbegin, rend) of the range list,
 // each range a contiguous run of sorted sources.
 struct NearItem {
     int tbegin, tcount;
     int rbegin, rend;
 };
+// Half a warp: its other half takes every second source.  Against blocks of 32
+// targets cut at tile borders, blocks of 16 cut where they stay compact cover
+// the level-5 sphere's near field at 128^3 with 118M lane pairs instead of
+// 161M (73M pairs lie inside eps), and sparse FP64 meshes, whose tiles hold
+// two or three targets, with full lanes instead of a tenth.
+constexpr int NEAR_TARGETS = 16;
+
+// Fits of a E(a^2 r^2) = erf(a r) / r on [0, eps^2] for the RADIAL near field
+// computed per pair.  FP32: one polynomial of degree NEAR_DEG32 in
+// u = 2 r^2 / eps^2 - 1, kept where a eps <= NEAR_Z32 (largest error 4e-9 of
+// 1/r, below FP32 rounding; a eps is 3.0 at tolerance 1e-5).  FP64: intervals
+// of width NEAR_W64 or less in x = (a r)^2, at most NEAR_INT64 of them, a
+// polynomial of degree NEAR_DEG64 in the local coordinate in [-1/2, 1/2] on
+// each (largest error 2e-15 of 1/r; a eps is 4.6 at tolerance 1e-10).
+constexpr int NEAR_DEG32 = 13;
+constexpr double NEAR_Z32 = 3.1;
+constexpr int NEAR_DEG64 = 9;
+constexpr int NEAR_INT64 = 64;
+constexpr double NEAR_W64 = 0.65;
 
 // Error codes written to the plan's sticky status word (the first one stays).
 enum { DEV_ERR_NONE = 0, DEV_ERR_BAD_ITEM = 1, DEV_ERR_BAD_INDEX = 2, DEV_ERR_NONFINITE = 3 };
@@ -118,7 +137,15 @@ struct DevPlan {
     const TileItem *gather_items; int n_gather;
     const NearItem *near_items;   int n_near;
     const int2 *near_ranges;
-    int near_chunk;               // deterministic mode: item slot per target block
+    // RADIAL near field computed per pair: 1 where the fits of a E apply;
+    // coefficients of -a E per cell of x (FP32), [k][interval] table (FP64)
+    int near_fit;
+    float near_c32[NEAR_DEG32 + 1];
+    const double *near_tab64; int near_ni64;
+    // lengths in cells of x: cell ratios y/x and z/x, intervals per unit of r^2
+    // (FP64), eps^2 and 2 / eps^2 (FP32); 1 / (4 pi h_x)
+    double near_ry, near_rz, near_iw, near_out;
+    float near_ryf, near_rzf, near_e2f, near_k1f, near_outf;
 
     // separable kernel: K_n(d) = A prod_q f_q(d_q / L_q), f_q(t) = sum_l hq[l] cos(2 pi l t)
     const void *sep_h[3]; int sep_nh[3];  // hq[0..nh-1], term l uses weight (l==0 ? 1 : 2) * hq[l]

@@ -26,7 +26,6 @@
 #include <cstring>
 #include <numeric>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "slp_plan_internal.h"
@@ -583,16 +582,17 @@ void grid_coords(const slp_plan_s &p, const double *x, double *g, int &cx, int &
     g[3] = (double)packed;
 }
 
-// sort points by (tile, Morton order inside the tile); fills perm and grid[.][4]
+// sort points by (tile, Morton order inside the tile), the tiles in Morton
+// order too, so that neighbours in the sort are neighbours in space across
+// tile borders; fills perm and grid[.][4]
 void sort_points(const slp_plan_s &p, const double *pts, int64_t n, int ts, std::vector<int32_t> &perm,
                  std::vector<double> &grid, std::vector<uint64_t> &keys_sorted) {
     std::vector<double> g(4 * n);
     std::vector<uint64_t> key(n);
-    const int ntx = (p.L[0] + ts - 1) / ts, nty = (p.L[1] + ts - 1) / ts;
     for (int64_t i = 0; i < n; ++i) {
         int cx, cy, cz;
         grid_coords(p, pts + 3 * i, &g[4 * i], cx, cy, cz);
-        const uint64_t tile = ((uint64_t)(cz / ts) * nty + (cy / ts)) * ntx + (cx / ts);
+        const uint64_t tile = morton3(cx / ts, cy / ts, cz / ts);
         const uint32_t mort = morton3(cx % ts, cy % ts, cz % ts);
         key[i] = (tile << 32) | mort;
     }
@@ -684,112 +684,176 @@ inline void phys(const slp_plan_s &p, const double *g, double *x) {
     for (int d = 0; d < 3; ++d) x[d] = ((c[d] + g[d]) - 0.5 * p.L[d]) * (p.P[d] / p.L[d]);
 }
 
-// near-field work list: target blocks of <= 32 sorted targets in one tile,
-// candidate source bins (aligned 2x2x2 cell blocks, contiguous in the sort)
-// whose bounding box lies within eps of the block's bounding box.
-void near_items(slp_plan_s &p, const std::vector<uint64_t> &skeys, const std::vector<uint64_t> &tkeys) {
-    p.near_items.clear();
-    p.near_ranges.clear();
-    p.near_blk_first.clear();
-    p.near_pairs = 0;
-    const int64_t NCH = 2048;  // sources per item
-    // target blocks
-    std::vector<std::pair<int, int>> blocks;
-    for (int64_t i = 0; i < p.N;) {
-        int64_t j = i;
-        const uint64_t tile = tkeys[i] >> 32;
-        while (j < p.N && (tkeys[j] >> 32) == tile && j - i < 32) ++j;
-        blocks.push_back({(int)i, (int)(j - i)});
-        i = j;
-    }
-    const bool all_pairs = p.kernel_mode == SLP_KERNEL_SEPARABLE || !(p.eps < p.diam);
-    // source bins: key = (tile, morton >> 3)
+// Runs of sorted points in aligned 2x2x2 cell blocks (contiguous in the sort),
+// with their bounding boxes, kept by row (bz, by) of blocks and by bx in a row
+// so that a box query walks rows.
+struct CellBins {
     struct Bin {
-        int b, e;
+        int b, e, bx;
         double lo[3], hi[3];
     };
     std::vector<Bin> bins;
-    std::unordered_map<uint64_t, int> bin_of;  // cell-block coordinate -> bin
-    if (!all_pairs) {
-        for (int64_t i = 0; i < p.Q;) {
+    std::vector<int> row;  // [nbz * nby + 1]
+    int nby = 0, nbz = 0;
+
+    // pos(k, x): physical position of sorted point k
+    template <typename Pos>
+    void build(const slp_plan_s &p, const std::vector<uint64_t> &keys, const std::vector<double> &grid, int64_t n,
+               Pos pos) {
+        nby = (p.L[1] + 1) / 2;
+        nbz = (p.L[2] + 1) / 2;
+        std::vector<Bin> found;
+        std::vector<int> at;
+        row.assign((size_t)nby * nbz + 1, 0);
+        for (int64_t i = 0; i < n;) {
             int64_t j = i;
-            const uint64_t bk = skeys[i] >> 3;
-            while (j < p.Q && (skeys[j] >> 3) == bk) ++j;
+            while (j < n && (keys[j] >> 3) == (keys[i] >> 3)) ++j;
+            const uint32_t packed = (uint32_t)grid[4 * i + 3];
             Bin bn;
             bn.b = (int)i;
             bn.e = (int)j;
+            bn.bx = (packed & 1023) / 2;
             for (int d = 0; d < 3; ++d) {
                 bn.lo[d] = 1e300;
                 bn.hi[d] = -1e300;
             }
             for (int64_t k = i; k < j; ++k) {
                 double x[3];
-                phys(p, &p.src_grid[4 * k], x);
+                pos(k, x);
                 for (int d = 0; d < 3; ++d) {
                     bn.lo[d] = std::min(bn.lo[d], x[d]);
                     bn.hi[d] = std::max(bn.hi[d], x[d]);
                 }
             }
-            const uint32_t packed = (uint32_t)p.src_grid[4 * i + 3];
-            const uint64_t bx = (packed & 1023) / 2, by = ((packed >> 10) & 1023) / 2, bz = ((packed >> 20) & 1023) / 2;
-            bin_of[(bz << 40) | (by << 20) | bx] = (int)bins.size();
-            bins.push_back(bn);
+            found.push_back(bn);
+            at.push_back((int)((packed >> 20) & 1023) / 2 * nby + (int)((packed >> 10) & 1023) / 2);
+            ++row[at.back() + 1];
             i = j;
         }
+        for (size_t r = 1; r < row.size(); ++r) row[r] += row[r - 1];
+        bins.resize(found.size());
+        std::vector<int> next(row.begin(), row.end() - 1);
+        for (size_t k = 0; k < found.size(); ++k) bins[next[at[k]]++] = found[k];
+        for (size_t r = 0; r + 1 < row.size(); ++r)
+            std::sort(bins.begin() + row[r], bins.begin() + row[r + 1],
+                      [](const Bin &x, const Bin &y) { return x.bx < y.bx; });
     }
-    const double eps = p.eps;
-    std::vector<int> found;
-    for (const auto &blk : blocks) {
-        std::vector<int2> rng;
-        if (all_pairs) {
-            rng.push_back(make_int2(0, (int)p.Q));
-        } else {
-            double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-            for (int t = blk.first; t < blk.first + blk.second; ++t) {
-                double x[3];
-                phys(p, &p.tgt_grid[4 * t], x);
-                for (int d = 0; d < 3; ++d) {
-                    lo[d] = std::min(lo[d], x[d]);
-                    hi[d] = std::max(hi[d], x[d]);
+
+    // Append the runs of sorted points in bins within rad of the box [lo, hi], ascending, neighbours joined.
+    void within(const slp_plan_s &p, const double *lo, const double *hi, double rad, double rad2,
+                std::vector<int2> &ranges) const {
+        const size_t first = ranges.size();
+        int b0[3], b1[3];
+        for (int d = 0; d < 3; ++d) {
+            const double h = p.P[d] / p.L[d];
+            const double u0 = (lo[d] - rad) / h + 0.5 * p.L[d], u1 = (hi[d] + rad) / h + 0.5 * p.L[d];
+            b0[d] = std::max(0, (int)std::floor(u0) - 1) / 2;
+            b1[d] = std::min(p.L[d] - 1, (int)std::floor(u1) + 1) / 2;
+        }
+        for (int bz = b0[2]; bz <= b1[2]; ++bz)
+            for (int by = b0[1]; by <= b1[1]; ++by) {
+                const Bin *e = bins.data() + row[(size_t)bz * nby + by + 1];
+                const Bin *k = std::lower_bound(bins.data() + row[(size_t)bz * nby + by], e, b0[0],
+                                                [](const Bin &x, int v) { return x.bx < v; });
+                for (; k < e && k->bx <= b1[0]; ++k) {
+                    double d2 = 0;
+                    for (int d = 0; d < 3; ++d) {
+                        const double g = std::max(0.0, std::max(k->lo[d] - hi[d], lo[d] - k->hi[d]));
+                        d2 += g * g;
+                    }
+                    if (d2 <= rad2) ranges.push_back(make_int2(k->b, k->e));
                 }
             }
-            int b0[3], b1[3];
+        std::sort(ranges.begin() + first, ranges.end(), [](const int2 &x, const int2 &y) { return x.x < y.x; });
+        size_t w = first;
+        for (size_t k = first; k < ranges.size(); ++k) {
+            if (w > first && ranges[w - 1].y == ranges[k].x)
+                ranges[w - 1].y = ranges[k].y;
+            else
+                ranges[w++] = ranges[k];
+        }
+        ranges.resize(w);
+    }
+};
+
+// near-field work list: blocks of at most NEAR_TARGETS consecutive sorted
+// targets, candidate source bins whose bounding box lies within eps of the
+// block's bounding box.
+void near_items(slp_plan_s &p, const std::vector<uint64_t> &skeys) {
+    p.near_items.clear();
+    p.near_ranges.clear();
+    p.near_blk_first.clear();
+    p.near_pairs = 0;
+    const bool all_pairs = p.kernel_mode == SLP_KERNEL_SEPARABLE || !(p.eps < p.diam);
+    const double eps = p.eps;
+    std::vector<double> tx(3 * (size_t)p.N);
+    for (int64_t i = 0; i < p.N; ++i) phys(p, &p.tgt_grid[4 * i], &tx[3 * i]);
+    // Target blocks: the cheapest cut of the sorted targets, a block costing
+    // (1 + diagonal / (2 eps))^2, about the surface within eps of it.  A block
+    // keeps its lanes whether full or not, so the cut trades short blocks
+    // against wide ones (a jump of the Morton order inside a block).
+    std::vector<double> best(p.N + 1, 0.0);
+    std::vector<int> from(p.N + 1, 0);
+    for (int64_t j = 1; j <= p.N; ++j) {
+        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+        best[j] = 1e300;
+        for (int64_t i = j - 1; i >= std::max<int64_t>(0, j - slp::NEAR_TARGETS); --i) {
+            double d2 = 0.0;
             for (int d = 0; d < 3; ++d) {
-                const double h = p.P[d] / p.L[d];
-                const double u0 = (lo[d] - eps) / h + 0.5 * p.L[d], u1 = (hi[d] + eps) / h + 0.5 * p.L[d];
-                b0[d] = std::max(0, (int)std::floor(u0) - 1) / 2;
-                b1[d] = std::min(p.L[d] - 1, (int)std::floor(u1) + 1) / 2;
+                lo[d] = std::min(lo[d], tx[3 * i + d]);
+                hi[d] = std::max(hi[d], tx[3 * i + d]);
+                d2 += (hi[d] - lo[d]) * (hi[d] - lo[d]);
             }
-            found.clear();
-            for (int bz = b0[2]; bz <= b1[2]; ++bz)
-                for (int by = b0[1]; by <= b1[1]; ++by)
-                    for (int bx = b0[0]; bx <= b1[0]; ++bx) {
-                        auto itb = bin_of.find(((uint64_t)bz << 40) | ((uint64_t)by << 20) | (uint64_t)bx);
-                        if (itb == bin_of.end()) continue;
-                        const Bin &bn = bins[itb->second];
-                        double d2 = 0;
-                        for (int d = 0; d < 3; ++d) {
-                            const double g = std::max(0.0, std::max(bn.lo[d] - hi[d], lo[d] - bn.hi[d]));
-                            d2 += g * g;
-                        }
-                        if (d2 <= eps * eps * (1.0 + 1e-9)) found.push_back(itb->second);
-                    }
-            std::sort(found.begin(), found.end(), [&](int a, int b) { return bins[a].b < bins[b].b; });
-            for (int f : found) {
-                if (!rng.empty() && rng.back().y == bins[f].b)
-                    rng.back().y = bins[f].e;
-                else
-                    rng.push_back(make_int2(bins[f].b, bins[f].e));
+            const double r = all_pairs ? 1.0 : 1.0 + 0.5 * std::sqrt(d2) / eps;
+            if (best[i] + r * r < best[j]) {
+                best[j] = best[i] + r * r;
+                from[j] = (int)i;
             }
         }
-        // chunk into items of <= NCH sources
+    }
+    std::vector<std::pair<int, int>> blocks;
+    for (int64_t j = p.N; j > 0; j = from[j]) blocks.push_back({from[j], (int)(j - from[j])});
+    std::reverse(blocks.begin(), blocks.end());
+    CellBins bins;
+    if (!all_pairs)
+        bins.build(p, skeys, p.src_grid, p.Q, [&](int64_t k, double *x) { phys(p, &p.src_grid[4 * k], x); });
+    std::vector<int2> ranges;
+    std::vector<size_t> first(blocks.size() + 1, 0);
+    int64_t listed = 0;  // (block, source) entries
+    for (size_t ib = 0; ib < blocks.size(); ++ib) {
+        const auto &blk = blocks[ib];
+        if (all_pairs) {
+            ranges.push_back(make_int2(0, (int)p.Q));
+        } else {
+            double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+            for (int t = blk.first; t < blk.first + blk.second; ++t)
+                for (int d = 0; d < 3; ++d) {
+                    lo[d] = std::min(lo[d], tx[3 * (size_t)t + d]);
+                    hi[d] = std::max(hi[d], tx[3 * (size_t)t + d]);
+                }
+            bins.within(p, lo, hi, eps, eps * eps * (1.0 + 1e-9), ranges);
+        }
+        first[ib + 1] = ranges.size();
+        for (size_t k = first[ib]; k < first[ib + 1]; ++k) listed += ranges[k].y - ranges[k].x;
+    }
+    // Sources per item: a warp works an item's sources off one after another,
+    // so a mesh with few target blocks needs short items to fill the GPU, and a
+    // large one enough items that the last round of warps is full.  Aim at 128
+    // items (warps) for each of 152 SMs (32 to 40 are resident), between 64
+    // sources (two warp loads) and 2048.  Near field per pair: level-5 sphere at
+    // 128^3 225 us at 48 items per SM, 199 us at 128; level-3 sphere 172 us in
+    // items of 2048, 14 us in items of 64.
+    const int64_t NCH = std::min<int64_t>(2048, std::max<int64_t>(64, round_up(listed / (152 * 128), 32)));
+    for (size_t ib = 0; ib < blocks.size(); ++ib) {
+        const auto &blk = blocks[ib];
         p.near_blk_first.push_back((int)p.near_items.size());
         int64_t acc = 0;
         slp::NearItem it;
         it.tbegin = blk.first;
         it.tcount = blk.second;
         it.rbegin = (int)p.near_ranges.size();
-        for (int2 r : rng) {
+        for (size_t k = first[ib]; k < first[ib + 1]; ++k) {
+            const int2 r = ranges[k];
             int b = r.x;
             while (b < r.y) {
                 const int take = (int)std::min<int64_t>(r.y - b, NCH - acc);
@@ -869,6 +933,63 @@ void build_dtab(slp_plan_s &p) {
                 const double w = W[0][kx] * W[1][ky] * W[2][kz];
                 p.Dtab[((size_t)kz * hy + ky) * Kx + kx] = cl / (w * w);
             }
+}
+
+// ---------------------------------------------------------------- near-field fits
+// Coefficients in powers of u, -1 <= u <= 1, of the degree-`deg` polynomial
+// nearest to f (its Chebyshev series, from 4 (deg + 1) nodes, truncated).
+template <typename F> std::vector<double> fit_powers(F f, int deg) {
+    const int K = 4 * (deg + 1);
+    std::vector<double> fv(K), cheb(deg + 1, 0.0);
+    for (int i = 0; i < K; ++i) fv[i] = f(std::cos(PI * (i + 0.5) / K));
+    for (int k = 0; k <= deg; ++k) {
+        for (int i = 0; i < K; ++i) cheb[k] += fv[i] * std::cos(PI * k * (i + 0.5) / K);
+        cheb[k] *= (k == 0 ? 1.0 : 2.0) / K;
+    }
+    std::vector<double> out(deg + 1, 0.0), t0(deg + 1, 0.0), t1(deg + 1, 0.0);
+    t0[0] = 1.0;  // T_k, T_{k+1} in powers of u
+    if (deg > 0) t1[1] = 1.0;
+    for (int k = 0; k <= deg; ++k) {
+        for (int j = 0; j <= deg; ++j) out[j] += cheb[k] * t0[j];
+        std::vector<double> t2(deg + 1, 0.0);
+        for (int j = 0; j < deg; ++j) t2[j + 1] = 2.0 * t1[j];
+        for (int j = 0; j <= deg; ++j) t2[j] -= t0[j];
+        t0.swap(t1);
+        t1.swap(t2);
+    }
+    return out;
+}
+
+// erf(sqrt x) / sqrt x
+double erf_ratio(double x) {
+    const double z = std::sqrt(std::max(x, 0.0));
+    return z < 1e-8 ? 2.0 / std::sqrt(PI) : std::erf(z) / z;
+}
+
+// The fits of -a E(a^2 r^2) (slp_internal.h), lengths in cells of x: FP32
+// coefficients into c32, the FP64 table [k][interval] into tab.  False where
+// the RADIAL kernel's a eps lies outside their range.
+bool near_fits(const slp_plan_s &p, float *c32, std::vector<double> &tab, int &ni) {
+    ni = 0;
+    if (p.kernel_mode != SLP_KERNEL_RADIAL || !(p.sigma_g > 0) || !std::isfinite(p.eps)) return false;
+    const double h = p.P[0] / p.L[0], a = h / (p.sigma_g * std::sqrt(2.0)), z = a * (p.eps / h), x1 = z * z;
+    if (p.prec == 32) {
+        if (z > slp::NEAR_Z32) return false;
+        const std::vector<double> c = fit_powers([&](double u) { return -a * erf_ratio(0.5 * (u + 1.0) * x1); }, slp::NEAR_DEG32);
+        for (int k = 0; k <= slp::NEAR_DEG32; ++k) c32[k] = (float)c[k];
+        return true;
+    }
+    const int n = std::max(1, (int)std::ceil(x1 / slp::NEAR_W64));
+    if (n > slp::NEAR_INT64) return false;
+    ni = n;
+    const double w = x1 / n;
+    tab.assign((size_t)(slp::NEAR_DEG64 + 1) * n, 0.0);
+    for (int i = 0; i < n; ++i) {
+        const std::vector<double> c = fit_powers([&](double u) { return -a * erf_ratio((i + 0.5 * (u + 1.0)) * w); }, slp::NEAR_DEG64);
+        double s = 1.0;  // the kernel's local coordinate is u / 2
+        for (int k = 0; k <= slp::NEAR_DEG64; ++k, s *= 2.0) tab[(size_t)k * n + i] = c[k] * s;
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------- active rows
@@ -1238,6 +1359,25 @@ template <typename T> slp_status upload_all(slp_plan_s &p) {
     d.near_ranges = (const int2 *)ptr;
     TRY(upload(p, &ptr, p.near_blk_first.data(), p.near_blk_first.size()));
     p.d_blk_first = (int *)ptr;
+    {
+        std::vector<double> tab;
+        d.near_fit = near_fits(p, d.near_c32, tab, d.near_ni64) ? 1 : 0;
+        d.near_tab64 = nullptr;
+        if (!tab.empty()) {
+            TRY(upload(p, &ptr, tab.data(), tab.size()));
+            d.near_tab64 = (const double *)ptr;
+        }
+        const double e2 = p.eps * p.eps / (d.h[0] * d.h[0]);
+        d.near_ry = d.h[1] / d.h[0];
+        d.near_rz = d.h[2] / d.h[0];
+        d.near_iw = d.near_ni64 / e2;
+        d.near_out = 1.0 / (4.0 * PI * d.h[0]);
+        d.near_ryf = (float)d.near_ry;
+        d.near_rzf = (float)d.near_rz;
+        d.near_e2f = (float)e2;
+        d.near_k1f = (float)(2.0 / e2);
+        d.near_outf = (float)d.near_out;
+    }
     if (p.opts.deterministic) TRY(dalloc(p, &d.phi_near, sizeof(T) * 32 * std::max<size_t>(1, p.near_items.size())));
     d.integration = p.opts.integration ? 1 : 0;
     if (d.integration) {
@@ -1356,82 +1496,6 @@ struct NearCandidates {
     std::vector<int2> ranges;
 };
 
-// Bins of the sorted targets (vertices): runs of one aligned 2x2x2-cell block,
-// contiguous in the sort, with their bounding boxes.
-struct TargetBins {
-    struct Bin {
-        int b, e;
-        double lo[3], hi[3];
-    };
-    std::vector<Bin> bins;
-    std::unordered_map<uint64_t, int> bin_of;
-};
-
-void target_bins(const slp_plan_s &p, const std::vector<uint64_t> &tkeys, const std::vector<double4> &tgt,
-                 TargetBins &tb) {
-    const int64_t N = p.N;
-    tb.bins.clear();
-    tb.bin_of.clear();
-    for (int64_t i = 0; i < N;) {
-        int64_t j = i;
-        const uint64_t bk = tkeys[i] >> 3;
-        while (j < N && (tkeys[j] >> 3) == bk) ++j;
-        TargetBins::Bin bn;
-        bn.b = (int)i;
-        bn.e = (int)j;
-        for (int d = 0; d < 3; ++d) {
-            bn.lo[d] = 1e300;
-            bn.hi[d] = -1e300;
-        }
-        for (int64_t k = i; k < j; ++k) {
-            const double x[3] = {tgt[k].x, tgt[k].y, tgt[k].z};
-            for (int d = 0; d < 3; ++d) {
-                bn.lo[d] = std::min(bn.lo[d], x[d]);
-                bn.hi[d] = std::max(bn.hi[d], x[d]);
-            }
-        }
-        const uint32_t packed = (uint32_t)p.tgt_grid[4 * i + 3];
-        const uint64_t bx = (packed & 1023) / 2, by = ((packed >> 10) & 1023) / 2, bz = ((packed >> 20) & 1023) / 2;
-        tb.bin_of[(bz << 40) | (by << 20) | bx] = (int)tb.bins.size();
-        tb.bins.push_back(bn);
-        i = j;
-    }
-}
-
-// Append to `ranges` the runs of sorted vertices in bins within rad of the box [lo, hi].
-void bins_within(const slp_plan_s &p, const TargetBins &tb, const double *lo, const double *hi, double rad,
-                 std::vector<int2> &ranges) {
-    const size_t first = ranges.size();
-    int b0[3], b1[3];
-    for (int d = 0; d < 3; ++d) {
-        const double h = p.P[d] / p.L[d];
-        const double u0 = (lo[d] - rad) / h + 0.5 * p.L[d], u1 = (hi[d] + rad) / h + 0.5 * p.L[d];
-        b0[d] = std::max(0, (int)std::floor(u0) - 1) / 2;
-        b1[d] = std::min(p.L[d] - 1, (int)std::floor(u1) + 1) / 2;
-    }
-    std::vector<int> found;
-    for (int bz = b0[2]; bz <= b1[2]; ++bz)
-        for (int by = b0[1]; by <= b1[1]; ++by)
-            for (int bx = b0[0]; bx <= b1[0]; ++bx) {
-                auto itb = tb.bin_of.find(((uint64_t)bz << 40) | ((uint64_t)by << 20) | (uint64_t)bx);
-                if (itb == tb.bin_of.end()) continue;
-                const TargetBins::Bin &bn = tb.bins[itb->second];
-                double d2 = 0;
-                for (int d = 0; d < 3; ++d) {
-                    const double g = std::max(0.0, std::max(bn.lo[d] - hi[d], lo[d] - bn.hi[d]));
-                    d2 += g * g;
-                }
-                if (d2 <= rad * rad) found.push_back(itb->second);
-            }
-    std::sort(found.begin(), found.end(), [&](int a2, int b2) { return tb.bins[a2].b < tb.bins[b2].b; });
-    for (int f : found) {
-        if (ranges.size() > first && ranges.back().y == tb.bins[f].b)
-            ranges.back().y = tb.bins[f].e;
-        else
-            ranges.push_back(make_int2(tb.bins[f].b, tb.bins[f].e));
-    }
-}
-
 void near_candidates(const slp_plan_s &p, const std::vector<uint64_t> &tkeys, double rad, bool all_pairs,
                      NearCandidates &c) {
     const int64_t N = p.N, M = p.M;
@@ -1461,8 +1525,9 @@ void near_candidates(const slp_plan_s &p, const std::vector<uint64_t> &tkeys, do
     blk_r0.assign(nblk + 1, 0);
     std::vector<int2> &ranges = c.ranges;
     ranges.clear();
-    TargetBins tb;
-    if (!all_pairs) target_bins(p, tkeys, tgt, tb);
+    auto pos = [&](int64_t k, double *x) { x[0] = tgt[k].x, x[1] = tgt[k].y, x[2] = tgt[k].z; };
+    CellBins bins;
+    if (!all_pairs) bins.build(p, tkeys, p.tgt_grid, p.N, pos);
     for (int b = 0; b < nblk; ++b) {
         const slp::NearItem &it = p.near_items[p.near_blk_first[b]];
         for (int t = it.tbegin; t < it.tbegin + it.tcount; ++t) tgt_block[t] = b;
@@ -1479,7 +1544,7 @@ void near_candidates(const slp_plan_s &p, const std::vector<uint64_t> &tkeys, do
                 hi[d] = std::max(hi[d], x[d]);
             }
         }
-        bins_within(p, tb, lo, hi, rad, ranges);
+        bins.within(p, lo, hi, rad, rad * rad, ranges);
     }
     blk_r0[nblk] = (int)ranges.size();
 }
@@ -1994,8 +2059,9 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         std::vector<double> tgrid;
         sort_points(p, p.V.data(), p.N, p.TSg, tperm, tgrid, tkeys);
         near_candidates(p, tkeys, rad, all_pairs, cand);  // vertex adjacency and bins of the plan's targets
-        TargetBins tb;
-        if (!all_pairs) target_bins(p, tkeys, cand.tgt, tb);
+        auto pos = [&](int64_t k, double *x) { x[0] = cand.tgt[k].x, x[1] = cand.tgt[k].y, x[2] = cand.tgt[k].z; };
+        CellBins bins;
+        if (!all_pairs) bins.build(p, tkeys, tgrid, p.N, pos);
         const int64_t nblk = (n + 31) / 32;
         cand.tgt_block.assign(n, 0);
         cand.blk_r0.assign(nblk + 1, 0);
@@ -2014,7 +2080,7 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
             if (all_pairs)
                 cand.ranges.push_back(make_int2(0, (int)p.N));
             else
-                bins_within(p, tb, lo, hi, rad, cand.ranges);
+                bins.within(p, lo, hi, rad, rad * rad, cand.ranges);
         }
         cand.blk_r0[nblk] = (int)cand.ranges.size();
     }
@@ -2613,7 +2679,7 @@ slp_status slp_plan(const slp_mesh *mesh, int quadrature, double tolerance, cons
     std::stable_sort(p->spread_items.begin(), p->spread_items.end(), by_size);
     std::stable_sort(p->gather_items.begin(), p->gather_items.end(), by_size);
     spread_groups(*p);
-    near_items(*p, skeys, tkeys);
+    near_items(*p, skeys);
     build_dtab(*p);
     active_region(*p);
     p->near_mode = SLP_NEAR_ON_THE_FLY;
