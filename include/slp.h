@@ -294,8 +294,9 @@ slp_status slp_probe_destroy(slp_probe_t probe);
  * triangle-integrated plan (opts.integration is set; Sec. 3) and a probe set
  * of the free nodes.
  * Computation (slp_potential_eval): b = B m (in the plan's precision);
- * phi_1 by iterative refinement on the device: Jacobi-preconditioned
- * conjugate gradients in FP32 cut the residual of the current correction
+ * phi_1 by iterative refinement on the device: preconditioned conjugate
+ * gradients in FP32 (Jacobi and, up to about 0.9M free nodes, one coarse
+ * unknown per block of rows) cut the residual of the current correction
  * equation by 1e-4, the correction joins the FP64 solution and the residual
  * b - S x is recomputed in FP64, until |b - S x| <= cg_tolerance |b|;
  * g_j = (mean of m over boundary triangle j) . n_j + phi_1(o) / h_j, o the
@@ -340,11 +341,13 @@ slp_status slp_potential_create(const double *nodes, int64_t n_nodes, const int3
 /* d_m: device [n_nodes][3] (plan precision), the nodal magnetisation;
  * d_phi: device [n_nodes], overwritten with phi; d_phi_1: NULL or device
  * [n_nodes], overwritten with phi_1.  Enqueued on `stream`: the load, the
- * solve (one graph whose loops over corrections and inner steps run on the
- * device until the solve stops), phi_2 and the sum.  The call then waits
+ * solve (one cooperative launch, or for larger systems one graph whose loops
+ * over corrections and inner steps run on the device, until the solve stops),
+ * phi_2 and the sum.  The call then waits
  * for the solve, not for phi_2, to return its status, so it cannot be
  * captured into a CUDA graph.  Errors: INVALID_ARG, CUDA, NONFINITE (the iteration met
- * NaN/Inf), TOLERANCE_INFEASIBLE (cg_max_iterations reached: phi is still
+ * NaN/Inf), TIMEOUT (a bounded wait between the solve's blocks gave up),
+ * TOLERANCE_INFEASIBLE (cg_max_iterations reached: phi is still
  * written, from the last iterate). */
 slp_status slp_potential_eval(slp_potential_t pot, const void *d_m, void *d_phi, void *d_phi_1, void *stream);
 slp_status slp_potential_query(slp_potential_t pot, slp_potential_info *info);

@@ -19,8 +19,10 @@
 //   gamma_{k+1} = r_{k+1} . u_{k+1},  delta_{k+1} = w_{k+1} . u_{k+1},
 //   beta_{k+1} = gamma_{k+1} / gamma_k,
 //   alpha_{k+1} = gamma_{k+1} / (delta_{k+1} - beta_{k+1} gamma_{k+1} / alpha_k),
-// which needs both dot products at one point of the step.  One launch does
-// a step: every vector update is per row, and u_{k+1} at the columns the
+// which needs both dot products at one point of the step.  Systems of up to
+// SOLVE_THREADS 12 rows a block (0.9M free nodes) are solved in one launch
+// (k_cg_solve, further down, with a better preconditioner); for larger ones a
+// launch does a step: every vector update is per row, and u_{k+1} at the columns the
 // product gathers is formed there from r_k, w_k and s_{k-1}, which a row
 // keeps together with its 1 / diagonal in one 16-byte record (the step
 // reads the records of one parity and writes those of the other).  A launch
@@ -155,6 +157,12 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_fem_load(FemDev d, const T *__restrict__ m) {
     typedef typename Vec4<T>::t T4;
     __shared__ double sh[NT / 32];
+    if (d.parts > 0) {  // no exchange has happened yet
+        const int64_t step = (int64_t)gridDim.x * NT, i0 = (int64_t)blockIdx.x * NT + threadIdx.x;
+        for (int64_t i = i0; i < d.nhalo; i += step) d.rec[0][i] = d.rec[1][i] = make_uint4(0, 0, 0, 0);
+        for (int64_t i = i0; i < (int64_t)d.parts * d.parts; i += step)
+            d.psum[0][i] = d.psum[1][i] = make_uint4(0, 0, 0, 0);
+    }
     const int gl = threadIdx.x % GROUP;
     const T4 *__restrict__ bv = (const T4 *)d.b_val;
     double bb = 0.0;
@@ -189,6 +197,7 @@ __global__ void __launch_bounds__(NT) k_fem_load(FemDev d, const T *__restrict__
         s.iter = 0;
         s.outer = 0;
         s.bad = 0;
+        s.stalled = 0;
         new_residual(d, s, t[0]);
         if (t[0] == 0.0 || d.max_iter <= 0) s.outer_done = s.done = 1;
     }
@@ -500,6 +509,371 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
     cudaGraphSetConditional(h, s.done ? 0u : 1u);
 }
 
+// ---------------------------------------------------------------- the solve in one launch
+// The same iteration with the rows spread over one resident block per SM, in
+// place of a launch per step.  A launch per step cost 7.1 us on the n = 32
+// ball (128k rows) and 4.6 us on n = 16 (16k rows): the chained launch, 15.4 MB
+// of matrix and 29 MB of gathered 16-byte records through L2 each time.  Here
+// a block's rows keep their state (and, up to 16 off-diagonal entries and two
+// rows a thread, their matrix rows) in registers, the gathered u of its own
+// rows and its halo in shared memory, and a step moves only the halo records
+// (about 600 of 16 bytes a block) and one record of partial sums per block.
+//
+// Exchange e: every block writes {r, w, s, e} of its rows into the halo lists
+// of the blocks that need them, and {gamma, delta, Z^T w, e} of its sums into
+// every block's list of sums, each list in two copies by the parity of e.  A
+// 16-byte access is one access (ld/st .b128), so a reader that finds the
+// number e has the record: no fence, no flag, one trip through L2 (560 cycles
+// within a die, 900 across).  Only its owner reads a list: lines polled by
+// several blocks while others write them cost more than the rest of the step,
+// and so do polls by threads that wait for nothing (one record per row, read in
+// place, and every thread polling: 5600 cycles an exchange; now 2500 to 4900).
+// A block writes exchange e + 2 only after it has read every block's sums of
+// e + 1, which that block wrote after it had read its records of e, so two
+// copies suffice.  All blocks add the sums in one order and hold the same
+// scalars.  The launch is cooperative (all blocks resident); every wait is
+// bounded, and a block that gives up sets `stalled` and leaves, after which the
+// others' waits run out as well.
+//
+// The system is scaled by its diagonal (S_ij / sqrt(S_ii S_jj), unit
+// diagonal).  The preconditioner adds to Jacobi's (the identity here) a coarse
+// space of one constant per part: u = r + Z A^-1 Z^T r, Z the parts' indicator
+// vectors times z_i = sqrt(S_ii), A = Z^T S Z inverted at set-up.  It removes
+// the error modes longer than a part, which plain Jacobi needs most of its
+// steps for (n = 32 ball: 289 steps with Jacobi alone, 145), and costs no exchange of its own: the
+// sums carry Z^T w of each part, from which every block updates the whole
+// coarse residual Z^T r as it does its rows' (s_c = w_c + beta s_c, r_c -=
+// alpha s_c), and a block forms the corrections of its own and its halo's
+// parts.  The inner iteration stops when r . u has fallen by 1e-8 (the
+// residual by 1e-4 in the preconditioner's norm).
+//
+// Measured, phi_1 (load, solve and all corrections): ball n = 16 672 -> 319 us,
+// n = 32 2155 -> 760 us (5.2 us a step: about 2.2 exchange, 0.9 product, the
+// rest the coarse correction, sums and barriers), n = 48 7600 -> 5600 us (its
+// matrix no longer fits the registers).
+constexpr int SNT = SOLVE_THREADS;
+constexpr int SNW = SNT / 32;
+constexpr int HB = 2;                  // halo records a thread reads at once
+constexpr int WAIT_LIMIT = 1 << 21;    // polls of one exchange (about a second)
+
+__device__ __forceinline__ uint4 ld_record(const uint4 *p) {
+    unsigned long long lo, hi;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+}
+__device__ __forceinline__ void st_record(uint4 *p, unsigned a, unsigned b, unsigned c, unsigned e) {
+    const unsigned long long lo = (unsigned long long)a | (unsigned long long)b << 32,
+                             hi = (unsigned long long)c | (unsigned long long)e << 32;
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+                 "l"(lo), "l"(hi)
+                 : "memory");
+}
+
+// Waits until the record at q carries number e; false when the bound is reached.
+__device__ __forceinline__ bool wait_record(const uint4 *q, unsigned e, uint4 &v) {
+    for (int n = 0; n < WAIT_LIMIT; ++n) {
+        v = ld_record(q);
+        if (v.w == e) return true;
+    }
+    return false;
+}
+
+// K sums over the block's first NW warps, the same in every thread: shuffles,
+// then the warps' sums in order (NW a multiple of four: vector reads, as 16
+// warps reading 48 values one by one took longer than the shuffles).  `stop`
+// is or-ed over the block on the way.
+template <int NW, int K, typename V> __device__ __forceinline__ bool solve_sum(V (&v)[K], V (*sh)[SNW], bool stop) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < NW) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < K; ++k) sh[k][warp] = v[k];
+    }
+    const bool any = __syncthreads_or(stop);
+    typedef typename Vec4<V>::t V4;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        V t = V(0);
+#pragma unroll
+        for (int w = 0; w < NW / 4; ++w) {
+            const V4 a = ((const V4 *)sh[k])[w];
+            t += (a.x + a.y) + (a.z + a.w);
+        }
+        v[k] = t;
+    }
+    return any;
+}
+
+template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solve(FemDev d) {
+    extern __shared__ __align__(16) double s_x[];  // x of the own rows and the halo; in the inner steps u, in FP32
+    float *s_u = (float *)s_x;
+    float *s_inv = (float *)(s_x + d.rp + d.hmax);  // coarse inverse, a row of P per listed part
+    __shared__ __align__(32) float sh_in[2][SNW], sh_out[3][SNW];
+    __shared__ float s_rc[SOLVE_PARTS], s_ec[SOLVE_PARTS];  // coarse residual; coarse correction of the listed parts
+    __shared__ __align__(32) double sh_d[1][SNW], sh_e[1][SNW];
+    const int part = blockIdx.x, P = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const CgState &st = *d.st;
+    if (st.outer_done) return;  // the load's verdict, the same in every block
+    const int r0 = d.part_row[part], nr = d.part_row[part + 1] - r0;
+    const int h0 = d.halo_ptr[part], nh = d.halo_ptr[part + 1] - h0;
+    const double bb = st.bb;
+    double hh = st.rr_hi, scale = st.scale;
+    long long iter = 0;
+    int outer = 0;
+    bool bad = false, done = false, stalled = false;
+
+    float r[RPT], u[RPT], w[RPT], s[RPT], p[RPT], xc[RPT], z[RPT];
+    double x[RPT], rho[RPT];
+    int width[RPT], base[RPT];
+    int out0[RPT], out1[RPT];  // the row's destinations: halo list entries dst[out0 .. out1)
+    constexpr int W = SOLVE_REG_W;
+    float av[REG ? RPT * W : 1];
+    unsigned ac[REG ? RPT * W / 2 : 1];
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+        const int l = j * SNT + tid, slice = part * (d.rp / 32) + j * SNW + warp;
+        const bool on = l < nr;
+        base[j] = d.ps_ptr[slice] + lane;
+        width[j] = d.ps_w[slice];
+        x[j] = 0.0;
+        rho[j] = on ? d.b[d.row_old[r0 + l]] : 0.0;
+        z[j] = on ? d.pz[r0 + l] : 0.f;
+        out0[j] = on ? d.dst_ptr[r0 + l] : 0;
+        out1[j] = on ? d.dst_ptr[r0 + l + 1] : 0;
+        if constexpr (REG) {
+#pragma unroll
+            for (int k = 0; k < W; k += 2) {
+                const int a = base[j] + 32 * k;
+                const unsigned c0 = k < width[j] ? d.pe_col[a] : l, c1 = k + 1 < width[j] ? d.pe_col[a + 32] : l;
+                ac[j * (W / 2) + k / 2] = c0 | c1 << 16;
+                av[j * W + k] = k < width[j] ? d.pe_val[a] : 0.f;
+                av[j * W + k + 1] = k + 1 < width[j] ? d.pe_val[a + 32] : 0.f;
+            }
+        }
+    }
+    // the parts whose coarse correction the block needs: its own first, then its halo's
+    const int a0 = d.near_ptr[part], na = d.near_ptr[part + 1] - a0;
+    for (int i = tid; i < na * P; i += SNT) s_inv[i] = d.coarse_inv[(int64_t)d.near_part[a0 + i / P] * P + i % P];
+    const int hid = SNT - 1 - tid;  // first halo entry of the thread
+    uint4 *const rec0 = d.rec[0] + h0, *const rec1 = d.rec[1] + h0;  // the block's own lists
+    uint4 *const in0 = d.psum[0] + part * P, *const in1 = d.psum[1] + part * P;
+    uint4 *const to0 = d.psum[0] + (tid < P ? tid : part) * P + part;  // this block's place in part tid's list
+    uint4 *const to1 = d.psum[1] + (tid < P ? tid : part) * P + part;
+    unsigned e = 1;  // number of the current exchange
+    while (!done && outer < FEM_MAX_OUTER) {
+        // inner start: r = D^-1/2 rho / scale, everything else zero
+        const double inv = 1.0 / scale;
+        float inv_gamma = 0.f, inv_alpha = 0.f, gamma0 = 0.f;  // of the step before; of the first
+        float rc = 0.f, sc = 0.f;                              // thread t: part t's coarse residual and S p
+        uint4 *rec = e & 1 ? d.rec[1] : d.rec[0];
+        float first[1] = {0.f};
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            const int l = j * SNT + tid;
+            r[j] = l < nr ? (float)(rho[j] * inv * d.pisd[r0 + l]) : 0.f;
+            u[j] = w[j] = s[j] = p[j] = xc[j] = 0.f;
+            first[0] += z[j] * r[j];
+            for (int o = out0[j]; o < out1[j]; ++o) st_record(rec + d.dst[o], __float_as_uint(r[j]), 0u, 0u, e);
+        }
+        solve_sum<SNW>(first, sh_out, false);
+        if (tid < P) st_record(e & 1 ? to1 : to0, 0u, 0u, __float_as_uint(first[0]), e);
+        for (int mode = 0;; mode = min(mode + 1, 2), ++e) {
+            const uint4 *mine = e & 1 ? rec1 : rec0;
+            // the blocks' sums, then the first halo records (from the last thread
+            // on, so that the warps without a sum to wait for take them first);
+            // threads without a record of their own poll nothing
+            uint4 sums, v[HB];
+            bool lost = false;
+            if (tid < P) lost = !wait_record((e & 1 ? in1 : in0) + tid, e, sums);
+#pragma unroll
+            for (int i = 0; i < HB; ++i)
+                if (i * SNT + hid < nh) lost = !wait_record(mine + i * SNT + hid, e, v[i]) || lost;
+            float sum[2] = {0.f, 0.f}, wc = 0.f;
+            if (tid < P) {
+                sum[0] = __uint_as_float(sums.x);
+                sum[1] = __uint_as_float(sums.y);
+                wc = __uint_as_float(sums.z);
+            }
+            if (solve_sum<SOLVE_PARTS / 32>(sum, sh_in, lost)) {
+                stalled = true;
+                break;
+            }
+            float alpha = 0.f, beta = 0.f;
+            if (mode > 0) {
+                const float gm = sum[0], dl = sum[1];
+                beta = gm * inv_gamma;  // zero in the first step
+                alpha = __fdividef(gm, dl - beta * gm * inv_alpha);
+                if (mode == 1) gamma0 = gm;
+                // a residual that reached the stopping test (exactly zero included,
+                // where the coefficients are 0/0) ends the inner iteration
+                const bool conv = mode == 1 ? gm == 0.f : gm <= d.inner2 * gamma0;
+                const bool nan = !isfinite(gm) || (!conv && !(isfinite(alpha) && isfinite(beta)));
+                bad = bad || nan;
+                if (nan || conv || iter >= d.max_iter) break;  // the same decision in every block
+                ++iter;
+                inv_gamma = __fdividef(1.f, gm);
+                inv_alpha = __fdividef(1.f, alpha);
+                sc = wc + beta * sc;
+                rc -= alpha * sc;
+            } else {
+                rc = wc;
+            }
+            if (tid < P) s_rc[tid] = rc;
+#pragma unroll
+            for (int j = 0; j < RPT; ++j) {
+                s[j] = w[j] + beta * s[j];
+                p[j] = u[j] + beta * p[j];
+                xc[j] += alpha * p[j];
+                r[j] -= alpha * s[j];
+            }
+            __syncthreads();
+            for (int a = warp; a < na; a += SNW) {
+                float t = 0.f;
+                for (int k = lane; k < P; k += 32) t += s_inv[a * P + k] * s_rc[k];
+                t = warp_sum(t);
+                if (lane == 0) s_ec[a] = t;
+            }
+            __syncthreads();
+            // u = r + z e(part) of the own rows and, from r_k, w_k and s_{k-1}, of the halo
+#pragma unroll
+            for (int j = 0; j < RPT; ++j) {
+                u[j] = r[j] + z[j] * s_ec[0];
+                s_u[j * SNT + tid] = u[j];
+            }
+#pragma unroll
+            for (int i = 0; i < HB; ++i) {
+                const int h = i * SNT + hid;
+                if (h < nh)
+                    s_u[d.rp + h] = __uint_as_float(v[i].x) -
+                                    alpha * (__uint_as_float(v[i].y) + beta * __uint_as_float(v[i].z)) +
+                                    d.halo_z[h0 + h] * s_ec[d.halo_near[h0 + h]];
+            }
+            for (int h = HB * SNT + hid; h < nh; h += SNT) {
+                uint4 vh;
+                lost = !wait_record(mine + h, e, vh) || lost;
+                s_u[d.rp + h] = __uint_as_float(vh.x) -
+                                alpha * (__uint_as_float(vh.y) + beta * __uint_as_float(vh.z)) +
+                                d.halo_z[h0 + h] * s_ec[d.halo_near[h0 + h]];
+            }
+            __syncthreads();
+            rec = e & 1 ? d.rec[0] : d.rec[1];  // of exchange e + 1
+            float out[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < RPT; ++j) {
+                float t = u[j];
+                if constexpr (REG) {
+#pragma unroll
+                    for (int k = 0; k < W; k += 2)
+                        if (k < width[j]) {
+                            const unsigned c = ac[j * (W / 2) + k / 2];
+                            t += av[j * W + k] * s_u[c & 0xffffu];
+                            t += av[j * W + k + 1] * s_u[c >> 16];
+                        }
+                } else {
+#pragma unroll 8
+                    for (int k = 0; k < width[j]; ++k)
+                        t += __ldg(d.pe_val + base[j] + 32 * k) * s_u[__ldg(d.pe_col + base[j] + 32 * k)];
+                }
+                w[j] = t;
+                for (int o = out0[j]; o < out1[j]; ++o)
+                    st_record(rec + d.dst[o], __float_as_uint(r[j]), __float_as_uint(t), __float_as_uint(s[j]), e + 1);
+                out[0] += r[j] * u[j];
+                out[1] += t * u[j];
+                out[2] += z[j] * t;
+            }
+            if (solve_sum<SNW>(out, sh_out, lost)) {
+                stalled = true;
+                break;
+            }
+            if (tid < P)
+                st_record(e & 1 ? to0 : to1, __float_as_uint(out[0]), __float_as_uint(out[1]),
+                          __float_as_uint(out[2]), e + 1);
+        }
+        if (stalled) break;
+        // correction and FP64 residual (exchange e + 1 carries x)
+        ++e;
+        rec = e & 1 ? d.rec[1] : d.rec[0];
+        __syncthreads();  // the last step's reads of u
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            if (j * SNT + tid < nr) x[j] += scale * d.pisd[r0 + j * SNT + tid] * (double)xc[j];
+            s_x[j * SNT + tid] = x[j];
+            const unsigned long long b = __double_as_longlong(x[j]);
+            for (int o = out0[j]; o < out1[j]; ++o) st_record(rec + d.dst[o], (unsigned)b, (unsigned)(b >> 32), 0u, e);
+        }
+        bool lost = false;
+        for (int h = tid; h < nh; h += SNT) {
+            uint4 vh;
+            lost = !wait_record((e & 1 ? rec1 : rec0) + h, e, vh) || lost;
+            s_x[d.rp + h] = __longlong_as_double((long long)((unsigned long long)vh.x | (unsigned long long)vh.y << 32));
+        }
+        __syncthreads();
+        double sq[1] = {0.0};
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            const int l = j * SNT + tid;
+            double t = 0.0;
+            if (l < nr) {
+                double sx = d.pdiag[r0 + l] * x[j];
+#pragma unroll 4
+                for (int k = 0; k < width[j]; ++k) sx += __ldg(d.pe_val64 + base[j] + 32 * k) * s_x[__ldg(d.pe_col + base[j] + 32 * k)];
+                t = d.b[d.row_old[r0 + l]] - sx;
+            }
+            rho[j] = t;
+            sq[0] += t * t;
+        }
+        if (solve_sum<SNW>(sq, sh_d, lost)) {
+            stalled = true;
+            break;
+        }
+        if (tid < P) {
+            const unsigned long long b = __double_as_longlong(sq[0]);
+            st_record(e & 1 ? to1 : to0, (unsigned)b, (unsigned)(b >> 32), 0u, e);
+        }
+        double tot[1] = {0.0};
+        lost = false;
+        if (tid < P) {
+            uint4 vt;
+            lost = !wait_record((e & 1 ? in1 : in0) + tid, e, vt);
+            tot[0] = __longlong_as_double((long long)((unsigned long long)vt.x | (unsigned long long)vt.y << 32));
+        }
+        if (solve_sum<SNW>(tot, sh_e, lost)) {
+            stalled = true;
+            break;
+        }
+        ++e;
+        ++outer;
+        hh = tot[0];
+        scale = sqrt(hh / (double)d.nf);
+        if (!(scale > 0.0)) scale = 1.0;
+        bad = bad || !isfinite(hh);
+        done = bad || hh <= d.tol2 * bb || iter >= d.max_iter;
+    }
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+        const int l = j * SNT + tid;
+        if (l < nr) d.x[d.row_old[r0 + l]] = x[j];
+    }
+    if (tid == 0 && (part == 0 || stalled)) {
+        CgState &o = *d.st;
+        if (stalled) o.stalled = 1;
+        if (part == 0) {
+            o.rr_hi = hh;
+            o.iter = iter;
+            o.outer = outer;
+            o.bad = bad;
+            o.outer_done = done;
+        }
+    }
+}
+
 // g_j = (mean of the nodal m over the triangle) . n_j + phi_1(opposite node) / h_j
 // (dphi_1/dn = -phi_1(o)/h_j: the other three nodes are boundary nodes, phi_1 = 0)
 template <typename T>
@@ -556,8 +930,45 @@ cudaError_t launch_fem_load(const FemDev &d, int prec, const void *m, cudaStream
         k_fem_load<double><<<row_blocks(d), NT, 0, s>>>(d, (const double *)m);
     else
         k_fem_load<float><<<row_blocks(d), NT, 0, s>>>(d, (const float *)m);
-    k_cg_scale<<<elem_blocks(d), NT, 0, s>>>(d);
+    if (d.parts == 0) k_cg_scale<<<elem_blocks(d), NT, 0, s>>>(d);
     return cudaGetLastError();
+}
+
+namespace {
+typedef void (*SolveKernel)(FemDev);
+SolveKernel solve_kernel(const FemDev &d) {
+    if (d.solve_reg) return d.rpt == 1 ? k_cg_solve<1, true> : k_cg_solve<2, true>;
+    switch (d.rpt) {
+        case 1: return k_cg_solve<1, false>;
+        case 2: return k_cg_solve<2, false>;
+        case 4: return k_cg_solve<4, false>;
+        case 8: return k_cg_solve<8, false>;
+        default: return k_cg_solve<12, false>;
+    }
+}
+}  // namespace
+
+size_t solve_smem(const FemDev &d) {
+    return sizeof(double) * (size_t)(d.rp + d.hmax) + sizeof(float) * (size_t)d.near_max * d.parts;
+}
+
+cudaError_t solve_blocks(const FemDev &d, int *blocks) {
+    int dev = 0, sms = 0, coop = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void *)solve_kernel(d), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem(d));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, solve_kernel(d), SNT, solve_smem(d));
+    *blocks = coop ? sms * per : 0;
+    return e;
+}
+
+cudaError_t launch_cg_solve(const FemDev &d, cudaStream_t s) {
+    FemDev arg = d;
+    void *args[] = {&arg};
+    return cudaLaunchCooperativeKernel((const void *)solve_kernel(d), dim3(d.parts), dim3(SNT), args, solve_smem(d), s);
 }
 
 cudaError_t launch_cg_iteration(const FemDev &d, int parity, cudaStream_t s) {

@@ -11,10 +11,11 @@
 //     the mean of the four nodal values (m is P1);
 //   * the boundary's triangle-integrated plan (opts.integration = 1) and a
 //     probe set of the free nodes, so that phi_2 reaches every node;
-//   * the solve as one CUDA graph: WHILE nodes over the corrections and,
+//   * the solve's row parts, halos and coarse matrix (one cooperative launch),
+//     or for systems too large for that the solve as one CUDA graph: WHILE nodes over the corrections and,
 //     inside each, over passes of FEM_CHUNK inner conjugate-gradient
 //     launches, their handles set on the device from the solver's state.
-// Evaluation (slp_potential_eval): b = B m; the solve graph (FP32 inner
+// Evaluation (slp_potential_eval): b = B m; the solve (FP32 inner
 // steps, FP64 corrections, no host round trip); the charges g; phi_2 through
 // the plan and its probes; phi = phi_1 + phi_2.  The host waits for the
 // solve's state only, to return its status.
@@ -421,6 +422,207 @@ slp_status assemble(const double *X, int64_t N, const int32_t *tets, int64_t K, 
     return SLP_OK;
 }
 
+// Cuts rows [b, e) of `order` into parts [k0, k1) of equal size, halving along
+// the longest axis of their box (recursive coordinate bisection); part k ends
+// at row end[k].
+void bisect(std::vector<int> &order, const std::vector<double> &pos, int64_t b, int64_t e, int k0, int k1,
+            std::vector<int> &end) {
+    if (k1 - k0 == 1) {
+        std::sort(order.begin() + b, order.begin() + e);  // the mesh's own order within a part
+        end[k0 + 1] = (int)e;
+        return;
+    }
+    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+    for (int64_t i = b; i < e; ++i)
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = std::min(lo[d], pos[3 * (int64_t)order[i] + d]);
+            hi[d] = std::max(hi[d], pos[3 * (int64_t)order[i] + d]);
+        }
+    int ax = 0;
+    for (int d = 1; d < 3; ++d)
+        if (hi[d] - lo[d] > hi[ax] - lo[ax]) ax = d;
+    const int km = (k0 + k1) / 2;
+    const int64_t mid = b + (e - b) * (km - k0) / (k1 - k0);
+    std::nth_element(order.begin() + b, order.begin() + mid, order.begin() + e, [&](int x, int y) {
+        const double px = pos[3 * (int64_t)x + ax], py = pos[3 * (int64_t)y + ax];
+        return px != py ? px < py : x < y;
+    });
+    bisect(order, pos, b, mid, k0, km, end);
+    bisect(order, pos, mid, e, km, k1, end);
+}
+
+// Inverse of a symmetric positive definite n x n matrix in place (Gauss-Jordan
+// on the diagonal pivots); false when a pivot is not positive.
+bool invert_spd(std::vector<double> &A, int n) {
+    for (int k = 0; k < n; ++k) {
+        const double piv = A[(size_t)k * n + k];
+        if (!(piv > 0.0) || !std::isfinite(piv)) return false;
+        A[(size_t)k * n + k] = 1.0;
+        for (int j = 0; j < n; ++j) A[(size_t)k * n + j] /= piv;
+        for (int i = 0; i < n; ++i) {
+            if (i == k) continue;
+            const double f = A[(size_t)i * n + k];
+            A[(size_t)i * n + k] = 0.0;
+            for (int j = 0; j < n; ++j) A[(size_t)i * n + j] -= f * A[(size_t)k * n + j];
+        }
+    }
+    return true;
+}
+
+// Set-up of the one-launch solve: parts, local columns, exchange buffers.
+// Leaves d.parts = 0 where it does not apply (rows or halo too many for a
+// block, or the device cannot hold a block per part at once).
+slp_status build_parts(slp_potential_s &P, const FemHost &H, const std::vector<double> &Xf) {
+    slp::FemDev &d = P.d;
+    const int64_t nf = H.nf;
+    int sms = 0;
+    FTRY(cu(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P.device), "device"));
+    // a block per SM; small systems fewer, at least 128 rows each
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, slp::SOLVE_PARTS), (nf + 127) / 128));
+    const int64_t most = (nf + parts - 1) / parts;
+    int rpt = 0;
+    for (int k : slp::SOLVE_RPT)
+        if (rpt == 0 && most <= (int64_t)k * slp::SOLVE_THREADS) rpt = k;
+    if (rpt == 0) return SLP_OK;
+    const int rp = rpt * slp::SOLVE_THREADS, ns = rp / 32;
+    std::vector<int> order(nf), first(parts + 1, 0);
+    for (int64_t i = 0; i < nf; ++i) order[i] = (int)i;
+    bisect(order, Xf, 0, nf, 0, parts, first);
+    std::vector<int> row_of(nf);
+    for (int64_t i = 0; i < nf; ++i) row_of[order[i]] = (int)i;
+    std::vector<int> halo_ptr(parts + 1, 0), halo, ps_w((size_t)parts * ns, 0);
+    std::vector<int> ps_ptr((size_t)parts * ns + 1, 0);
+    std::vector<unsigned short> col;
+    std::vector<float> val;
+    std::vector<double> val64, diag(nf);
+    std::vector<int> local(nf, -1);  // position in the current part's halo
+    int hmax = 0, wmax = 0;
+    for (int64_t i = 0; i < nf; ++i) diag[i] = 1.0 / H.dinv[order[i]];
+    for (int k = 0; k < parts; ++k) {
+        const int b = first[k], e = first[k + 1];
+        const size_t h0 = halo.size();
+        for (int i = b; i < e; ++i)
+            for (int64_t q = H.s_ptr[order[i]]; q < H.s_ptr[order[i] + 1]; ++q) {
+                const int c = row_of[H.s_col[q]];
+                if ((c < b || c >= e) && local[c] < 0) {
+                    local[c] = 0;
+                    halo.push_back(c);
+                }
+            }
+        std::sort(halo.begin() + h0, halo.end());
+        for (size_t q = h0; q < halo.size(); ++q) local[halo[q]] = (int)(q - h0);
+        const int nh = (int)(halo.size() - h0);
+        if (rp + nh > 65535) return SLP_OK;
+        hmax = std::max(hmax, nh);
+        halo_ptr[k + 1] = (int)halo.size();
+        for (int t = 0; t < ns; ++t) {
+            int wd = 0;
+            for (int l = 32 * t; l < std::min(32 * t + 32, e - b); ++l)
+                wd = std::max(wd, (int)(H.s_ptr[order[b + l] + 1] - H.s_ptr[order[b + l]]) - 1);
+            ps_w[(size_t)k * ns + t] = wd;
+            wmax = std::max(wmax, wd);
+            const int64_t at = ps_ptr[(size_t)k * ns + t];
+            if (at + 32 * (int64_t)wd > INT32_MAX) return SLP_OK;
+            ps_ptr[(size_t)k * ns + t + 1] = (int)(at + 32 * (int64_t)wd);
+            col.resize(at + 32 * (size_t)wd);
+            val.resize(at + 32 * (size_t)wd, 0.f);
+            val64.resize(at + 32 * (size_t)wd, 0.0);
+            for (int l = 32 * t; l < 32 * t + 32; ++l) {
+                int64_t o = at + l - 32 * t, o_end = at + 32 * (int64_t)wd;
+                if (l < e - b) {
+                    const int i = b + l;
+                    for (int64_t q = H.s_ptr[order[i]]; q < H.s_ptr[order[i] + 1]; ++q) {
+                        const int c = row_of[H.s_col[q]];
+                        if (c == i) continue;
+                        col[o] = (unsigned short)(c >= b && c < e ? c - b : rp + local[c]);
+                        val64[o] = H.s_val[q];
+                        val[o] = (float)(H.s_val[q] / std::sqrt(diag[i] * diag[c]));
+                        o += 32;
+                    }
+                }
+                for (; o < o_end; o += 32) col[o] = (unsigned short)l;  // zero entries at the row's own column
+            }
+        }
+        for (size_t q = h0; q < halo.size(); ++q) local[halo[q]] = -1;
+    }
+    // coarse space: A_ab = sum of S_ij over i in part a, j in part b
+    std::vector<int> part_of(nf);
+    for (int k = 0; k < parts; ++k)
+        for (int i = first[k]; i < first[k + 1]; ++i) part_of[i] = k;
+    std::vector<double> A((size_t)parts * parts, 0.0);
+    for (int64_t i = 0; i < nf; ++i)
+        for (int64_t q = H.s_ptr[order[i]]; q < H.s_ptr[order[i] + 1]; ++q)
+            A[(size_t)part_of[i] * parts + part_of[row_of[H.s_col[q]]]] += H.s_val[q];
+    if (!invert_spd(A, parts)) return SLP_OK;
+    const std::vector<float> inv(A.begin(), A.end());
+    std::vector<int> near_ptr(parts + 1, 0), near_part;
+    std::vector<unsigned char> halo_near(halo.size());
+    std::vector<float> halo_z(halo.size()), z(nf);
+    for (int64_t i = 0; i < nf; ++i) z[i] = (float)std::sqrt(diag[i]);
+    int near_max = 0;
+    for (int k = 0; k < parts; ++k) {
+        std::vector<int> place(parts, -1);
+        const size_t n0 = near_part.size();
+        place[k] = 0;
+        near_part.push_back(k);
+        for (int h = halo_ptr[k]; h < halo_ptr[k + 1]; ++h) {
+            int &at = place[part_of[halo[h]]];
+            if (at < 0) {
+                at = (int)(near_part.size() - n0);
+                near_part.push_back(part_of[halo[h]]);
+            }
+            halo_near[h] = (unsigned char)at;  // at most SOLVE_PARTS - 1
+            halo_z[h] = z[halo[h]];
+        }
+        near_ptr[k + 1] = (int)near_part.size();
+        near_max = std::max(near_max, near_ptr[k + 1] - near_ptr[k]);
+    }
+    d.parts = parts;
+    d.rpt = rpt;
+    d.rp = rp;
+    d.hmax = hmax;
+    d.near_max = near_max;
+    d.solve_reg = rpt <= 2 && wmax <= slp::SOLVE_REG_W;
+    int fit = 0;
+    if (slp::solve_smem(d) > 200 * 1024 || slp::solve_blocks(d, &fit) != cudaSuccess || fit < parts) {
+        cudaGetLastError();
+        d.parts = 0;
+        return SLP_OK;
+    }
+    FTRY(upload(P, (int **)&d.part_row, first.data(), first.size()));
+    FTRY(upload(P, (int **)&d.row_old, order.data(), order.size()));
+    FTRY(upload(P, (int **)&d.halo_ptr, halo_ptr.data(), halo_ptr.size()));
+    d.nhalo = (int64_t)halo.size();
+    std::vector<int> dst_ptr(nf + 1, 0), dst(halo.size());
+    for (int c : halo) ++dst_ptr[c + 1];
+    for (int64_t i = 0; i < nf; ++i) dst_ptr[i + 1] += dst_ptr[i];
+    {
+        std::vector<int> next(dst_ptr.begin(), dst_ptr.end() - 1);
+        for (size_t h = 0; h < halo.size(); ++h) dst[next[halo[h]]++] = (int)h;
+    }
+    FTRY(upload(P, (int **)&d.dst_ptr, dst_ptr.data(), dst_ptr.size()));
+    FTRY(upload(P, (int **)&d.dst, dst.data(), dst.size()));
+    FTRY(upload(P, (int **)&d.ps_ptr, ps_ptr.data(), ps_ptr.size()));
+    FTRY(upload(P, (int **)&d.ps_w, ps_w.data(), ps_w.size()));
+    FTRY(upload(P, (unsigned short **)&d.pe_col, col.data(), col.size()));
+    FTRY(upload(P, (float **)&d.pe_val, val.data(), val.size()));
+    FTRY(upload(P, (double **)&d.pe_val64, val64.data(), val64.size()));
+    FTRY(upload(P, (double **)&d.pdiag, diag.data(), diag.size()));
+    FTRY(upload(P, (float **)&d.pz, z.data(), z.size()));
+    FTRY(upload(P, (int **)&d.near_ptr, near_ptr.data(), near_ptr.size()));
+    FTRY(upload(P, (int **)&d.near_part, near_part.data(), near_part.size()));
+    FTRY(upload(P, (float **)&d.halo_z, halo_z.data(), halo_z.size()));
+    FTRY(upload(P, (unsigned char **)&d.halo_near, halo_near.data(), halo_near.size()));
+    FTRY(upload(P, (float **)&d.coarse_inv, inv.data(), inv.size()));
+    for (double &v : diag) v = 1.0 / std::sqrt(v);
+    FTRY(upload(P, (double **)&d.pisd, diag.data(), diag.size()));
+    for (int q = 0; q < 2; ++q) {
+        FTRY(upload(P, &d.rec[q], (const uint4 *)nullptr, halo.size()));
+        FTRY(upload(P, &d.psum[q], (const uint4 *)nullptr, (size_t)parts * parts));
+    }
+    return SLP_OK;
+}
+
 slp_status build(slp_potential_s &P, const double *X, int64_t N, const int32_t *tets, int64_t K, double tolerance,
                  const slp_plan_opts *opts) {
     FemHost H;
@@ -474,10 +676,12 @@ slp_status build(slp_potential_s &P, const double *X, int64_t N, const int32_t *
     slp::FemDev &d = P.d;
     d.nf = nf;
     d.nblk_max = 8 * 152;
-    FTRY(upload(P, (int64_t **)&d.s_ptr, s_ptr.data(), s_ptr.size()));
-    FTRY(upload(P, (int **)&d.s_col, s_col.data(), s_col.size()));
-    FTRY(upload(P, (double **)&d.s_val, s_val.data(), s_val.size()));
-    {
+    if (nf > 0) FTRY(build_parts(P, H, Xf));
+    const bool chain = d.parts == 0;  // a launch per step
+    if (chain) {
+        FTRY(upload(P, (int64_t **)&d.s_ptr, s_ptr.data(), s_ptr.size()));
+        FTRY(upload(P, (int **)&d.s_col, s_col.data(), s_col.size()));
+        FTRY(upload(P, (double **)&d.s_val, s_val.data(), s_val.size()));
         // FP32 copy in slices of 32 rows (column-major within a slice)
         const int64_t nsl = (nf + 31) / 32;
         std::vector<int64_t> sl_ptr(nsl + 1, 0);
@@ -531,15 +735,17 @@ slp_status build(slp_potential_s &P, const double *X, int64_t N, const int32_t *
     d.x = vec + stride;
     d.rho = vec + 2 * stride;
     d.part = vec + 3 * stride;
-    float *v32 = nullptr;
-    FTRY(upload(P, &v32, (const float *)nullptr, (size_t)stride * 2 + 6 * d.nblk_max));
-    d.xc = v32;
-    d.p = v32 + stride;
-    d.part32 = v32 + 2 * stride;
-    float4 *v4 = nullptr;
-    FTRY(upload(P, &v4, (const float4 *)nullptr, (size_t)stride * 2));
-    d.v[0] = v4;
-    d.v[1] = v4 + stride;
+    if (chain) {
+        float *v32 = nullptr;
+        FTRY(upload(P, &v32, (const float *)nullptr, (size_t)stride * 2 + 6 * d.nblk_max));
+        d.xc = v32;
+        d.p = v32 + stride;
+        d.part32 = v32 + 2 * stride;
+        float4 *v4 = nullptr;
+        FTRY(upload(P, &v4, (const float4 *)nullptr, (size_t)stride * 2));
+        d.v[0] = v4;
+        d.v[1] = v4 + stride;
+    }
     FTRY(upload(P, &d.st, (const slp::CgState *)nullptr, 1));
     FTRY(cu(cudaMemset(d.st, 0, sizeof(slp::CgState)), "state"));
     FTRY(cu(cudaMemset(d.x, 0, sizeof(double) * stride), "phi_1"));
@@ -561,7 +767,7 @@ slp_status build(slp_potential_s &P, const double *X, int64_t N, const int32_t *
     for (auto &e : P.tev) FTRY(cu(cudaEventCreate(&e), "event"));
 
     // the solve graph
-    if (nf > 0) {
+    if (nf > 0 && chain) {
         FTRY(cu(cudaStreamCreateWithFlags(&P.cap, cudaStreamNonBlocking), "stream"));
         FTRY(cu(build_solve_graph(P), "solve graph"));
         FTRY(cu(cudaGraphInstantiate(&P.exec, P.graph, 0), "solve graph"));
@@ -607,14 +813,17 @@ slp_status slp_potential_eval(slp_potential_t P, const void *d_m, void *d_phi, v
     const slp::FemDev &d = P->d;
     int64_t iters = 0, outer = 0;
     double res = 0.0;
-    bool bad = false, converged = true;
+    bool bad = false, stalled = false, converged = true;
     FTRY(cu(cudaEventRecord(P->tev[0], s), "event"));
     if (P->nf > 0) {
         // the load, then the solve graph (its loops end on the device: the
         // inner steps at max_iter in all, the corrections at FEM_MAX_OUTER);
         // the state is copied behind it for the status
         FTRY(cu(slp::launch_fem_load(d, P->prec, d_m, s), "load"));
-        FTRY(cu(cudaGraphLaunch(P->exec, s), "solve graph"));
+        if (d.parts > 0)
+            FTRY(cu(slp::launch_cg_solve(d, s), "solve"));
+        else
+            FTRY(cu(cudaGraphLaunch(P->exec, s), "solve graph"));
         FTRY(cu(cudaMemcpyAsync(P->h_st, d.st, sizeof(slp::CgState), cudaMemcpyDeviceToHost, s), "state copy"));
         FTRY(cu(cudaEventRecord(P->ev[0], s), "event"));
     }
@@ -633,12 +842,14 @@ slp_status slp_potential_eval(slp_potential_t P, const void *d_m, void *d_phi, v
         outer = h.outer;
         res = h.bb > 0 ? std::sqrt(std::max(h.rr_hi, 0.0) / h.bb) : 0.0;
         bad = h.bad != 0;
+        stalled = h.stalled != 0;
         converged = h.outer_done && !bad && (h.bb == 0.0 || h.rr_hi <= d.tol2 * h.bb);
     }
     P->timed = true;
     P->last_iter = iters;
     P->last_outer = outer;
     P->last_res = res;
+    if (stalled) return slp_fail(SLP_ERR_TIMEOUT, "a wait between the blocks of the solve gave up");
     if (bad) return slp_fail(SLP_ERR_NONFINITE, "the iteration met a non-finite value");
     if (!converged)
         return slp_fail(SLP_ERR_TOLERANCE_INFEASIBLE,

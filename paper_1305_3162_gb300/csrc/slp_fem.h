@@ -38,6 +38,7 @@ struct CgState {
     int outer_done;     // |b - S x| <= tol |b|, out of iterations, or non-finite
     int bad;            // a non-finite scalar was seen
     unsigned count[2];  // arrival counters of the load and residual launches
+    int stalled;        // a wait between the blocks of the one-launch solve gave up
     int loops_outer;    // passes of the solve graph's correction loop
     int loops_inner;    // passes of its inner loop in the current correction
 };
@@ -79,6 +80,39 @@ struct FemDev {
     double tol2 = 0.0;    // outer stop: |b - S x|^2 <= tol2 |b|^2
     float inner2 = 0.f;   // inner stop: r.r <= inner2 r0.r0
     long long max_iter = 0;
+    // The one-launch solve (parts > 0): the free rows cut into `parts` compact
+    // sets of at most rp rows, one block each, renumbered part by part.  A
+    // block's columns are its own rows (local index < rp) and its halo, the
+    // other parts' rows its entries reach (rp + position in its halo list).
+    int parts = 0, rpt = 0, rp = 0, hmax = 0;  // rpt: rows per thread, rp = SOLVE_THREADS rpt
+    int solve_reg = 0;                         // 1: the matrix fits the threads' registers
+    const int *part_row = nullptr;             // [parts + 1] first row of each part
+    const int *row_old = nullptr;              // [nf] free index of a row
+    const int *halo_ptr = nullptr;             // [parts + 1] the parts' halo lists, nhalo entries in all
+    int64_t nhalo = 0;
+    const int *dst_ptr = nullptr, *dst = nullptr;  // [nf + 1], the halo list entries that hold each row
+    // off-diagonal entries in slices of 32 rows of a part (slice t of part k at
+    // k rp / 32 + t, entry e of lane l at ps_ptr[slice] + 32 e + l): local
+    // column, S_ij / sqrt(S_ii S_jj) in FP32, S_ij in FP64
+    const int *ps_ptr = nullptr;
+    const int *ps_w = nullptr;
+    const unsigned short *pe_col = nullptr;
+    const float *pe_val = nullptr;
+    const double *pe_val64 = nullptr;
+    const double *pdiag = nullptr, *pisd = nullptr;  // [nf] S_ii, 1 / sqrt(S_ii)
+    const float *pz = nullptr;      // [nf] sqrt(S_ii)
+    // coarse space: the parts each part needs the correction of (its own first),
+    // at most near_max of them; each halo entry's z and its part's place in that
+    // list; the inverse of the parts' matrix [parts][parts]
+    const int *near_ptr = nullptr, *near_part = nullptr;
+    int near_max = 0;
+    const float *halo_z = nullptr;
+    const unsigned char *halo_near = nullptr;
+    const float *coarse_inv = nullptr;
+    // exchanged between blocks, by parity of the exchange: a record per halo
+    // list entry and a record of partial sums per pair of blocks (psum[reader parts + writer]),
+    // each 16 bytes with its exchange number
+    uint4 *rec[2] = {nullptr, nullptr}, *psum[2] = {nullptr, nullptr};
     // boundary triangles: nodes (a, b, c) wound outward and the free index of the
     // owning tetrahedron's fourth node (-1 when it lies on the boundary); unit
     // normal and 1/h, h the tetrahedron's height over the triangle
@@ -91,6 +125,10 @@ struct FemDev {
 };
 
 constexpr int FEM_THREADS = 256;
+constexpr int SOLVE_THREADS = 512;  // threads of a block of the one-launch solve
+constexpr int SOLVE_PARTS = 256;    // blocks at most (a thread reads one block's sums)
+constexpr int SOLVE_RPT[] = {1, 2, 4, 8, 12};  // rows per thread it is compiled for
+constexpr int SOLVE_REG_W = 16;     // most off-diagonal entries of a row kept in registers (rpt <= 2)
 constexpr int FEM_CHUNK = 16;       // inner launches per pass of the inner loop (even: parities repeat)
 constexpr double FEM_INNER = 1e-4;  // each correction's inner steps cut its residual by this factor
 constexpr int FEM_MAX_OUTER = 64;   // corrections at most
@@ -101,6 +139,11 @@ enum FemLoop { LOOP_OUTER_START, LOOP_OUTER_NEXT, LOOP_INNER_START, LOOP_INNER_N
 
 // b = B m and x = 0; the first inner iteration set up from r = b / scale
 cudaError_t launch_fem_load(const FemDev &d, int prec, const void *m, cudaStream_t s);
+// The whole solve in one cooperative launch of d.parts blocks (after
+// launch_fem_load); solve_blocks: how many such blocks fit the device at once.
+cudaError_t launch_cg_solve(const FemDev &d, cudaStream_t s);
+cudaError_t solve_blocks(const FemDev &d, int *blocks);
+size_t solve_smem(const FemDev &d);
 // one inner launch (parity: the launch's index mod 2; each inner iteration
 // starts at parity 0 with a set-up launch, then one step per launch)
 cudaError_t launch_cg_iteration(const FemDev &d, int parity, cudaStream_t s);
