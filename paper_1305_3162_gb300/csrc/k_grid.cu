@@ -656,7 +656,11 @@ __global__ void k_wtab_build(const float4 *__restrict__ src_grid, int64_t Q, dou
 // tile plus halo of grid B is staged in shared memory (same padded layout as
 // the spread), together with the item's target coordinates, permutation,
 // near-field parts and window values; then one warp per target sums its
-// (2M)^3 window box, lanes over the (y, z) rows of the box.
+// (2M)^3 window box, lanes over the (y, z) rows of the box.  An item of fewer
+// targets than warps gives each target two or four warps, which take the
+// passes over its rows in turn; their parts are added in order.
+
+constexpr int GATHER_SPLIT = 4;  // most warps of one target
 
 template <typename T, int M, int TS>
 __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) {
@@ -671,7 +675,8 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
     T *wv = tile + ((G::SIZE + 3) & ~3);  // [GC][3W]
     T *sf = wv + GC * GW;               // [3][GC] fractions
     T *sphi = sf + 3 * GC;              // [GC] near-field parts
-    int *sidx = (int *)(sphi + GC);     // [2][GC] packed cell, output index
+    T *part = sphi + GC;                // [GATHER_SPLIT][8] sums of one pass group of a shared target
+    int *sidx = (int *)(part + 8 * GATHER_SPLIT);  // [2][GC] packed cell, output index
 
     const TileItem it = p.gather_items[blockIdx.x];
     const int nt = it.end - it.begin;
@@ -772,21 +777,27 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
     }
     __syncthreads();
 
-    for (int t = warp; t < nt; t += nwarps) {
+    // warps per target
+    const int wpt = nt >= nwarps ? 1 : (2 * nt >= nwarps ? 2 : GATHER_SPLIT);
+    auto put = [&](int t, T v) {
+        v += sphi[t];
+        check_finite3(p, v, v, v);
+        phi[sidx[GC + t]] = v;
+    };
+    for (int u = warp; u < nt * wpt; u += nwarps) {
+        const int t = u / wpt, sub = u - t * wpt;
         int cx, cy, cz;
         unpack_cell(sidx[t], cx, cy, cz);
         const int lx = cx - it.c0x, ly = cy - it.c0y, lz = cz - it.c0z;
-        if ((unsigned)lx >= (unsigned)TS || (unsigned)ly >= (unsigned)TS || (unsigned)lz >= (unsigned)TS) {
-            set_error(p.err, DEV_ERR_BAD_ITEM);
-            continue;
-        }
+        const bool ok = (unsigned)lx < (unsigned)TS && (unsigned)ly < (unsigned)TS && (unsigned)lz < (unsigned)TS;
+        if (!ok) set_error(p.err, DEV_ERR_BAD_ITEM);
         const T *w = wv + t * GW;
-        const T *base = tile + lz * PS + ly * RS + lx + XO;
+        const T *base = tile + (ok ? lz * PS + ly * RS + lx : 0) + XO;
         T acc = T(0);
 #pragma unroll
         for (int rep = 0; rep < (W * W + 31) / 32; ++rep) {
             const int pi = lane + 32 * rep;
-            if (pi < W * W) {
+            if (pi < W * W && (rep & (wpt - 1)) == sub) {
                 const int iy = pi % W, iz = pi / W;
                 const T *row = base + iz * PS + iy * RS;
                 T s = T(0);
@@ -796,10 +807,19 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
             }
         }
         acc = warp_sum(acc);
-        if (lane == 0) {
-            const T v = acc + sphi[t];
-            check_finite3(p, v, v, v);
-            phi[sidx[GC + t]] = v;
+        if (lane == 0 && ok) {
+            if (wpt == 1)
+                put(t, acc);
+            else
+                part[t * GATHER_SPLIT + sub] = acc;
+        }
+    }
+    if (wpt > 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < nt) {
+            T v = T(0);
+            for (int k = 0; k < wpt; ++k) v += part[threadIdx.x * GATHER_SPLIT + k];
+            put(threadIdx.x, v);
         }
     }
 }
@@ -816,13 +836,27 @@ __global__ void k_zero4(float4 *p, int64_t n4) {
 // Spread of wide windows (2m > 10): one tile per block, no per-warp copies.
 // The block stages the window values of SB sources at a time in shared
 // memory (from the FP64 window table or evaluated), the x values times the
-// charge; then warp w adds, source after source, the box points of the
-// tile's z planes z = w, w + nwarps, ... (lanes over the (x, y) points of a
-// plane), so every tile element is updated by one warp in source order: no
-// atomics, and one tile holds many sources, so the flush of the halo tile
-// into the grid (global atomics) is shared by all of them.
+// charge.  It has M warps, and warp w owns the tile's z planes z = w (mod M):
+// of every source's 2M planes exactly two, so the warps' work is equal and each
+// tile element is updated by one warp in source order (no atomics).  A lane
+// holds the box row of one y in one of the two planes: per source one product
+// wy wz and 2M multiply-adds into registers, which are read from and go back to
+// the tile once per run of sources of the same cell.
+//
+// In FP64 (M = 7) the bound is the FP64 pipe, 2 lanes per SM: 15 instructions
+// a warp and source, 28 of 32 lanes busy, where a product per box point and
+// planes dealt to 8 warps took twice the instructions at 7/8 of the warps.
+// Level-4 sphere at 128^3 (35840 sources): 595 -> 265 us; the 8x8 cube:
+// 90 -> 35 us.
+template <typename T, int M, int TS> struct PlaneGeom {
+    static constexpr int W = 2 * M;
+    static constexpr int TE = TS + W - 1;
+    static constexpr int RS = TE | 1;  // odd: the lanes of a row update, one per y, on different banks
+    static constexpr int PS = TE * RS;
+    static constexpr int SIZE = TE * PS;
+};
 template <typename T, int M, int TS> struct PlaneSmem {
-    typedef TileGeom<M, TS> G;
+    typedef PlaneGeom<T, M, TS> G;
     static constexpr int SB = 32;  // sources per staged batch
     __host__ __device__ static size_t coef_off() { return ((size_t)G::SIZE + 3) & ~(size_t)3; }
     __host__ __device__ static size_t wv_off(int wdeg) {
@@ -834,15 +868,14 @@ template <typename T, int M, int TS> struct PlaneSmem {
 };
 
 template <typename T, int M, int TS>
-__global__ void __launch_bounds__(256) k_spread_planes(DevPlan p, int fused_kind, const T *__restrict__ in) {
-    pdl_wait();
-    pdl_trigger();
+__global__ void __launch_bounds__(32 * M) k_spread_planes(DevPlan p, int fused_kind, const T *__restrict__ in) {
     typedef typename VecT<T>::T4 T4;
-    typedef TileGeom<M, TS> G;
+    typedef PlaneGeom<T, M, TS> G;
     typedef PlaneSmem<T, M, TS> SM;
-    constexpr int W = G::W, TE = G::TE, RS = G::RS, PS = G::PS, XO = G::XO, XE = G::XE, SB = SM::SB;
+    constexpr int W = G::W, TE = G::TE, RS = G::RS, PS = G::PS, SB = SM::SB, NT = 32 * M;
+    static_assert(2 * W <= 32, "a lane per row of two planes");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     T *tile = (T *)smem_raw;
     T *coef = tile + SM::coef_off();
     T *wv = tile + SM::wv_off(p.wdeg);  // [SB][3W]
@@ -852,16 +885,19 @@ __global__ void __launch_bounds__(256) k_spread_planes(DevPlan p, int fused_kind
     const TileItem it = p.spread_items[blockIdx.x];
     const int nsrc = it.end - it.begin;
     if (p.ks > 1) in = (const T *)p.in_st[blockIdx.y];  // state of a batched launch
-    for (int i = threadIdx.x; i < G::SIZE; i += blockDim.x) tile[i] = T(0);
+    for (int i = threadIdx.x; i < G::SIZE; i += NT) tile[i] = T(0);
     if (sizeof(T) == 4)
-        for (int i = threadIdx.x; i < ncoef; i += blockDim.x) coef[i] = ((const T *)p.wcoef)[i];
+        for (int i = threadIdx.x; i < ncoef; i += NT) coef[i] = ((const T *)p.wcoef)[i];
     const T inv_m = T(1) / T(M);
     const T beta = (T)p.beta, isb = (T)p.inv_sinh_beta;
     const T4 *src = (const T4 *)p.src_grid;
+    const int iy = lane % W, upper = lane / W;  // the lane's row, in the warp's lower or upper plane
+    pdl_wait();
+    pdl_trigger();
     for (int b0 = 0; b0 < nsrc; b0 += SB) {
         const int nb = min(SB, nsrc - b0);
         __syncthreads();  // the previous batch's values are no longer read; the tile and coef are set
-        for (int idx = threadIdx.x; idx < nb * 3 * W; idx += blockDim.x) {
+        for (int idx = threadIdx.x; idx < nb * 3 * W; idx += NT) {
             const int sidx = idx / (3 * W), j = idx - sidx * 3 * W, ax = j / W, i = j - ax * W;
             const int k = it.begin + b0 + sidx;
             T v;
@@ -883,7 +919,7 @@ __global__ void __launch_bounds__(256) k_spread_planes(DevPlan p, int fused_kind
                 v *= fused_kind >= 0 ? source_charge<T>(p, k, fused_kind, in) : ((const T *)p.qbuf)[k];
             wv[sidx * 3 * W + j] = v;
         }
-        for (int sidx = threadIdx.x; sidx < nb; sidx += blockDim.x) {
+        for (int sidx = threadIdx.x; sidx < nb; sidx += NT) {
             int cx, cy, cz;
             unpack_cell(packed_cell(src[it.begin + b0 + sidx].w), cx, cy, cz);
             const int lx = cx - it.c0x, ly = cy - it.c0y, lz = cz - it.c0z;
@@ -895,35 +931,42 @@ __global__ void __launch_bounds__(256) k_spread_planes(DevPlan p, int fused_kind
             }
         }
         __syncthreads();
-        for (int sidx = 0; sidx < nb; ++sidx) {
-            const int c = cell[sidx];
-            if (c < 0) continue;
-            const int lx = c & 255, ly = (c >> 8) & 255, lz = c >> 16;
-            const T *w = wv + sidx * 3 * W;
-            // the first of the warp's planes at or after lz
-            int iz = ((warp - lz) % nwarps + nwarps) % nwarps;
-            for (; iz < W; iz += nwarps) {
-                const T wz = w[2 * W + iz];
-                T *plane = tile + (lz + iz) * PS + ly * RS + lx + XO;
-                for (int pi = lane; pi < W * W; pi += 32) {
-                    const int iy = pi / W, ix = pi - iy * W;
-                    plane[iy * RS + ix] += w[ix] * (w[W + iy] * wz);
+        for (int s0 = 0; s0 < nb;) {
+            const int c = cell[s0];
+            int s1 = s0 + 1;
+            while (s1 < nb && cell[s1] == c) ++s1;
+            if (c >= 0 && upper < 2) {
+                const int lx = c & 255, ly = (c >> 8) & 255, lz = c >> 16;
+                const int iz = (warp + M * TS - lz) % M + M * upper;  // lz + iz = warp (mod M)
+                T *row = tile + (lz + iz) * PS + (ly + iy) * RS + lx;
+                T acc[W];
+#pragma unroll
+                for (int ix = 0; ix < W; ++ix) acc[ix] = row[ix];
+                for (int s = s0; s < s1; ++s) {
+                    const T *w = wv + s * 3 * W;
+                    const T b = w[W + iy] * w[2 * W + iz];
+#pragma unroll
+                    for (int ix = 0; ix < W; ++ix) acc[ix] += w[ix] * b;
                 }
+#pragma unroll
+                for (int ix = 0; ix < W; ++ix) row[ix] = acc[ix];
             }
+            __syncwarp();  // the next run's rows may be another lane's of this warp
+            s0 = s1;
         }
     }
     __syncthreads();
 
     const int Lx = p.L[0], Ly = p.L[1], Lz = p.L[2];
-    const int gxs = it.c0x - M + 1 - XO, gy0 = it.c0y - M + 1, gz0 = it.c0z - M + 1;
+    const int gx0 = it.c0x - M + 1, gy0 = it.c0y - M + 1, gz0 = it.c0z - M + 1;
     T *grid = (T *)p.gridA + blockIdx.y * p.st_grid;
-    for (int i = threadIdx.x; i < TE * TE * XE; i += blockDim.x) {
-        const int x = i % XE, r = i / XE;
-        const int iy = r % TE, iz = r / TE;
-        const T v = tile[iz * PS + iy * RS + x];
+    for (int i = threadIdx.x; i < TE * TE * TE; i += NT) {
+        const int x = i % TE, r = i / TE;
+        const int y = r % TE, z = r / TE;
+        const T v = tile[z * PS + y * RS + x];
         if (v == T(0)) continue;
-        const int gx = (gxs + x) & (Lx - 1);
-        const int gy = (gy0 + iy) & (Ly - 1), gz = (gz0 + iz) & (Lz - 1);
+        const int gx = (gx0 + x) & (Lx - 1);
+        const int gy = (gy0 + y) & (Ly - 1), gz = (gz0 + z) & (Lz - 1);
         atomicAdd(grid + ((int64_t)gz * Ly + gy) * Lx + gx, v);
     }
 }
@@ -978,7 +1021,7 @@ static cudaError_t spread_mt(const DevPlan &p, int fused_kind, const void *in, c
         if (e != cudaSuccess) return e;
     }
     if (p.n_spread > 0) {
-        const cudaError_t le = launch_k(k_spread_planes<T, M, TS>, dim3(p.n_spread, p.ks), 256, sm, s, p, fused_kind,
+        const cudaError_t le = launch_k(k_spread_planes<T, M, TS>, dim3(p.n_spread, p.ks), 32 * M, sm, s, p, fused_kind,
                                         (const T *)in);
         if (le != cudaSuccess) return le;
     }
@@ -988,7 +1031,7 @@ static cudaError_t spread_mt(const DevPlan &p, int fused_kind, const void *in, c
 template <typename T, int M, int TS> static cudaError_t gather_mt(const DevPlan &p, void *phi, cudaStream_t s) {
     typedef TileGeom<M, TS> G;
     const size_t GC = (size_t)p.gather_chunk;
-    const size_t sm = ((size_t)((G::SIZE + 3) & ~3) + GC * (3 * 2 * M + 4)) * sizeof(T) + 2 * GC * sizeof(int);
+    const size_t sm = ((size_t)((G::SIZE + 3) & ~3) + GC * (3 * 2 * M + 4) + 8 * GATHER_SPLIT) * sizeof(T) + 2 * GC * sizeof(int);
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_gather<T, M, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;

@@ -554,7 +554,8 @@ slp_status choose_parameters(slp_plan_s &p) {
     }
     // targets: larger tiles (fewer gather items, each tile load shared by more targets)
     p.TSg = 8;
-    while (p.TSg > 2 && std::pow((double)(p.TSg + 2 * p.m + 3), 3) * esz > 40 * 1024) p.TSg /= 2;
+    const int gather_kb = p.prec == 64 ? 80 : 40;  // FP64 m = 7: 4^3 cells, not the two or three targets of 2^3
+    while (p.TSg > 2 && std::pow((double)(p.TSg + 2 * p.m + 3), 3) * esz > gather_kb * 1024) p.TSg /= 2;
     p.TE = p.TS + 2 * p.m - 1;
     return SLP_OK;
 }
@@ -2655,9 +2656,13 @@ slp_status slp_plan(const slp_mesh *mesh, int quadrature, double tolerance, cons
         // spread chunk: about four items per SM, 128..1024 sources, a multiple of 32
         int64_t ch = (p->Q + 152 * 4 - 1) / (152 * 4);
         ch = std::max<int64_t>(128, std::min<int64_t>(1024, (ch + 31) / 32 * 32));
+        // wide windows: an item's tile costs about as much as one source to
+        // clear and flush, and the FP64 pipe of an SM is the limit, so even
+        // shares of it matter more: about eight items per SM
+        if (p->m > 5) ch = std::max<int64_t>(8, std::min<int64_t>(1024, round_up((p->Q + 152 * 8 - 1) / (152 * 8), 8)));
         tile_items(p->src_grid, skeys, p->Q, p->TS, (int)ch, p->spread_items);
     }
-    // gather items of GATHER_CHUNK targets, or of half that when the full
+    // gather items of GATHER_CHUNK targets, or (automatic) of half that when the full
     // size leaves fewer than four items per SM (small, latency-bound gathers)
     if (o.gather_item_targets != 0 && o.gather_item_targets != 32 && o.gather_item_targets != 64) {
         delete p;
@@ -2672,6 +2677,12 @@ slp_status slp_plan(const slp_mesh *mesh, int quadrature, double tolerance, cons
     if (o.gather_item_targets == 0 && p->gather_items.size() < 4 * 152) {
         p->gather_chunk = slp::GATHER_CHUNK / 2;
         tile_items(p->tgt_grid, tkeys, p->N, p->TSg, p->gather_chunk, p->gather_items);
+        // FP64, where a target costs an SM about 1800 cycles of its FP64 pipe:
+        // shorter items, down to 8, until there are four per SM (gather_chunk
+        // stays the bound).  602 targets at 64^3: 41 us in 23 items of up to 32,
+        // 16 us in 77 of up to 8
+        for (int most = p->gather_chunk / 2; p->prec == 64 && most >= 8 && p->gather_items.size() < 4 * 152; most /= 2)
+            tile_items(p->tgt_grid, tkeys, p->N, p->TSg, most, p->gather_items);
     }
     // largest items first: blocks are dispatched in index order, so this
     // schedules the long items early and the short ones fill the tail
