@@ -51,13 +51,14 @@ constexpr int NEAR_TARGETS = 16;
 
 // Fits of a E(a^2 r^2) = erf(a r) / r on [0, eps^2] for the RADIAL near field
 // computed per pair.  FP32: one polynomial of degree NEAR_DEG32 in
-// u = 2 r^2 / eps^2 - 1, kept where a eps <= NEAR_Z32 (largest error 4e-9 of
-// 1/r, below FP32 rounding; a eps is 3.0 at tolerance 1e-5).  FP64: intervals
+// u = 2 r^2 / eps^2 - 1, kept where a eps <= NEAR_Z32 (largest error 1e-8 of
+// 1/r, below FP32 rounding; a eps is 3.0 at tolerance 1e-5, 3.2 on automatic
+// grids).  FP64: intervals
 // of width NEAR_W64 or less in x = (a r)^2, at most NEAR_INT64 of them, a
 // polynomial of degree NEAR_DEG64 in the local coordinate in [-1/2, 1/2] on
 // each (largest error 2e-15 of 1/r; a eps is 4.6 at tolerance 1e-10).
-constexpr int NEAR_DEG32 = 13;
-constexpr double NEAR_Z32 = 3.1;
+constexpr int NEAR_DEG32 = 14;
+constexpr double NEAR_Z32 = 3.5;
 constexpr int NEAR_DEG64 = 9;
 constexpr int NEAR_INT64 = 64;
 constexpr double NEAR_W64 = 0.65;

@@ -288,7 +288,7 @@ void radial_params(slp_plan_s &p, double c) {
     p.sigma_g = s;
     for (int d = 0; d < 3; ++d) p.P[d] = p.D[d] + p.diam + 2.0 * c * s;
     p.R = p.diam + c * s;
-    const double tnf = std::min(0.5, p.tol * NFAC);
+    const double tnf = std::min(0.5, p.tol * p.split_share * NFAC);
     p.eps = s * std::sqrt(2.0) * erfc_inv(tnf);
 }
 
@@ -386,6 +386,76 @@ slp_status expsum_params(slp_plan_s &p) {
     return SLP_OK;
 }
 
+// The automatic grid: of the equal-spacing grids whose longest axis has 32, 64,
+// ..., 1024 cells, the one whose evaluation is estimated cheapest.
+//   far field: the launches, and per grid point of the five passes' active
+//     regions (the body's share of the period and the window) the rates the
+//     passes run at from 128^3 to 512^3;
+//   near field: the nodal operator at the HBM rate, its rows counted by a sample
+//     of vertices; charges at the points (no operator) at a tenth, as the plan
+//     does not know the input (all of it where the operator is switched off).
+// Sized by the number of points alone (2 sqrt(Q + N) cells), a level-5 sphere
+// of 143360 sources got 1024^3 cells and 4035 us an evaluation; here 128^3 and
+// 52 us (256^3: 93).  cube131 (618k sources) 1024^3, 3385 us; here 256^3, 404 us
+// (512^3: 502).  level-3 sphere 256^3, 69 us; here 64^3, 31 us.
+// A coarser grid carries more of the kernel's split error (the level-5 sphere:
+// 3.7e-7 at 1024^3, 9.8e-7 at 128^3), so automatic grids split with AUTO_SPLIT
+// of the tolerance: cube40 at 128^3 1.35e-6 -> 3.7e-7 (5.3e-7 at 1024^3 before),
+// sphere4 at 64^3 1.3e-6 -> 2.6e-7, plate100 1.4e-6 -> 4.0e-7, for 1 to 4 us.
+constexpr double AUTO_SPLIT = 0.3;
+
+bool cheapest_grid(const slp_plan_s &p, double c, int out[3]) {
+    const bool f64 = p.prec == 64;
+    const double dmax = std::max(p.D[0], std::max(p.D[1], p.D[2]));
+    // distances from up to 32 vertices to up to 32768
+    std::vector<double> dist;
+    const int64_t step_t = std::max<int64_t>(1, p.N / 32), step_v = std::max<int64_t>(1, p.N / 32768);
+    int64_t nt = 0, nv = (p.N + step_v - 1) / step_v;
+    for (int64_t i = step_t / 2; i < p.N; i += step_t, ++nt)
+        for (int64_t j = 0; j < p.N; j += step_v) {
+            double d2 = 0.0;
+            for (int d = 0; d < 3; ++d) d2 += (p.V[3 * i + d] - p.V[3 * j + d]) * (p.V[3 * i + d] - p.V[3 * j + d]);
+            dist.push_back(d2);
+        }
+    double best = 1e300;
+    for (int g = 32; g <= 1024; g <<= 1) {
+        int L[3], n[3];
+        for (int d = 0; d < 3; ++d) {
+            const double want = g * (p.D[d] + p.diam) / (dmax + p.diam);
+            L[d] = 16;
+            while (L[d] < 1024 && want >= L[d] * 1.4142135623730951) L[d] <<= 1;
+            n[d] = L[d] / 2;
+        }
+        if (!radial_feasible(p, n, c)) continue;
+        slp_plan_s q;
+        q.tol = p.tol;
+        q.split_share = p.split_share;
+        q.diam = p.diam;
+        for (int d = 0; d < 3; ++d) {
+            q.D[d] = p.D[d];
+            q.n[d] = n[d];
+        }
+        radial_params(q, c);
+        double act[3];  // grid points the body and its window span
+        for (int d = 0; d < 3; ++d) act[d] = std::min<double>(L[d], p.D[d] / q.P[d] * L[d] + 2 * p.m);
+        const double kx = 0.25 * L[0];
+        const double fx = act[1] * act[2] * L[0], fy = act[2] * kx * L[1], fz = n[1] * kx * L[2];
+        const double far = f64 ? 120.0 + 4e-5 * fx + 1.2e-4 * fy + 9e-5 * fz : 32.0 + 6.6e-6 * fx + 7.4e-6 * fy + 5.4e-6 * fz;
+        int64_t in = 0;
+        for (double d2 : dist) in += d2 < q.eps * q.eps;
+        const double share = (double)in / ((double)nt * nv);
+        const double op = share * (double)p.N * (double)p.N * (f64 ? 32.0 : 16.0);
+        const double pairs = share * (double)p.N * (double)p.Q * (f64 ? 5.7e-5 : 1.25e-6);
+        const bool fly = p.opts.near_mode == SLP_NEAR_ON_THE_FLY || op > 20e9;
+        const double t = far + (fly ? pairs : op / 6.5e6 + 0.1 * pairs);
+        if (t < best) {
+            best = t;
+            for (int d = 0; d < 3; ++d) out[d] = L[d];
+        }
+    }
+    return best < 1e300;
+}
+
 slp_status choose_parameters(slp_plan_s &p) {
     // bounding box and enclosing-ball diameter of targets (sources are convex
     // combinations of targets, so they lie inside both)
@@ -426,8 +496,19 @@ slp_status choose_parameters(slp_plan_s &p) {
         if (L[d] > 0 && (!is_pow2(L[d]) || L[d] < 8 || L[d] > 1024))
             return fail(SLP_ERR_INVALID_ARG, "grid[%d] = %d must be a power of two in [8, 1024]", d, L[d]);
     }
-    const double tk = std::min(0.1, p.tol * KFAC);
-    const double c = std::sqrt(2.0 * std::log(1.0 / tk));
+    int mode = p.opts.kernel_mode;
+    // an automatic grid for the radial kernel (point plans): sized by cost, with
+    // a smaller share of the tolerance for the kernel split (AUTO_SPLIT)
+    const bool by_cost = L[0] < 0 && L[1] < 0 && L[2] < 0 && !p.opts.integration &&
+                         (mode == SLP_KERNEL_AUTO || mode == SLP_KERNEL_RADIAL);
+    p.split_share = by_cost ? AUTO_SPLIT : 1.0;
+    double tk = std::min(0.1, p.tol * p.split_share * KFAC);
+    double c = std::sqrt(2.0 * std::log(1.0 / tk));
+    if (by_cost && !cheapest_grid(p, c, L)) {
+        p.split_share = 1.0;
+        tk = std::min(0.1, p.tol * KFAC);
+        c = std::sqrt(2.0 * std::log(1.0 / tk));
+    }
     p.c_band = c;
     if (L[0] < 0 || L[1] < 0 || L[2] < 0) {
         // automatic: equal spacing at about (Q + N)^(1/2) cells across the body
@@ -444,7 +525,6 @@ slp_status choose_parameters(slp_plan_s &p) {
     }
     int nreq[3] = {L[0] / 2, L[1] / 2, L[2] / 2};
 
-    int mode = p.opts.kernel_mode;
     if (mode == SLP_KERNEL_AUTO) {
         if (radial_feasible(p, nreq, c))
             mode = SLP_KERNEL_RADIAL;
@@ -2258,6 +2338,24 @@ enum {
     SLOT_NEAR_ZERO, SLOT_NEAR, SLOT_NEAR_REDUCE, SLOT_GATHER, SLOT_FFT_XY, SLOT_IFFT_YX, SLOT_FFT_YZY
 };
 
+// The near-field product in the main stream, before the spread, instead of
+// beside the far field?  Beside it, it fills the latency-bound passes' idle
+// SMs; but its short blocks also keep the larger blocks of the other stream
+// waiting for room, and where both are bound by HBM there is nothing to fill.
+// So first in line where the operator is large (the far field is a small part
+// of the evaluation; with several states, which share one pass over it, the
+// pass is longer still) or the grids exceed L2.  Measured, beside -> first:
+// cube200 at 512^3 (2.4 GB) 1002 -> 844 us, plate400 (5.1 GB) 884 -> 852,
+// cube400 at 1024^3 (9 GB) 5660 -> 5232, cube131 at 512^3 (0.5 GB) 506 -> 487;
+// cube131 at 256^3 (1.9 GB) 404 -> 410, sphere6 at 256^3 (0.3 GB) 147 -> 163,
+// sphere5 at 128^3 52 -> 64.  Eight states: torus400 (1.1 GB) 811 -> 790 us,
+// cube74 at 256^3 (0.2 GB) 693 -> 694, plate90 104 -> 129.
+bool near_product_first(const slp_plan_s &p, int states) {
+    const double es = p.prec == 64 ? 8 : 4;
+    const double op = 4 * es * (double)p.nm_nnz, grids = 2 * es * 2.0 * p.row_pairs.size() * p.L[0];
+    return op >= (states > 1 ? 0.8e9 : 2.1e9) || grids >= 96e6;
+}
+
 // Enqueue the evaluation up to stage `last`.
 //   serial (prof != NULL, or ex == NULL): charges, spread, 5 FFT passes, near
 //     field into phi_part, gather (far field + phi_part) on s; with prof,
@@ -2265,7 +2363,8 @@ enum {
 //   concurrent (ex != NULL, no prof): the near field runs on ex->aux (lowest
 //     priority) while the spread, FFT passes and gather run on ex->main
 //     (highest priority, so the latency-bound FFT blocks are dispatched ahead
-//     of pending near-field blocks); both fork from s, the gather waits for
+//     of pending near-field blocks), or ahead of them on ex->main
+//     (near_product_first); both fork from s, the gather waits for
 //     the near field, and s waits for the gather.
 slp_status run_pipeline(slp_plan_s &p, const slp::DevPlan &d, int kind, const void *d_in, void *d_phi,
                         cudaStream_t s, int last, SlpProfile *prof, SlpExec *ex) {
@@ -2326,15 +2425,17 @@ slp_status run_pipeline(slp_plan_s &p, const slp::DevPlan &d, int kind, const vo
         TRY(timed(SLOT_CHARGES, s, [&] { return slp::launch_charges(d, kind, d_in, s); }, "charges"));
     }
     if (last <= SLP_STAGE_CHARGES) return SLP_OK;
-    cudaStream_t caller = s;
+    cudaStream_t caller = s, near_stream = s;
+    const bool near_first = concurrent && use_matrix && near_product_first(p, 1);
     if (concurrent) {
         TRY(cuda_status(cudaEventRecord(ex->fork, s), "fork"));
-        TRY(cuda_status(cudaStreamWaitEvent(ex->aux, ex->fork, 0), "fork wait"));
+        if (!near_first) TRY(cuda_status(cudaStreamWaitEvent(ex->aux, ex->fork, 0), "fork wait"));
         TRY(cuda_status(cudaStreamWaitEvent(ex->main, ex->fork, 0), "fork wait"));
         s = ex->main;
-        TRY(near_branch(ex->aux));
-        if (tl) TRY(cuda_status(cudaEventRecord(tl[3], ex->aux), "timeline"));
-        TRY(cuda_status(cudaEventRecord(ex->join, ex->aux), "join"));
+        near_stream = near_first ? s : ex->aux;
+        TRY(near_branch(near_stream));
+        if (tl) TRY(cuda_status(cudaEventRecord(tl[3], near_stream), "timeline"));
+        if (!near_first) TRY(cuda_status(cudaEventRecord(ex->join, ex->aux), "join"));
     }
     if (tri || det)
         TRY(timed(SLOT_SPREAD, s, [&] {
@@ -2372,7 +2473,7 @@ slp_status run_pipeline(slp_plan_s &p, const slp::DevPlan &d, int kind, const vo
     if (last <= SLP_STAGE_IFFT_X) return SLP_OK;
     if (tl) TRY(cuda_status(cudaEventRecord(tl[2], s), "timeline"));
     if (concurrent) {
-        TRY(cuda_status(cudaStreamWaitEvent(s, ex->join, 0), "join wait"));
+        if (!near_first) TRY(cuda_status(cudaStreamWaitEvent(s, ex->join, 0), "join wait"));
     } else if (last >= SLP_STAGE_NEAR) {
         TRY(near_branch(s));
     } else {
@@ -2422,11 +2523,15 @@ slp_status run_states(slp_plan_s &p, const slp::DevPlan &d, int kind, const void
         const int K = std::min(slp::NEAR_STATES, S - c0);
         slp::StatePtrs sp = {};
         for (int k = 0; k < K; ++k) sp.in[k] = ins[c0 + k];
-        TRY(cuda_status(cudaEventRecord(ex->fork, m), "fork"));
-        TRY(cuda_status(cudaStreamWaitEvent(ex->aux, ex->fork, 0), "fork wait"));
-        TRY(cuda_status(slp::launch_nodal_prep_states(d, sp, K, ex->aux), "nodal prep"));
-        TRY(cuda_status(slp::launch_near_matrix_states(d, K, ex->aux), "near-field matrix"));
-        TRY(cuda_status(cudaEventRecord(ex->join, ex->aux), "join"));
+        const bool first = near_product_first(p, K);
+        cudaStream_t ns = first ? m : ex->aux;
+        if (!first) {
+            TRY(cuda_status(cudaEventRecord(ex->fork, m), "fork"));
+            TRY(cuda_status(cudaStreamWaitEvent(ns, ex->fork, 0), "fork wait"));
+        }
+        TRY(cuda_status(slp::launch_nodal_prep_states(d, sp, K, ns), "nodal prep"));
+        TRY(cuda_status(slp::launch_near_matrix_states(d, K, ns), "near-field matrix"));
+        if (!first) TRY(cuda_status(cudaEventRecord(ex->join, ns), "join"));
         // the far field in batches of kf states: one launch per kernel per batch
         // (grid.y = state), state f at scratch copy f and near-field part f0 + f
         int nbatch = 0;
@@ -2455,7 +2560,7 @@ slp_status run_states(slp_plan_s &p, const slp::DevPlan &d, int kind, const void
                 TRY(cuda_status(slp::launch_fft_inverse_y(dk, m), "ifft y"));
                 TRY(cuda_status(slp::launch_fft_inverse_x(dk, m), "ifft x"));
             }
-            if (f0 == 0) TRY(cuda_status(cudaStreamWaitEvent(m, ex->join, 0), "join wait"));
+            if (f0 == 0 && !first) TRY(cuda_status(cudaStreamWaitEvent(m, ex->join, 0), "join wait"));
             TRY(cuda_status(slp::launch_gather(dk, outs[c0 + f0], m), "gather"));
         }
         if (launches) *launches += 2 + nbatch * (p.launches_per_eval - 2);

@@ -93,6 +93,7 @@ struct slp_plan_s {
     int aslot = 0;
     int *d_blk_first = nullptr;
     int launches_per_eval = 0;
+    double split_share = 1.0;  // share of the tolerance the kernel's split may use
     int64_t near_pairs_within = -1;
     int64_t nm_nnz = 0;
     SlpExec exec;  // for evaluations on the plan's own scratch
