@@ -282,12 +282,29 @@ __device__ __forceinline__ double rsqrt_refined(double x) {
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// -a E(a^2 r^2) from the table [k][ni] at x = r^2 iw, iw intervals per unit of
+// r^2; false outside the table (r >= eps).  The interval is read off the low
+// word of x - 1/2 + 1.5 2^52.
+__device__ __forceinline__ bool table_value(const double *tab, int ni, double iw, double r2, double &e) {
+    constexpr double MAGIC = 6755399441055744.0;  // 1.5 2^52
+    const double t = fma(r2, iw, -0.5);            // interval i holds [i - 1/2, i + 1/2)
+    const double tm = t + MAGIC;
+    const int i = __double2loint(tm);
+    const double u = t - (tm - MAGIC);
+    const bool in = (unsigned)i < (unsigned)ni;
+    const double *c = tab + (in ? i : 0);
+    e = c[NEAR_DEG64 * ni];
+#pragma unroll
+    for (int k = NEAR_DEG64 - 1; k >= 0; --k) e = fma(e, u, c[k * ni]);
+    return in;
+}
+
 // FP64: this GPU's FP64 pipe (2 lanes per SM) bounds it, so everything that is
 // not the pair's own arithmetic is kept off it: about 27 FP64 operations per
 // pair (3 subtractions, 5 for r^2, 5 for the reciprocal square root, 3 for the
 // interval and its local coordinate, 9 of the degree-9 polynomial, 2 for the
 // sum) where rsqrt, erfc and the conversions of the cell differences took over
-// 100.  The interval is read off the low word of x / width + 1.5 2^52.
+// 100.
 // Level-4 sphere at 128^3 (63M pairs listed): 129 -> 3.6 ms, level-3 20.4 ->
 // 0.35 ms, both with the work list's full 16-target blocks.
 __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial64(DevPlan p) {
@@ -315,7 +332,6 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial64(DevPlan p) {
     warp_box((float)tz, lo[2], hi[2]);
     const double ry = p.near_ry, rz = p.near_rz, iw = p.near_iw;
     const float reach2 = p.near_e2f * 1.001f, ryf = p.near_ryf, rzf = p.near_rzf;
-    constexpr double MAGIC = 6755399441055744.0;  // 1.5 2^52
     const double4 *src = (const double4 *)p.src_grid;
     const double *qb = (const double *)p.qbuf;
     double acc = 0.0;
@@ -338,16 +354,8 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial64(DevPlan p) {
                 const double4 v = st[warp][j];
                 const double dx = tx - v.x, dy = (ty - v.y) * ry, dz = (tz - v.z) * rz;
                 const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-                // interval i holds x / width in [i - 1/2, i + 1/2): a shift of 1/2 makes it [i, i + 1)
-                const double t = fma(r2, iw, -0.5);
-                const double tm = t + MAGIC;
-                const int i = __double2loint(tm);
-                const double u = t - (tm - MAGIC);  // in [-1/2, 1/2]
-                const bool in = (unsigned)i < (unsigned)ni;
-                const double *ct = tab + (in ? i : 0);
-                double e = ct[NEAR_DEG64 * ni];
-#pragma unroll
-                for (int k = NEAR_DEG64 - 1; k >= 0; --k) e = fma(e, u, ct[k * ni]);
+                double e;
+                const bool in = table_value(tab, ni, iw, r2, e);
                 const double w = rsqrt_refined(r2) + e;
                 acc = fma(in ? v.w : 0.0, w, acc);
             }
@@ -425,7 +433,13 @@ cudaError_t launch_near_reduce(const DevPlan &p, const int *blk_first, int nblk,
 // order.  Each evaluation is then a sparse product streamed from HBM.
 namespace slp {
 
-__device__ __forceinline__ double nm_kernel(const NMBuild &b, double dx, double dy, double dz, double r2) {
+__device__ __forceinline__ double nm_kernel(const NMBuild &b, const double *tab, double dx, double dy, double dz,
+                                            double r2) {
+    if (b.ni > 0) {
+        double e;
+        if (!table_value(tab, b.ni, b.iw, r2, e)) return 0.0;
+        return fma(rsqrt_refined(r2 * b.iw), b.sqrt_iw, e) * 0.079577471545947667884;  // in range whatever the units
+    }
     const double ri = rsqrt(r2);
     if (b.kernel_mode == 2) {
         const double kn = sep_factor(b.sep_h[0], b.sep_nh[0], dx / b.P[0]) *
@@ -437,12 +451,22 @@ __device__ __forceinline__ double nm_kernel(const NMBuild &b, double dx, double 
     return erfc(r2 * ri * b.inv_s_sqrt2) * ri * 0.079577471545947667884;
 }
 
-// pass 0: count non-zeros per row (and near pairs); pass 1: fill.
+// pass 0: count the entries per row (vertices with a quadrature point of an
+// adjacent triangle within eps) and the near pairs; pass 1: fill.  The kernel is
+// evaluated in FP64, three times per pair (once per vertex of the triangle), so
+// the FP64 pipe bounds the fill: the table's 25 operations where erfc and rsqrt
+// took over 100, and no evaluation in the count.  Plan of plate400 (319M
+// entries) 2.56 -> 0.80 s, of sphere5 at 128^3 (6M) 0.23 -> 0.085 s.
 template <typename T4>
 __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, int64_t *__restrict__ counts,
                                                   int64_t *__restrict__ pairs, const int64_t *__restrict__ rowptr,
                                                   T4 *__restrict__ val) {
+    __shared__ double tab[(NEAR_DEG64 + 1) * NEAR_INT64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (pass == 1) {
+        for (int i = threadIdx.x; i < (NEAR_DEG64 + 1) * b.ni; i += blockDim.x) tab[i] = b.tab[i];
+        __syncthreads();
+    }
     const int64_t t = (int64_t)blockIdx.x * 8 + warp;
     if (t >= b.N) return;
     const double4 xt = b.tgt[t];
@@ -455,6 +479,7 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, int64_t *
             const int u = u0 + lane;
             double wx = 0.0, wy = 0.0, wz = 0.0;
             int v = -1;
+            bool nz = false;
             if (u < rg.y) {
                 v = b.tgt_perm[u];
                 for (int e = b.vt_ptr[v]; e < b.vt_ptr[v + 1]; ++e) {
@@ -467,7 +492,8 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, int64_t *
                         const double dx = xt.x - y.x, dy = xt.y - y.y, dz = xt.z - y.z;
                         const double r2 = dx * dx + dy * dy + dz * dz;
                         if (r2 < b.eps2 && r2 > 0.0) {
-                            acc += y.w * nm_kernel(b, dx, dy, dz, r2) * b.lam[3 * s + a];
+                            nz = true;
+                            if (pass == 1) acc += y.w * nm_kernel(b, tab, dx, dy, dz, r2) * b.lam[3 * s + a];
                             if (a == 0) ++npairs;
                         }
                     }
@@ -476,7 +502,6 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, int64_t *
                     wz += acc * n.z;
                 }
             }
-            const bool nz = (v >= 0) && (wx != 0.0 || wy != 0.0 || wz != 0.0);
             const unsigned bal = __ballot_sync(0xffffffffu, nz);
             if (pass == 1 && nz) {
                 const int pos = __popc(bal & ((1u << lane) - 1u));

@@ -315,6 +315,11 @@ struct NMBuild {
     double P[3];
     const double *es_w, *es_g;  // EXPSUM terms, physical units
     int es_n;
+    // RADIAL: -a E as a table (slp_internal.h), physical lengths, ni intervals
+    // over [0, eps2), iw of them per unit of r^2 (ni = 0: erfc)
+    const double *tab;
+    int ni;
+    double iw, sqrt_iw;
 };
 cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, int64_t *counts, int64_t *pairs,
                             const int64_t *rowptr, void *val, cudaStream_t s);

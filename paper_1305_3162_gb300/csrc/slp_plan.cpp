@@ -1047,22 +1047,12 @@ double erf_ratio(double x) {
     return z < 1e-8 ? 2.0 / std::sqrt(PI) : std::erf(z) / z;
 }
 
-// The fits of -a E(a^2 r^2) (slp_internal.h), lengths in cells of x: FP32
-// coefficients into c32, the FP64 table [k][interval] into tab.  False where
-// the RADIAL kernel's a eps lies outside their range.
-bool near_fits(const slp_plan_s &p, float *c32, std::vector<double> &tab, int &ni) {
-    ni = 0;
-    if (p.kernel_mode != SLP_KERNEL_RADIAL || !(p.sigma_g > 0) || !std::isfinite(p.eps)) return false;
-    const double h = p.P[0] / p.L[0], a = h / (p.sigma_g * std::sqrt(2.0)), z = a * (p.eps / h), x1 = z * z;
-    if (p.prec == 32) {
-        if (z > slp::NEAR_Z32) return false;
-        const std::vector<double> c = fit_powers([&](double u) { return -a * erf_ratio(0.5 * (u + 1.0) * x1); }, slp::NEAR_DEG32);
-        for (int k = 0; k <= slp::NEAR_DEG32; ++k) c32[k] = (float)c[k];
-        return true;
-    }
-    const int n = std::max(1, (int)std::ceil(x1 / slp::NEAR_W64));
-    if (n > slp::NEAR_INT64) return false;
-    ni = n;
+// The table [k][interval] of -a E(a^2 r^2) over [0, eps^2) (slp_internal.h) in
+// the units of a and eps; its number of intervals, 0 where they would be too many.
+int near_table(double a, double eps, std::vector<double> &tab) {
+    const double x1 = a * a * eps * eps;
+    const int n = std::max(1, (int)std::ceil(std::min(x1 / slp::NEAR_W64, 1e6)));
+    if (n > slp::NEAR_INT64) return 0;
     const double w = x1 / n;
     tab.assign((size_t)(slp::NEAR_DEG64 + 1) * n, 0.0);
     for (int i = 0; i < n; ++i) {
@@ -1070,6 +1060,24 @@ bool near_fits(const slp_plan_s &p, float *c32, std::vector<double> &tab, int &n
         double s = 1.0;  // the kernel's local coordinate is u / 2
         for (int k = 0; k <= slp::NEAR_DEG64; ++k, s *= 2.0) tab[(size_t)k * n + i] = c[k] * s;
     }
+    return n;
+}
+
+bool radial_near(const slp_plan_s &p) {
+    return p.kernel_mode == SLP_KERNEL_RADIAL && p.sigma_g > 0 && std::isfinite(p.eps);
+}
+
+// The fits for the near field per pair, lengths in cells of x: FP32
+// coefficients into c32, or the FP64 table into tab.  False where the RADIAL
+// kernel's a eps lies outside their range.
+bool near_fits(const slp_plan_s &p, float *c32, std::vector<double> &tab, int &ni) {
+    ni = 0;
+    if (!radial_near(p)) return false;
+    const double h = p.P[0] / p.L[0], a = h / (p.sigma_g * std::sqrt(2.0)), z = a * (p.eps / h);
+    if (p.prec == 64) return (ni = near_table(a, p.eps / h, tab)) > 0;
+    if (z > slp::NEAR_Z32) return false;
+    const std::vector<double> c = fit_powers([&](double u) { return -a * erf_ratio(0.5 * (u + 1.0) * z * z); }, slp::NEAR_DEG32);
+    for (int k = 0; k <= slp::NEAR_DEG32; ++k) c32[k] = (float)c[k];
     return true;
 }
 
@@ -1630,6 +1638,18 @@ void near_candidates(const slp_plan_s &p, const std::vector<uint64_t> &tkeys, do
     blk_r0[nblk] = (int)ranges.size();
 }
 
+// The RADIAL kernel's table for the operator's assembly, in physical lengths.
+slp_status near_build_table(const slp_plan_s &p, slp::NMBuild &nb, TmpBuf &buf) {
+    std::vector<double> tab;
+    nb.ni = radial_near(p) ? near_table(nb.inv_s_sqrt2, p.eps, tab) : 0;
+    if (nb.ni == 0) return SLP_OK;
+    TRY(tmp_upload(buf, tab.data(), tab.size()));
+    nb.tab = (const double *)buf.p;
+    nb.iw = nb.ni / nb.eps2;
+    nb.sqrt_iw = std::sqrt(nb.iw);
+    return SLP_OK;
+}
+
 slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) {
     const int64_t N = p.N, M = p.M, q = p.q;
     double r_adj = 0.0;
@@ -1686,6 +1706,8 @@ slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) 
     nb.eps2 = std::isfinite(p.eps) ? p.eps * p.eps : 1e300;
     nb.inv_s_sqrt2 = p.sigma_g > 0 ? 1.0 / (p.sigma_g * std::sqrt(2.0)) : 0.0;
     nb.kernel_mode = p.kernel_mode;
+    TmpBuf b_tab;
+    TRY(near_build_table(p, nb, b_tab));
     if (p.kernel_mode == SLP_KERNEL_SEPARABLE) {
         for (int a = 0; a < 3; ++a) {
             TRY(tmp_upload(b_h[a], p.sep_h[a].data(), p.sep_h[a].size()));
@@ -2281,6 +2303,8 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         nb.eps2 = std::isfinite(p.eps) ? p.eps * p.eps : 1e300;
         nb.inv_s_sqrt2 = p.sigma_g > 0 ? 1.0 / (p.sigma_g * std::sqrt(2.0)) : 0.0;
         nb.kernel_mode = p.kernel_mode;
+        TmpBuf b_tab;
+        TRY(near_build_table(p, nb, b_tab));
         TmpBuf b_esw, b_esg;
         if (p.kernel_mode == SLP_KERNEL_SEPARABLE) {
             for (int a = 0; a < 3; ++a) {
