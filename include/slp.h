@@ -133,7 +133,7 @@ typedef struct {
     int fuse_plane_passes; /* x and y FFT passes fused per z plane (a cluster of four CTAs per
                               plane, the plane spectrum in distributed shared memory): 0 off, 1 on
                               where the plane fits, -1 automatic (on when there are at least two
-                              active planes per SM) */
+                              active planes per SM, and on grids of up to 64 cells along x and y) */
     int fuse_column_passes; /* the y pass, the z pass with the kernel multiply and the inverse y pass
                                fused, one cluster of four CTAs per stored x frequency holding that
                                slab of the spectrum in distributed shared memory (needs equal y and

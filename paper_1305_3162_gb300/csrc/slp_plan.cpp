@@ -1374,7 +1374,12 @@ template <typename T> slp_status upload_all(slp_plan_s &p) {
         const size_t sm = slp::fused_plane_smem(d, PB);
         const bool fits = maxp > 0 && sm <= std::min<size_t>((size_t)optin, 200 * 1024);
         const int want = p.opts.fuse_plane_passes;
-        d.fuse_pb = (fits && (want == 1 || (want < 0 && p.nz_act >= 2 * nsm))) ? PB : 0;
+        // automatic: with two active planes per SM, or on grids of up to 64 x 64
+        // cells a plane, whose passes are all launch and latency: sphere2 at 32^3
+        // 29.5 -> 26.1 us, sphere3 at 64^3 29.5 -> 27.0, cube8 FP64 at 32^3 88 ->
+        // 76, sphere3 FP64 at 64^3 137 -> 136 (at 128^3: sphere4 40.2 -> 40.7)
+        const bool small = std::max(p.L[0], p.L[1]) <= 64;
+        d.fuse_pb = (fits && (want == 1 || (want < 0 && (small || p.nz_act >= 2 * nsm)))) ? PB : 0;
         // fused column passes: equal y and z lengths the column engine
         // compiles (32..256), at most 512 threads a CTA, within shared memory
         d.yzy_g = d.yzy_zc = d.yzy_zp = 0;
