@@ -221,8 +221,9 @@ def _algorithmic(info, stage, w, pairs_within):
         # nodal m (user order) read, permutation read, sorted 4-vectors written
         "nodal_prep": ("hbm", 3 * es * N + 4 * N + 4 * es * N),
         "near_zero": ("hbm", es * N),
-        # operator entries, row pointers, sorted m read; near-field parts written
-        "near": (("hbm", info["near_matrix_nnz"] * 4 * es + 8 * (N + 1) + 4 * es * N + es * N)
+        # operator (three weights per (target, vertex) pair, a column per four), group
+        # pointers, sorted m read; near-field parts written
+        "near": (("hbm", info["near_matrix_nnz"] * (3 * es + 1) + 2 * N + 4 * es * N + es * N)
                  if info["near_mode"] == 2 else ("alu", NEAR_FLOPS_PER_PAIR * pairs_within)),
         "near_reduce": ("hbm", es * N + es * 32 * info["n_near_items"]),
     }
@@ -233,13 +234,14 @@ def _eval_bytes(info):
     """Algorithmic bytes of one whole evaluation: the stage-separated model
     16Q + 16N + 25G bytes (FP32; each stage reads its input and writes its
     output once, single-pass FFTs; twice that in FP64) plus, for the
-    precomputed near-field operator, its 16-byte entries and row pointers."""
+    precomputed near-field operator, three weights per (target, vertex) pair, a
+    column per four of them and the group pointers."""
     es = 4 if info["precision"] == 32 else 8
     L = info["grid"]
     G = L[0] * L[1] * L[2]
     N, Q = info["n_targets"], info["n_sources"]
     model = (es // 4) * (16 * Q + 16 * N + 25 * G)
-    near = 4 * es * info["near_matrix_nnz"] + 8 * (N + 1) if info["near_mode"] == 2 else 0
+    near = (3 * es + 1) * info["near_matrix_nnz"] + 2 * N if info["near_mode"] == 2 else 0
     return model, near
 
 

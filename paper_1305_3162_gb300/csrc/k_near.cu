@@ -428,9 +428,9 @@ cudaError_t launch_near_reduce(const DevPlan &p, const int *blk_first, int nblk,
 //   W_iv = sum_{k near x_i, v a vertex of tri(k)} w_k (N - N_s)(x_i - y_k) lambda_{s(k), a(v)} n_{j(k)}.
 // The paper precomputes the near-field integrals in the set-up phase and
 // applies them as a sparse matrix (Sec. 3.4); here W is assembled once per
-// plan on the GPU in FP64 (two passes: count, fill) and stored as one
-// 4-vector (W_x, W_y, W_z, vertex id) per non-zero, rows in sorted target
-// order.  Each evaluation is then a sparse product streamed from HBM.
+// plan on the GPU in FP64 (two passes: count, fill) and stored by groups of
+// four rows in sorted target order.  Each evaluation is then a sparse product
+// streamed from HBM.
 namespace slp {
 
 __device__ __forceinline__ double nm_kernel(const NMBuild &b, const double *tab, double dx, double dy, double dz,
@@ -451,186 +451,245 @@ __device__ __forceinline__ double nm_kernel(const NMBuild &b, const double *tab,
     return erfc(r2 * ri * b.inv_s_sqrt2) * ri * 0.079577471545947667884;
 }
 
-// pass 0: count the entries per row (vertices with a quadrature point of an
-// adjacent triangle within eps) and the near pairs; pass 1: fill.  The kernel is
-// evaluated in FP64, three times per pair (once per vertex of the triangle), so
-// the FP64 pipe bounds the fill: the table's 25 operations where erfc and rsqrt
-// took over 100, and no evaluation in the count.  Plan of plate400 (319M
-// entries) 2.56 -> 0.80 s, of sphere5 at 128^3 (6M) 0.23 -> 0.085 s.
+// One warp per group of NM_ROWS consecutive sorted targets, a candidate vertex
+// per lane.  An entry is a vertex with a quadrature point of an adjacent
+// triangle within eps of some target of the group; its weights are zero for the
+// others.  pass 0: count the group's entries, its (target, vertex) pairs with a
+// point inside and the near pairs; pass 1: fill.  The kernel is evaluated in
+// FP64, three times per pair (once per vertex of the triangle), so the FP64 pipe
+// bounds the fill: the table's 25 operations where erfc and rsqrt took over 100,
+// no evaluation in the count, and vertices out of every target's reach passed
+// over.  Plan of plate400 (319M pairs) 2.56 -> 0.83 s, of sphere5 at 128^3 (6M)
+// 0.23 -> 0.09 s.
 template <typename T4>
-__global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, int64_t *__restrict__ counts,
-                                                  int64_t *__restrict__ pairs, const int64_t *__restrict__ rowptr,
-                                                  T4 *__restrict__ val) {
+__global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, NMCount *__restrict__ counts,
+                                                  const int64_t *__restrict__ gptr, int *__restrict__ col,
+                                                  T4 *__restrict__ val, int64_t stride) {
+    constexpr int R = NM_ROWS;
     __shared__ double tab[(NEAR_DEG64 + 1) * NEAR_INT64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (pass == 1) {
         for (int i = threadIdx.x; i < (NEAR_DEG64 + 1) * b.ni; i += blockDim.x) tab[i] = b.tab[i];
         __syncthreads();
     }
-    const int64_t t = (int64_t)blockIdx.x * 8 + warp;
-    if (t >= b.N) return;
-    const double4 xt = b.tgt[t];
-    const int blk = b.tgt_block[t];
-    int64_t out = pass == 1 ? rowptr[t] : 0;
-    int64_t cnt = 0, npairs = 0;
-    for (int r = b.blk_r0[blk]; r < b.blk_r0[blk + 1]; ++r) {
-        const int2 rg = b.ranges[r];
+    const int64_t g = (int64_t)blockIdx.x * 8 + warp;
+    if (R * g >= b.N) return;
+    const int nr = (int)min((int64_t)R, b.N - R * g);
+    double4 x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = b.tgt[R * g + min(r, nr - 1)];
+    const int blk = b.grp_block[g];
+    int64_t out = pass == 1 ? gptr[g] : 0;
+    int64_t cnt = 0, npairs = 0, nnz = 0;
+    for (int rr = b.blk_r0[blk]; rr < b.blk_r0[blk + 1]; ++rr) {
+        const int2 rg = b.ranges[rr];
         for (int u0 = rg.x; u0 < rg.y; u0 += 32) {
             const int u = u0 + lane;
-            double wx = 0.0, wy = 0.0, wz = 0.0;
-            int v = -1;
-            bool nz = false;
+            double wx[R], wy[R], wz[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) wx[r] = wy[r] = wz[r] = 0.0;
+            unsigned reach = 0, hit = 0;  // targets: worth a look; with a point inside
             if (u < rg.y) {
-                v = b.tgt_perm[u];
+                const double4 xv = b.vpos[u];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double dx = x[r].x - xv.x, dy = x[r].y - xv.y, dz = x[r].z - xv.z;
+                    if (r < nr && dx * dx + dy * dy + dz * dz <= b.reach2) reach |= 1u << r;
+                }
+            }
+            if (reach) {
+                const int v = b.tgt_perm[u];
                 for (int e = b.vt_ptr[v]; e < b.vt_ptr[v + 1]; ++e) {
                     const int ent = b.vt_ent[e];
                     const int j = ent >> 2, a = ent & 3;
                     const double4 n = b.nrm[j];
-                    double acc = 0.0;
+                    double acc[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) acc[r] = 0.0;
                     for (int s = 0; s < b.q; ++s) {
                         const double4 y = b.src[(int64_t)j * b.q + s];
-                        const double dx = xt.x - y.x, dy = xt.y - y.y, dz = xt.z - y.z;
-                        const double r2 = dx * dx + dy * dy + dz * dz;
-                        if (r2 < b.eps2 && r2 > 0.0) {
-                            nz = true;
-                            if (pass == 1) acc += y.w * nm_kernel(b, tab, dx, dy, dz, r2) * b.lam[3 * s + a];
-                            if (a == 0) ++npairs;
+                        const double yw = pass == 1 ? y.w * b.lam[3 * s + a] : 0.0;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const double dx = x[r].x - y.x, dy = x[r].y - y.y, dz = x[r].z - y.z;
+                            const double r2 = dx * dx + dy * dy + dz * dz;
+                            if ((reach >> r & 1) && r2 < b.eps2 && r2 > 0.0) {
+                                hit |= 1u << r;
+                                if (pass == 1) acc[r] += yw * nm_kernel(b, tab, dx, dy, dz, r2);
+                                if (a == 0) ++npairs;
+                            }
                         }
                     }
-                    wx += acc * n.x;
-                    wy += acc * n.y;
-                    wz += acc * n.z;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        wx[r] += acc[r] * n.x;
+                        wy[r] += acc[r] * n.y;
+                        wz[r] += acc[r] * n.z;
+                    }
                 }
             }
-            const unsigned bal = __ballot_sync(0xffffffffu, nz);
-            if (pass == 1 && nz) {
-                const int pos = __popc(bal & ((1u << lane) - 1u));
+            const unsigned bal = __ballot_sync(0xffffffffu, hit != 0);
+            if (pass == 1 && hit) {
+                const int64_t at = out + cnt + __popc(bal & ((1u << lane) - 1u));
                 T4 o;
-                o.x = wx;
-                o.y = wy;
-                o.z = wz;
-                o.w = pack_id(o.w, u);  // vertex (sorted target position) in the fourth component
-                val[out + cnt + pos] = o;
+                col[at] = u;  // vertex: sorted target position
+                o.x = wx[0], o.y = wx[1], o.z = wx[2], o.w = wx[3];
+                val[at] = o;
+                o.x = wy[0], o.y = wy[1], o.z = wy[2], o.w = wy[3];
+                val[at + stride] = o;
+                o.x = wz[0], o.y = wz[1], o.z = wz[2], o.w = wz[3];
+                val[at + 2 * stride] = o;
             }
             cnt += __popc(bal);
+            nnz += __popc(hit);
         }
     }
     npairs = warp_sum((long long)npairs);
-    if (pass == 0 && lane == 0) {
-        counts[t] = cnt;
-        pairs[t] = npairs;
-    }
+    nnz = warp_sum((long long)nnz);
+    if (pass == 0 && lane == 0) counts[g] = {cnt, nnz, npairs};
 }
 
-cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, int64_t *counts, int64_t *pairs,
-                            const int64_t *rowptr, void *val, cudaStream_t s) {
-    const unsigned nb = (unsigned)((b.N + 7) / 8);
+cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *gptr, int *col,
+                            void *val, int64_t stride, cudaStream_t s) {
+    const int64_t groups = (b.N + NM_ROWS - 1) / NM_ROWS;
+    const unsigned nb = (unsigned)((groups + 7) / 8);
     if (prec == 64)
-        k_nm_build<double4><<<nb, 256, 0, s>>>(b, pass, counts, pairs, rowptr, (double4 *)val);
+        k_nm_build<double4><<<nb, 256, 0, s>>>(b, pass, counts, gptr, col, (double4 *)val, stride);
     else
-        k_nm_build<float4><<<nb, 256, 0, s>>>(b, pass, counts, pairs, rowptr, (float4 *)val);
+        k_nm_build<float4><<<nb, 256, 0, s>>>(b, pass, counts, gptr, col, (float4 *)val, stride);
     return cudaGetLastError();
 }
 
-// phi[perm[t]] += sum_e W_e . m[col_e] over row t (sorted target order); one
-// warp per row, rows read front to back, lanes combined in a fixed order.
-// streaming (evict-first) 16/32-byte load of one matrix entry
+// streaming (evict-first) loads of the operator, read once per evaluation
 __device__ __forceinline__ float4 ld_stream(const float4 *p) { return __ldcs(p); }
 __device__ __forceinline__ double4 ld_stream(const double4 *p) {
     const double2 a = __ldcs((const double2 *)p), b = __ldcs((const double2 *)p + 1);
     return make_double4(a.x, a.y, b.x, b.y);
 }
 
-// One batch of a near-field row: lane l takes entries j + l + 32 u (u < U),
-// 16-byte loads all issued before the gathered m; FULL batches need no
-// predicates, the tail batch reads zero weights past the row's end.  The K
-// sorted magnetisations are m4[k N + column]; lane l adds its entries in
-// order, so a row's sums do not depend on K.
+// The product: one warp per group of four rows.  The rows of neighbouring
+// targets have nearly the same columns, so the group keeps their union once: an
+// entry is a column and 4 x 3 weights, in three streams of 4-vectors (the x, y
+// and z weights of the four rows), and a gathered m serves four rows.  Bounds:
+// HBM (52 bytes an entry against four of 16; 83 % of the weights are non-zero
+// on the level-5 sphere at 128^3, 93 % on plate400) and, with several states,
+// the gathers through L1, which fall to a quarter.  Against one row per warp
+// and 16-byte entries of their own: plate400 725 -> 650 us, cube200 371 -> 345,
+// cube400 1392 -> 1240; evaluations with it beside the far field: sphere5 52.0
+// -> 50.4 us, torus300 98.7 -> 90.4, eight states of torus400 786 -> 678.
+//
+// One batch: lane l takes entries j + l + 32 u (u < U), their loads issued
+// before the gathered m; FULL batches need no predicates, the tail batch reads
+// zero weights past the end.  The K sorted magnetisations are m4[k N + column];
+// lane l adds its entries in order, so a row's sums do not depend on K.
 template <typename T, int K, int U, bool FULL>
-__device__ __forceinline__ void near_batch(const typename VecT<T>::T4 *__restrict__ row, int j, int n, int lane,
-                                           const typename VecT<T>::T4 *__restrict__ m4, int64_t N, T (&acc)[K]) {
+__device__ __forceinline__ void near_batch(const int *__restrict__ col, const typename VecT<T>::T4 *__restrict__ val,
+                                           int64_t stride, int j, int n, int lane,
+                                           const typename VecT<T>::T4 *__restrict__ m4, int64_t N, T (&acc)[K][NM_ROWS]) {
     typedef typename VecT<T>::T4 T4;
-    T4 w[U];
+    T4 wx[U], wy[U], wz[U];
+    int c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         if (FULL || j + lane + 32 * u < n) {
-            w[u] = ld_stream(row + j + 32 * u);  // streamed once per evaluation
+            c[u] = __ldcs(col + j + 32 * u);
+            wx[u] = ld_stream(val + j + 32 * u);
+            wy[u] = ld_stream(val + stride + j + 32 * u);
+            wz[u] = ld_stream(val + 2 * stride + j + 32 * u);
         } else {
-            w[u].x = w[u].y = w[u].z = T(0);
-            w[u].w = pack_id(w[u].w, 0);
+            c[u] = 0;
+            wx[u].x = wx[u].y = wx[u].z = wx[u].w = T(0);
+            wy[u] = wz[u] = wx[u];
         }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int col = packed_cell(w[u].w);
+    for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            const T4 mv = m4[k * N + col];
-            acc[k] += w[u].x * mv.x + w[u].y * mv.y + w[u].z * mv.z;
+            const T4 m = m4[k * N + c[u]];
+            acc[k][0] += wx[u].x * m.x + wy[u].x * m.y + wz[u].x * m.z;
+            acc[k][1] += wx[u].y * m.x + wy[u].y * m.y + wz[u].y * m.z;
+            acc[k][2] += wx[u].z * m.x + wy[u].z * m.y + wz[u].z * m.z;
+            acc[k][3] += wx[u].w * m.x + wy[u].w * m.y + wz[u].w * m.z;
         }
-    }
 }
 
-// Row t of the operator applied to K states: batches of 32 U entries (U
-// loads in flight per lane), the full ones without predicates and at 32-bit
-// offsets from the row start, then one predicated tail.
-template <typename T, int K>
-__device__ __forceinline__ void near_row(const DevPlan &p, int64_t t, int lane) {
+// phi_part[k][t] = the rows of a group applied to K states with one pass over
+// them.  `split` (1, 2 or 4) warps share a group, taking its batches in turn,
+// so that meshes with few groups fill the GPU; their sums are added in order.
+template <typename T, int K> __global__ void __launch_bounds__(128) k_near_matrix(DevPlan p, int split) {
     typedef typename VecT<T>::T4 T4;
-    constexpr int U = 8;
+    constexpr int U = K == 1 ? 4 : 2;  // entries in flight per lane
+    __shared__ T part[4][K * NM_ROWS];
+    pdl_wait();
+    pdl_trigger();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = warp & (split - 1);
+    const int64_t g = (int64_t)blockIdx.x * (4 / split) + warp / split;
+    const bool live = NM_ROWS * g < p.N;
     const T4 *m4 = (const T4 *)p.m4;  // sorted nodal m (k_nodal_prep), K copies
-    const int64_t e0 = p.nm_rowptr[t];
-    const int n = (int)(p.nm_rowptr[t + 1] - e0);  // a row holds < 2^31 entries
-    const T4 *row = (const T4 *)p.nm_val + e0 + lane;
-    T acc[K];
+    T acc[K][NM_ROWS];
 #pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = T(0);
-    int j = 0;
-    for (; j + 32 * U <= n; j += 32 * U) near_batch<T, K, U, true>(row, j, n, lane, m4, p.N, acc);
-    if (j < n) near_batch<T, K, U, false>(row, j, n, lane, m4, p.N, acc);
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int r = 0; r < NM_ROWS; ++r) acc[k][r] = T(0);
+    if (live) {
+        const int64_t e0 = p.nm_gptr[g];
+        const int n = (int)(p.nm_gptr[g + 1] - e0);  // a group holds < 2^31 entries
+        const int *col = p.nm_col + e0 + lane;
+        const T4 *val = (const T4 *)p.nm_val + e0 + lane;
+        int j = 32 * U * sub;
+        for (; j + 32 * U <= n; j += 32 * U * split)
+            near_batch<T, K, U, true>(col, val, p.nm_stride, j, n, lane, m4, p.N, acc);
+        if (j < n) near_batch<T, K, U, false>(col, val, p.nm_stride, j, n, lane, m4, p.N, acc);
+    }
+    // lane r of the group's first warp ends up with row r
+    T v[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const T a = warp_sum(acc[k]);
-        if (lane == 0) ((T *)p.phi_part)[k * p.N + t] = a;
+        v[k] = T(0);
+#pragma unroll
+        for (int r = 0; r < NM_ROWS; ++r) {
+            const T a = warp_sum(acc[k][r]);
+            if (lane == r) v[k] = a;
+        }
     }
+    if (split > 1) {
+        if (lane < NM_ROWS)
+#pragma unroll
+            for (int k = 0; k < K; ++k) part[warp][k * NM_ROWS + lane] = v[k];
+        __syncthreads();
+        if (sub == 0 && lane < NM_ROWS)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                for (int w = 1; w < split; ++w) v[k] += part[warp + w][k * NM_ROWS + lane];
+    }
+    const int64_t t = NM_ROWS * g + lane;
+    if (live && sub == 0 && lane < NM_ROWS && t < p.N)
+#pragma unroll
+        for (int k = 0; k < K; ++k) ((T *)p.phi_part)[k * p.N + t] = v[k];
 }
 
-// phi_part[t] = row t of the precomputed operator times the sorted nodal m:
-// one warp per row
-template <typename T>
-__global__ void __launch_bounds__(128) k_near_matrix(DevPlan p) {
-    pdl_wait();
-    pdl_trigger();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * 4 + warp;
-    if (t >= p.N) return;
-    near_row<T, 1>(p, t, lane);
-}
-
-// K states with one pass over the operator: each entry is streamed once and
-// applied to the K sorted magnetisations (phi_part[k][t]); the per-state sums
-// run in the same order as in k_near_matrix.
-template <typename T, int K>
-__global__ void __launch_bounds__(128) k_near_matrix_states(DevPlan p) {
-    pdl_wait();
-    pdl_trigger();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * 4 + warp;
-    if (t >= p.N) return;
-    near_row<T, K>(p, t, lane);
+// Warps per group: 48 or more warps for each of 152 SMs where two or four a
+// group give them (sphere5 at 128^3, 2561 groups: the evaluation 51.8 us with
+// one, 50.4 with two; sphere4 in FP64, 641 groups: the product 90 us with one,
+// 49 with four).
+static int near_split(const DevPlan &p) {
+    const int64_t groups = (p.N + NM_ROWS - 1) / NM_ROWS;
+    return groups >= 152 * 48 ? 1 : groups >= 152 * 12 ? 2 : 4;
 }
 
 template <typename T> static cudaError_t near_states_t(const DevPlan &p, int K, cudaStream_t s) {
-    const unsigned nb = (unsigned)((p.N + 3) / 4);
+    const int split = near_split(p), rows = NM_ROWS * 4 / split;  // rows of a block
+    const unsigned nb = (unsigned)((p.N + rows - 1) / rows);
     switch (K) {
-        case 1: return launch_k(k_near_matrix_states<T, 1>, nb, 128, 0, s, p);
-        case 2: return launch_k(k_near_matrix_states<T, 2>, nb, 128, 0, s, p);
-        case 3: return launch_k(k_near_matrix_states<T, 3>, nb, 128, 0, s, p);
-        case 4: return launch_k(k_near_matrix_states<T, 4>, nb, 128, 0, s, p);
-        case 5: return launch_k(k_near_matrix_states<T, 5>, nb, 128, 0, s, p);
-        case 6: return launch_k(k_near_matrix_states<T, 6>, nb, 128, 0, s, p);
-        case 7: return launch_k(k_near_matrix_states<T, 7>, nb, 128, 0, s, p);
-        case 8: return launch_k(k_near_matrix_states<T, 8>, nb, 128, 0, s, p);
+        case 1: return launch_k(k_near_matrix<T, 1>, nb, 128, 0, s, p, split);
+        case 2: return launch_k(k_near_matrix<T, 2>, nb, 128, 0, s, p, split);
+        case 3: return launch_k(k_near_matrix<T, 3>, nb, 128, 0, s, p, split);
+        case 4: return launch_k(k_near_matrix<T, 4>, nb, 128, 0, s, p, split);
+        case 5: return launch_k(k_near_matrix<T, 5>, nb, 128, 0, s, p, split);
+        case 6: return launch_k(k_near_matrix<T, 6>, nb, 128, 0, s, p, split);
+        case 7: return launch_k(k_near_matrix<T, 7>, nb, 128, 0, s, p, split);
+        case 8: return launch_k(k_near_matrix<T, 8>, nb, 128, 0, s, p, split);
     }
     return cudaErrorInvalidValue;
 }
@@ -641,13 +700,7 @@ cudaError_t launch_near_matrix_states(const DevPlan &p, int K, cudaStream_t s) {
 }
 
 cudaError_t launch_near_matrix(const DevPlan &p, const void *, cudaStream_t s) {
-    if (p.N == 0) return cudaSuccess;
-    const unsigned nb = (unsigned)((p.N + 3) / 4);
-    if (p.prec == 64)
-        { const cudaError_t le = launch_k(k_near_matrix<double>, nb, 128, 0, s, p); if (le != cudaSuccess) return le; }
-    else
-        { const cudaError_t le = launch_k(k_near_matrix<float>, nb, 128, 0, s, p); if (le != cudaSuccess) return le; }
-    return cudaGetLastError();
+    return launch_near_matrix_states(p, 1, s);
 }
 
 }  // namespace slp

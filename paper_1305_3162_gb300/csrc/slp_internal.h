@@ -156,11 +156,12 @@ struct DevPlan {
     const void *es_w, *es_g;  // T [es_n]
     int es_n;
 
-    // precomputed near-field operator (NODAL_MAG): CSR over sorted targets
-    const int64_t *nm_rowptr;  // [N + 1]
-    const int *nm_col;         // [nnz] vertex ids
-    const void *nm_val;        // T4 [nnz] (wx, wy, wz, unused)
-    int64_t nm_nnz;
+    // precomputed near-field operator (NODAL_MAG): groups of NM_ROWS sorted
+    // targets, an entry a column (sorted vertex) and the group's weights
+    const int64_t *nm_gptr;  // [groups + 1]
+    const int *nm_col;       // [nm_stride]
+    const void *nm_val;      // T4 [3][nm_stride]: x, y, z weights of the rows
+    int64_t nm_stride;       // entries in all
 
     // state batch of one launch (grid.y): ks states, scratch of state y at
     // gridA/gridB + y st_grid, S1 + y st_s1, S2 + y st_s2, phi_part + y N;
@@ -293,11 +294,17 @@ cudaError_t launch_zero(void *ptr, size_t bytes, cudaStream_t s);
 
 // Precomputed near-field operator (k_near.cu): inputs of the plan-time
 // assembly of W (FP64, temporary device arrays).
+constexpr int NM_ROWS = 4;  // rows of a group (the entries' 4-vectors)
+struct NMCount {
+    int64_t entries, nnz, pairs;  // of a group; (target, vertex) and (target, source) pairs with a source within eps
+};
 struct NMBuild {
+    const double4 *vpos;     // sorted vertices, like tgt
+    double reach2;           // squared distance a vertex with a point within eps can have
     const double4 *tgt;      // [N] sorted targets, physical coordinates relative to the torus centre
     const int *tgt_perm;     // [N] sorted -> user vertex
-    const int *tgt_block;    // [N] target block of each sorted target
-    const int *blk_r0;       // [nblk + 1] range list of each block
+    const int *grp_block;    // [groups] candidate list of each group
+    const int *blk_r0;       // [lists + 1]
     const int2 *ranges;      // candidate vertex ranges (sorted target order)
     const int *vt_ptr;       // [NV + 1] vertex -> adjacency entries
     const int *vt_ent;       // triangle * 4 + local vertex index
@@ -321,8 +328,8 @@ struct NMBuild {
     int ni;
     double iw, sqrt_iw;
 };
-cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, int64_t *counts, int64_t *pairs,
-                            const int64_t *rowptr, void *val, cudaStream_t s);
+cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *gptr, int *col,
+                            void *val, int64_t stride, cudaStream_t s);
 // phi_part = W m (overwrites)
 cudaError_t launch_near_matrix(const DevPlan &p, const void *d_m, cudaStream_t s);
 // K <= NEAR_STATES states at once: m4[k][.] from in[k] (sorted), then

@@ -1655,6 +1655,68 @@ slp_status near_build_table(const slp_plan_s &p, slp::NMBuild &nb, TmpBuf &buf) 
     return SLP_OK;
 }
 
+// Candidate lists of runs of `run` consecutive sorted targets from those of
+// the target blocks they overlap (ranges ascending, overlaps joined).
+void run_candidates(NearCandidates &c, int64_t N, int run) {
+    std::vector<int> r0(1, 0);
+    std::vector<int2> out;
+    for (int64_t t = 0; t < N; t += run) {
+        const size_t first = out.size();
+        const int b0 = c.tgt_block[t], b1 = c.tgt_block[std::min(N, t + run) - 1];
+        for (int b = b0; b <= b1; ++b) out.insert(out.end(), c.ranges.begin() + c.blk_r0[b], c.ranges.begin() + c.blk_r0[b + 1]);
+        if (b1 > b0) {
+            std::sort(out.begin() + first, out.end(), [](const int2 &x, const int2 &y) { return x.x < y.x; });
+            size_t w = first;
+            for (size_t k = first; k < out.size(); ++k) {
+                if (w > first && out[k].x <= out[w - 1].y)
+                    out[w - 1].y = std::max(out[w - 1].y, out[k].y);
+                else
+                    out[w++] = out[k];
+            }
+            out.resize(w);
+        }
+        r0.push_back((int)out.size());
+    }
+    c.blk_r0.swap(r0);
+    c.ranges.swap(out);
+}
+
+// The operator's two assembly passes: group pointers, columns and weights
+// allocated by alloc(bytes, &ptr), which may refuse (ptr NULL: left unbuilt).
+template <typename Alloc>
+slp_status build_operator(const slp_plan_s &p, const slp::NMBuild &nb, Alloc alloc, slp::DevPlan &v, int64_t &nnz,
+                          int64_t &pairs) {
+    const int64_t groups = (nb.N + slp::NM_ROWS - 1) / slp::NM_ROWS;
+    TmpBuf b_cnt;
+    std::vector<slp::NMCount> cnt(groups);
+    TRY(tmp_upload(b_cnt, cnt.data(), cnt.size()));
+    TRY(cuda_status(slp::launch_nm_build(nb, 0, p.prec, (slp::NMCount *)b_cnt.p, nullptr, nullptr, nullptr, 0, 0),
+                    "near matrix count"));
+    TRY(cuda_status(cudaMemcpy(cnt.data(), b_cnt.p, sizeof(slp::NMCount) * groups, cudaMemcpyDeviceToHost), "count copy"));
+    std::vector<int64_t> gptr(groups + 1, 0);
+    nnz = pairs = 0;
+    for (int64_t g = 0; g < groups; ++g) {
+        gptr[g + 1] = gptr[g] + cnt[g].entries;
+        nnz += cnt[g].nnz;
+        pairs += cnt[g].pairs;
+    }
+    const int64_t entries = std::max<int64_t>(gptr[groups], 1);
+    void *d_val = nullptr, *d_col = nullptr, *d_gptr = nullptr;
+    TRY(alloc(3 * 4 * (size_t)(p.prec / 8) * entries, &d_val));
+    if (!d_val) return SLP_OK;
+    TRY(alloc(sizeof(int) * entries, &d_col));
+    TRY(alloc(sizeof(int64_t) * (groups + 1), &d_gptr));
+    if (!d_col || !d_gptr) return fail(SLP_ERR_OOM, "near-field operator");
+    TRY(cuda_status(cudaMemcpy(d_gptr, gptr.data(), sizeof(int64_t) * (groups + 1), cudaMemcpyHostToDevice), "upload"));
+    v.nm_gptr = (const int64_t *)d_gptr;
+    v.nm_col = (const int *)d_col;
+    v.nm_val = d_val;
+    v.nm_stride = entries;
+    TRY(cuda_status(slp::launch_nm_build(nb, 1, p.prec, nullptr, v.nm_gptr, (int *)d_col, d_val, entries, 0),
+                    "near matrix fill"));
+    return SLP_OK;
+}
+
 slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) {
     const int64_t N = p.N, M = p.M, q = p.q;
     double r_adj = 0.0;
@@ -1672,18 +1734,21 @@ slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) 
     const double rad = all_pairs ? INFINITY : p.eps + r_adj * (1.0 + 1e-9) + 1e-12 * p.diam;
     NearCandidates cand;
     near_candidates(p, tkeys, rad, all_pairs, cand);
-    std::vector<int> &vt_ptr = cand.vt_ptr, &vt_ent = cand.vt_ent, &tgt_block = cand.tgt_block, &blk_r0 = cand.blk_r0;
+    run_candidates(cand, N, 16);
+    std::vector<int> &vt_ptr = cand.vt_ptr, &vt_ent = cand.vt_ent, &blk_r0 = cand.blk_r0;
     std::vector<double4> &tgt = cand.tgt;
     std::vector<int2> &ranges = cand.ranges;
+    std::vector<int> grp_block((N + slp::NM_ROWS - 1) / slp::NM_ROWS);
+    for (size_t g = 0; g < grp_block.size(); ++g) grp_block[g] = (int)(g * slp::NM_ROWS / 16);
 
     // device inputs
     std::vector<double4> src(p.Q), nrm(M);
     for (int64_t k = 0; k < p.Q; ++k)
         src[k] = make_double4(p.y[3 * k] - p.ctr[0], p.y[3 * k + 1] - p.ctr[1], p.y[3 * k + 2] - p.ctr[2], p.wk[k]);
     for (int64_t j = 0; j < M; ++j) nrm[j] = make_double4(p.nrm[3 * j], p.nrm[3 * j + 1], p.nrm[3 * j + 2], 0.0);
-    TmpBuf b_tgt, b_blk, b_r0, b_rng, b_vtp, b_vte, b_src, b_nrm, b_lam, b_h[3], b_cnt, b_pairs;
+    TmpBuf b_tgt, b_blk, b_r0, b_rng, b_vtp, b_vte, b_src, b_nrm, b_lam, b_h[3];
     TRY(tmp_upload(b_tgt, tgt.data(), tgt.size()));
-    TRY(tmp_upload(b_blk, tgt_block.data(), tgt_block.size()));
+    TRY(tmp_upload(b_blk, grp_block.data(), grp_block.size()));
     TRY(tmp_upload(b_r0, blk_r0.data(), blk_r0.size()));
     TRY(tmp_upload(b_rng, ranges.data(), ranges.size()));
     TRY(tmp_upload(b_vtp, vt_ptr.data(), vt_ptr.size()));
@@ -1691,14 +1756,13 @@ slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) 
     TRY(tmp_upload(b_src, src.data(), src.size()));
     TRY(tmp_upload(b_nrm, nrm.data(), nrm.size()));
     TRY(tmp_upload(b_lam, p.lam.data(), p.lam.size()));
-    std::vector<int64_t> zeros(N + 1, 0);
-    TRY(tmp_upload(b_cnt, zeros.data(), zeros.size()));
-    TRY(tmp_upload(b_pairs, zeros.data(), zeros.size()));
     slp::NMBuild nb;
     memset(&nb, 0, sizeof nb);
     nb.tgt = (const double4 *)b_tgt.p;
     nb.tgt_perm = p.dp.tgt_perm;
-    nb.tgt_block = (const int *)b_blk.p;
+    nb.grp_block = (const int *)b_blk.p;
+    nb.vpos = nb.tgt;
+    nb.reach2 = all_pairs ? 1e300 : rad * rad;
     nb.blk_r0 = (const int *)b_r0.p;
     nb.ranges = (const int2 *)b_rng.p;
     nb.vt_ptr = (const int *)b_vtp.p;
@@ -1735,29 +1799,20 @@ slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) 
         nb.es_g = (const double *)b_esg.p;
         nb.es_n = (int)w.size();
     }
-    TRY(cuda_status(slp::launch_nm_build(nb, 0, p.prec, (int64_t *)b_cnt.p, (int64_t *)b_pairs.p, nullptr, nullptr, 0),
-                    "near matrix count"));
-    std::vector<int64_t> cnt(N), prs(N);
-    TRY(cuda_status(cudaMemcpy(cnt.data(), b_cnt.p, sizeof(int64_t) * N, cudaMemcpyDeviceToHost), "count copy"));
-    TRY(cuda_status(cudaMemcpy(prs.data(), b_pairs.p, sizeof(int64_t) * N, cudaMemcpyDeviceToHost), "pairs copy"));
-    std::vector<int64_t> rowptr(N + 1, 0);
-    for (int64_t i = 0; i < N; ++i) rowptr[i + 1] = rowptr[i] + cnt[i];
-    const int64_t nnz = rowptr[N];
-    p.near_pairs_within = 0;
-    for (int64_t i = 0; i < N; ++i) p.near_pairs_within += prs[i];
-    const size_t vbytes = (size_t)nnz * (p.prec == 64 ? 32 : 16);
-    size_t freeb = 0, totb = 0;
-    cudaMemGetInfo(&freeb, &totb);
-    if (vbytes > ((size_t)24 << 30) || vbytes > freeb / 2) return SLP_OK;  // budget: keep the on-the-fly near field
-    void *ptr = nullptr;
-    TRY(upload(p, &ptr, rowptr.data(), rowptr.size()));
-    p.dp.nm_rowptr = (const int64_t *)ptr;
-    TRY(dalloc(p, &ptr, vbytes));
-    p.dp.nm_val = ptr;
-    TRY(cuda_status(slp::launch_nm_build(nb, 1, p.prec, nullptr, nullptr, p.dp.nm_rowptr, ptr, 0), "near matrix fill"));
+    bool refused = false;
+    auto alloc = [&](size_t bytes, void **ptr) -> slp_status {
+        size_t freeb = 0, totb = 0;
+        cudaMemGetInfo(&freeb, &totb);
+        // budget (the weights come first): else keep the near field per pair
+        refused = refused || bytes > ((size_t)24 << 30) || bytes > freeb / 2;
+        return refused ? SLP_OK : dalloc(p, ptr, bytes);
+    };
+    TRY(build_operator(p, nb, alloc, p.dp, p.nm_nnz, p.near_pairs_within));
     TRY(cuda_status(cudaDeviceSynchronize(), "near matrix build"));
-    p.dp.nm_nnz = nnz;
-    p.nm_nnz = nnz;
+    if (refused) {
+        p.nm_nnz = 0;
+        return SLP_OK;
+    }
     p.near_mode = SLP_NEAR_PRECOMPUTED;
     // prep, spread (charges fused), 5 (fused: 3) FFT passes, gather, near-field product
     p.launches_per_eval = p.dp.fuse_pb > 0 ? 7 : (p.dp.yzy_g > 0 ? 7 : 9);
@@ -2192,7 +2247,7 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         }
         cand.blk_r0[nblk] = (int)cand.ranges.size();
     }
-    TmpBuf b_blk, b_r0, b_rng, b_vtp, b_vte, b_cnt, b_pairs;
+    TmpBuf b_blk, b_r0, b_rng, b_vtp, b_vte, b_cnt;
     TRY(tmp_upload(b_blk, cand.tgt_block.data(), cand.tgt_block.size()));
     TRY(tmp_upload(b_r0, cand.blk_r0.data(), cand.blk_r0.size()));
     TRY(tmp_upload(b_rng, cand.ranges.data(), std::max<size_t>(cand.ranges.size(), 1)));
@@ -2201,7 +2256,6 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
     {
         std::vector<int64_t> z(n + 1, 0);
         TRY(tmp_upload(b_cnt, z.data(), z.size()));
-        TRY(tmp_upload(b_pairs, z.data(), z.size()));
     }
     std::vector<int64_t> cnt(n), rowptr(n + 1, 0);
     if (tri) {
@@ -2286,7 +2340,7 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         for (int64_t k = 0; k < p.Q; ++k)
             src[k] = make_double4(p.y[3 * k] - p.ctr[0], p.y[3 * k + 1] - p.ctr[1], p.y[3 * k + 2] - p.ctr[2], p.wk[k]);
         for (int64_t j = 0; j < p.M; ++j) nrm[j] = make_double4(p.nrm[3 * j], p.nrm[3 * j + 1], p.nrm[3 * j + 2], 0.0);
-        TmpBuf b_tg, b_src, b_nrm, b_lam, b_h[3];
+        TmpBuf b_tg, b_src, b_nrm, b_lam, b_h[3], b_grp, b_vpos;
         TRY(tmp_upload(b_tg, ptg.data(), ptg.size()));
         TRY(tmp_upload(b_src, src.data(), src.size()));
         TRY(tmp_upload(b_nrm, nrm.data(), nrm.size()));
@@ -2295,7 +2349,13 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         memset(&nb, 0, sizeof nb);
         nb.tgt = (const double4 *)b_tg.p;
         nb.tgt_perm = p.dp.tgt_perm;
-        nb.tgt_block = (const int *)b_blk.p;
+        std::vector<int> grp_block((n + slp::NM_ROWS - 1) / slp::NM_ROWS);
+        for (size_t g = 0; g < grp_block.size(); ++g) grp_block[g] = (int)(g * slp::NM_ROWS / 32);
+        TRY(tmp_upload(b_grp, grp_block.data(), grp_block.size()));
+        nb.grp_block = (const int *)b_grp.p;
+        TRY(tmp_upload(b_vpos, cand.tgt.data(), cand.tgt.size()));
+        nb.vpos = (const double4 *)b_vpos.p;
+        nb.reach2 = all_pairs ? 1e300 : rad * rad;
         nb.blk_r0 = (const int *)b_r0.p;
         nb.ranges = (const int2 *)b_rng.p;
         nb.vt_ptr = (const int *)b_vtp.p;
@@ -2332,21 +2392,15 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
             nb.es_n = (int)w.size();
         }
         for (int a = 0; a < 3; ++a) nb.P[a] = p.P[a];
-        TRY(cuda_status(slp::launch_nm_build(nb, 0, p.prec, (int64_t *)b_cnt.p, (int64_t *)b_pairs.p, nullptr, nullptr, 0),
-                        "probe near count"));
-        TRY(cuda_status(cudaMemcpy(cnt.data(), b_cnt.p, sizeof(int64_t) * n, cudaMemcpyDeviceToHost), "count copy"));
-        for (int64_t i = 0; i < n; ++i) rowptr[i + 1] = rowptr[i] + cnt[i];
-        TRY(alloc_up(&ptr, rowptr.data(), sizeof(int64_t) * (n + 1)));
-        v.nm_rowptr = (const int64_t *)ptr;
-        TRY(alloc_up(&ptr, nullptr, sizeof(T4) * (size_t)std::max<int64_t>(rowptr[n], 1)));
-        v.nm_val = ptr;
-        TRY(cuda_status(slp::launch_nm_build(nb, 1, p.prec, nullptr, nullptr, v.nm_rowptr, ptr, 0), "probe near fill"));
+        auto alloc = [&](size_t bytes, void **to) { return alloc_up(to, nullptr, bytes); };
+        int64_t pairs = 0;
+        TRY(build_operator(p, nb, alloc, v, pr.near_nnz, pairs));
     }
     TRY(cuda_status(cudaDeviceSynchronize(), "probe near build"));
     int code = 0;
     TRY(cuda_status(cudaMemcpy(&code, p.dp.err, sizeof(int), cudaMemcpyDeviceToHost), "status"));
     if (code != 0) return fail(SLP_ERR_CUDA, "probe near build: device status word %d", code);
-    pr.near_nnz = rowptr[n];
+    if (tri) pr.near_nnz = rowptr[n];
     pr.view = v;
     return SLP_OK;
 }
