@@ -698,6 +698,9 @@ void tile_items(const std::vector<double> &grid, const std::vector<uint64_t> &ke
         while (j < n && (keys[j] >> 32) == tile) ++j;
         const uint32_t packed = (uint32_t)grid[4 * i + 3];
         const int cx = packed & 1023, cy = (packed >> 10) & 1023, cz = (packed >> 20) & 1023;
+        // full chunks and a rest, not even shares: the rests, dispatched last, fill
+        // the tail of a launch (level-5 sphere, 692 items on 608 places: 57.1 us
+        // an evaluation, even shares 60.5)
         for (int64_t b = i; b < j; b += chunk) {
             slp::TileItem it;
             it.c0x = cx / ts * ts;
@@ -2841,9 +2844,11 @@ slp_status slp_plan(const slp_mesh *mesh, int quadrature, double tolerance, cons
     sort_points(*p, p->y.data(), p->Q, p->TS, p->src_perm, p->src_grid, skeys);
     sort_points(*p, p->V.data(), p->N, p->TSg, p->tgt_perm, p->tgt_grid, tkeys);
     {
-        // spread chunk: about four items per SM, 128..1024 sources, a multiple of 32
+        // spread chunk: about four items per SM, 32..1024 sources, a multiple of
+        // 32 (at least 128: sphere3 at 64^3 29.9 us an evaluation, 24.4 at 32;
+        // cube20 at 128^3 39.4, 35.0; torus120 36.7, 33.1 at its 64)
         int64_t ch = (p->Q + 152 * 4 - 1) / (152 * 4);
-        ch = std::max<int64_t>(128, std::min<int64_t>(1024, (ch + 31) / 32 * 32));
+        ch = std::max<int64_t>(32, std::min<int64_t>(1024, (ch + 31) / 32 * 32));
         // wide windows: an item's tile costs about as much as one source to
         // clear and flush, and the FP64 pipe of an SM is the limit, so even
         // shares of it matter more: about eight items per SM
