@@ -13,11 +13,12 @@
 //   IY  S2 -> S1, zero-padded inverse along y
 //   IX  S1 -> grid B (real), two rows per complex inverse FFT
 //
-// Each pass stages a batch of 1-D transforms in shared memory and runs a
-// mixed-radix (8/4/2) Stockham autosort FFT on them; consecutive threads
-// work on consecutive columns, so shared-memory accesses are conflict free
-// and global accesses coalesce along the contiguous axis.  FX also writes
-// zeros back to grid A so the next spread starts from a clean grid.
+// Transforms are mixed radix (8/4/2).  Lengths 32 to 1024 along y and z and 128
+// to 1024 along x run with the length fixed at compile time and the elements
+// in registers (column and row engines below); the others stage a batch of 1-D
+// transforms in shared memory.  Global accesses coalesce along the contiguous
+// axis.  FX also writes zeros back to grid A so the next spread starts from a
+// clean grid.
 //
 // All passes are restricted to the plan's active region: the row pairs of
 // grid A the spread can reach (FX), and the rows of grid B the gather reads
@@ -555,7 +556,7 @@ __global__ void __launch_bounds__(256) k_ix(DevPlan p, int PB) {
 // frequency stages of fft_columns_inplace (radix 8, then 4 or 2 for the
 // remaining bits).  Stage 0 reads its elements from global memory and the
 // last stage writes them back; between stages the elements are exchanged
-// through one shared buffer [L][CB + 1] with one barrier per exchange.  A
+// through one shared buffer [L][CB] with one barrier per exchange.  A
 // thread writes back exactly the positions it read, so a stage needs no
 // barrier between its read and its write.
 constexpr int CB = 8;
@@ -590,25 +591,31 @@ template <int LG> __device__ __forceinline__ int col_freq(int p) {
     return k;
 }
 
+// twiddles by stage: W^(r j) of the stage with step Q (its elements are Q apart)
+// at r Q + j, so a stage reads consecutive j at constant offsets r Q
+template <typename C, int LG> __device__ __forceinline__ void col_twiddles(C *tw, const C *full) {
+    for (int i = threadIdx.x; i < (1 << LG); i += blockDim.x) {
+        const int lgi = i > 0 ? 31 - __clz(i) : 0;
+        const int S = (LG - 1 - lgi) / 3, lgQ = LG - 3 * S - 3;
+        if (lgQ >= 0) tw[i] = full[(((i >> lgQ) * (i & ((1 << lgQ) - 1))) << (3 * S)) & ((1 << LG) - 1)];
+    }
+}
+
 // stage S on the eight elements of task t (forward: DFT then twiddle;
 // inverse: conjugate twiddle then DFT)
 template <typename C, int LG, int S, bool INV> __device__ __forceinline__ void col_stage(C (&v)[8], int t, const C *tw) {
     typedef ColShape<LG> Sh;
     if constexpr (S < Sh::S8) {
         constexpr int lgQ = LG - 3 * S - 3;
-        const int j = t & ((1 << lgQ) - 1);
-        if (INV && j != 0) {
+        const C *w = tw + (t & ((1 << lgQ) - 1));
+        if constexpr (INV && lgQ > 0) {
 #pragma unroll
-            for (int r = 1; r < 8; ++r) {
-                C w = tw[((r * j) << (3 * S)) & (Sh::L - 1)];
-                w.y = -w.y;
-                v[r] = cmul(v[r], w);
-            }
+            for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], cconj(w[r << lgQ]));
         }
         dft8<C, INV>(v);
-        if (!INV && j != 0) {
+        if constexpr (!INV && lgQ > 0) {
 #pragma unroll
-            for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[((r * j) << (3 * S)) & (Sh::L - 1)]);
+            for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[r << lgQ]);
         }
     } else if constexpr (Sh::REM == 2) {
         dft4<C, INV>(v[0], v[1], v[2], v[3]);
@@ -619,13 +626,32 @@ template <typename C, int LG, int S, bool INV> __device__ __forceinline__ void c
     }
 }
 
-template <typename C, int LG, int S> __device__ __forceinline__ void col_put(C *buf, const C (&v)[8], int t, int b) {
+// Position p of the exchange buffer, rows of CB columns.  A half-warp (FP32)
+// holds two neighbouring tasks, whose positions differ in bit 0 or, in the last
+// stage, in bit 3; with bit 3 folded into bit 0 the two rows lie in different
+// halves of the banks in every stage (rows of CB + 1 collide in one bank in all
+// but the last, which doubles those wavefronts).  With the twiddles by stage
+// and the constant offsets below, 512^3 serial: FY 39 -> 38, FZ 89 -> 74,
+// IY 42 -> 35 us, FZ with 75 % of its issue slots taken.
+__device__ __forceinline__ int col_at(int p) { return (p ^ ((p >> 3) & 1)) * CB; }
+
+// col_at is linear over exclusive or, and element r of a task differs from
+// element 0 in bits that are zero there: two addresses per stage (with bit 0 as
+// it is and flipped), constant offsets from them
+template <int LG, int S, typename F> __device__ __forceinline__ void col_each(int t, int b, F f) {
+    constexpr int lgQ = S < ColShape<LG>::S8 ? LG - 3 * S - 3 : 0;
+    const int a0 = col_at(col_idx<LG, S>(t, 0)) + b, a1 = a0 ^ CB;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) buf[col_idx<LG, S>(t, r) * (CB + 1) + b] = v[r];
+    for (int r = 0; r < 8; ++r) {
+        const int c = r << lgQ, at = c ^ ((c >> 3) & 1);
+        f(r, ((at & 1) ? a1 : a0) + (at & ~1) * CB);
+    }
+}
+template <typename C, int LG, int S> __device__ __forceinline__ void col_put(C *buf, const C (&v)[8], int t, int b) {
+    col_each<LG, S>(t, b, [&](int r, int at) { buf[at] = v[r]; });
 }
 template <typename C, int LG, int S> __device__ __forceinline__ void col_get(const C *buf, C (&v)[8], int t, int b) {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = buf[col_idx<LG, S>(t, r) * (CB + 1) + b];
+    col_each<LG, S>(t, b, [&](int r, int at) { v[r] = buf[at]; });
 }
 
 // forward stages S .. NS-1 (the elements of stage S - 1 are in v and are
@@ -659,8 +685,8 @@ __device__ __forceinline__ void k_fy_c_body(const DevPlan &p) {
     typedef ColShape<LG> Sh;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = (C *)smem_raw;
-    C *tw = buf + Sh::L * (CB + 1);
-    for (int i = threadIdx.x; i < Sh::L; i += blockDim.x) tw[i] = ((const C *)p.tw[1])[i];
+    C *tw = buf + Sh::L * CB;
+    col_twiddles<C, LG>(tw, (const C *)p.tw[1]);
     const int b = threadIdx.x & (CB - 1), t = threadIdx.x >> 3;
     const int Kx = p.Kx, ny = p.n[1];
     const int ntile = Kx / CB;
@@ -705,8 +731,8 @@ __global__ void __launch_bounds__(1 << LG, (1024 >> LG) > 0 ? (1024 >> LG) : 1) 
     typedef ColShape<LG> Sh;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = (C *)smem_raw;
-    C *tw = buf + Sh::L * (CB + 1);
-    for (int i = threadIdx.x; i < Sh::L; i += blockDim.x) tw[i] = ((const C *)p.tw[2])[i];
+    C *tw = buf + Sh::L * CB;
+    col_twiddles<C, LG>(tw, (const C *)p.tw[2]);
     const int b = threadIdx.x & (CB - 1), t = threadIdx.x >> 3;
     const int Kx = p.Kx, ny = p.n[1], nz = p.n[2];
     const int ntile = Kx / CB;
@@ -765,8 +791,8 @@ __device__ __forceinline__ void k_iy_c_body(const DevPlan &p) {
     typedef ColShape<LG> Sh;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = (C *)smem_raw;
-    C *tw = buf + Sh::L * (CB + 1);
-    for (int i = threadIdx.x; i < Sh::L; i += blockDim.x) tw[i] = ((const C *)p.tw[1])[i];
+    C *tw = buf + Sh::L * CB;
+    col_twiddles<C, LG>(tw, (const C *)p.tw[1]);
     const int b = threadIdx.x & (CB - 1), t = threadIdx.x >> 3;
     const int Kx = p.Kx, ny = p.n[1];
     const int ntile = Kx / CB;
@@ -805,88 +831,213 @@ __global__ void __launch_bounds__(1 << LG, (1024 >> LG)) k_iy_c(DevPlan p) { k_i
 template <typename T, int LG>
 __global__ void __launch_bounds__(1 << LG) k_iy_c_long(DevPlan p) { k_iy_c_body<T, LG>(p); }
 
-// ---------------------------------------------------------------- x inverse, compile-time length
-// The inverse row pass with Lx = 2^LG fixed at compile time: CB row pairs per block,
-// L / 8 threads per pair (t fastest, so a warp touches consecutive x), one
-// radix-8 butterfly per thread per stage (radix 8 stages, then 4 or 2).
-// Stockham stages take natural-order input (the first stage reads the
-// spectrum straight from S1) and leave natural-order output, which is read
-// back by consecutive x.  One shared buffer: a stage reads its eight inputs,
-// waits, writes its eight outputs, waits.
-template <typename C, int LG, int S, bool INV>
-__device__ __forceinline__ void stk_compute_store(C *buf, C (&v)[8], int t, int b, const C *tw) {
-    typedef ColShape<LG> Sh;
-    constexpr int LGR = S < Sh::S8 ? 3 : Sh::REM;
-    constexpr int R = 1 << LGR, NB = 8 / R, lgNs = 3 * S;
+// ---------------------------------------------------------------- row engine
+// The row passes FX and IX with Lx = 2^LG fixed at compile time.  A row pair is
+// one complex transform by L / 8 threads, t fastest, so a warp reads and writes
+// consecutive x of the grid and consecutive frequencies of S1: stage 0 takes
+// its elements from global memory, and the last inverse stage writes them
+// back.  Radix-8 Stockham stages (then 4 or 2) keep eight elements per thread
+// in registers and exchange them through a buffer of the pair's own (pairs of up to
+// 32 threads need no block barrier).
+//   buffer: element i at row_at(i); the 16 (FP32) or 8 (FP64) lanes of one
+//     wavefront hit different banks both in the stores of every stage (strides
+//     1, 8 and blocks of 8 in steps of 64) and in the loads (consecutive i);
+//   twiddles: [stage][r][k], read by consecutive k (stage s at 8^s - 8, L - 8
+//     entries in all); a thread requests its share of them and its row before
+//     it waits for either.
+// The passes are bound by the latency of their global reads (a third of the
+// cycles of FX, the largest share), not by shared memory any more.  FP32 512^3
+// serial, cold cache: FX 53 -> 55 us (with 40 registers; 50 at 32, but the
+// spills cost more on short rows), IX 55 -> 29 us (a [L][9] buffer with the
+// pair as the minor index collided in 3 to 5 of 8 accesses); with the column
+// engine's changes the 512^3 evaluation 815 -> 758, the 128^3 one 57.2 -> 54.1 us.
+// threads per block of the row passes
+constexpr int ROW_THREADS(int lg) { return lg <= 7 ? 128 : 256; }
+template <int LG> struct RowShape {
+    static constexpr int L = 1 << LG, TPB = L / 8, NT = ROW_THREADS(LG), PB = NT / TPB;
+    static constexpr int S8 = LG / 3, REM = LG - 3 * S8, NS = S8 + (REM ? 1 : 0);
+    template <int S> __host__ __device__ static constexpr int lgr() { return S < S8 ? 3 : REM; }
+};
+template <typename T> __device__ __forceinline__ int row_at(int i) {
+    if constexpr (sizeof(T) == 4)
+        return i ^ (((i >> 4) & 3) | ((i >> 6) & 1) * 12);
+    else
+        return i ^ ((i >> 3) & 7);
+}
+// (a barrier per pair by number would reserve all 16 of a block and leave four
+// blocks per SM)
+template <int TPB> __device__ __forceinline__ void row_sync() {
+    if constexpr (TPB <= 32)
+        __syncwarp();
+    else
+        __syncthreads();
+}
+// this thread's share of the twiddles, in registers until the rows are requested
+template <typename C, int LG> struct RowTwiddles {
+    static constexpr int NT = RowShape<LG>::NT, N = (1 << LG) / NT;
+    C c[N];
+    __device__ __forceinline__ void load(const C *full) {
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-        const int j = t + u * (Sh::L / 8);
-        const int k = j & ((1 << lgNs) - 1);
+        for (int e = 0; e < N; ++e) {
+            const int i = threadIdx.x + e * NT;
+            const int lgNs = i < 8 ? 0 : (31 - __clz(i)) / 3 * 3;
+            const int lgr = LG - lgNs < 3 ? LG - lgNs : 3;
+            const int k = i & ((1 << lgNs) - 1), r = i >> lgNs;
+            c[e] = full[((r * k) << (LG - lgNs - lgr)) & ((1 << LG) - 1)];
+        }
+    }
+    __device__ __forceinline__ void store(C *tw) const {
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const int i = threadIdx.x + e * NT;
+            if (i >= 8) tw[i - 8] = c[e];
+        }
+    }
+};
+// stage S of thread t on its eight elements; w[u R + r] becomes output
+// row_out<S>(t, u, r)
+template <int LG, int S> __device__ __forceinline__ int row_out(int t, int u, int r) {
+    typedef RowShape<LG> Sh;
+    const int j = t + u * Sh::TPB;
+    const int k = j & ((1 << (3 * S)) - 1);
+    return ((j - k) << Sh::template lgr<S>()) + k + (r << (3 * S));
+}
+template <typename C, int LG, int S, bool INV>
+__device__ __forceinline__ void row_stage(C (&v)[8], int t, const C *tw) {
+    typedef RowShape<LG> Sh;
+    constexpr int R = 1 << Sh::template lgr<S>(), Ns = 1 << (3 * S);
+#pragma unroll
+    for (int u = 0; u < 8 / R; ++u) {
         C *w = v + u * R;
-        if constexpr (lgNs > 0) {
+        if constexpr (S > 0) {
+            const int k = (t + u * Sh::TPB) & (Ns - 1);
 #pragma unroll
             for (int r = 1; r < R; ++r) {
-                C tt = tw[((r * k) << (LG - lgNs - LGR)) & (Sh::L - 1)];
-                if (INV) tt.y = -tt.y;
-                w[r] = cmul(w[r], tt);
+                C c = tw[r * Ns + k - 8];  // stage S starts at Ns - 8
+                if (INV) c.y = -c.y;
+                w[r] = cmul(w[r], c);
             }
         }
-        if constexpr (R == 8) dft8<C, INV>(w);
-        if constexpr (R == 4) dft4<C, INV>(w[0], w[1], w[2], w[3]);
-        if constexpr (R == 2) dft2(w[0], w[1]);
-        const int base = ((j - k) << LGR) + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) buf[(base + (r << lgNs)) * (CB + 1) + b] = w[r];
+        dftR<C, R, INV>(w);
     }
 }
-// inputs of stage S for thread t: elements j + r L / R, j = t + u L / 8
-template <typename C, int LG, int S>
-__device__ __forceinline__ void stk_load(const C *buf, C (&v)[8], int t, int b) {
-    typedef ColShape<LG> Sh;
-    constexpr int LGR = S < Sh::S8 ? 3 : Sh::REM;
-    constexpr int R = 1 << LGR, NB = 8 / R;
+// row_at is linear over exclusive or and the bits of t, u and r are disjoint
+template <typename C, int LG, int S> __device__ __forceinline__ void row_load(const C *buf, C (&v)[8], int t) {
+    typedef RowShape<LG> Sh;
+    constexpr int R = 1 << Sh::template lgr<S>();
+    typedef decltype(v[0].x) T;
+    const int a = row_at<T>(t);
 #pragma unroll
-    for (int u = 0; u < NB; ++u)
+    for (int u = 0; u < 8 / R; ++u)
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[u * R + r] = buf[(t + u * (Sh::L / 8) + r * (Sh::L >> LGR)) * (CB + 1) + b];
+        for (int r = 0; r < R; ++r) v[u * R + r] = buf[a ^ row_at<T>(u * Sh::TPB + r * (Sh::L / R))];
 }
-// stages S .. NS-1 (stage S - 1 already stored); ends with a barrier
+template <typename C, int LG, int S> __device__ __forceinline__ void row_store(C *buf, const C (&v)[8], int t) {
+    typedef RowShape<LG> Sh;
+    constexpr int R = 1 << Sh::template lgr<S>();
+    typedef decltype(v[0].x) T;
+    const int a = row_at<T>(row_out<LG, S>(t, 0, 0));
+#pragma unroll
+    for (int u = 0; u < 8 / R; ++u)
+#pragma unroll
+        for (int r = 0; r < R; ++r) buf[a ^ row_at<T>(row_out<LG, S>(0, u, r))] = v[u * R + r];
+}
+// stages S .. NS - 1; v holds stage S - 1's outputs on entry and the last
+// stage's on return
 template <typename C, int LG, int S, bool INV>
-__device__ __forceinline__ void stk_from(C *buf, int t, int b, const C *tw) {
-    if constexpr (S < ColShape<LG>::NS) {
-        C v[8];
-        stk_load<C, LG, S>(buf, v, t, b);
-        __syncthreads();
-        stk_compute_store<C, LG, S, INV>(buf, v, t, b, tw);
-        __syncthreads();
-        stk_from<C, LG, S + 1, INV>(buf, t, b, tw);
+__device__ __forceinline__ void row_from(C *buf, C (&v)[8], int t, const C *tw) {
+    typedef RowShape<LG> Sh;
+    if constexpr (S < Sh::NS) {
+        if constexpr (S > 1) row_sync<Sh::TPB>();  // stage S - 1's loads are done
+        row_store<C, LG, S - 1>(buf, v, t);
+        row_sync<Sh::TPB>();
+        row_load<C, LG, S>(buf, v, t);
+        row_stage<C, LG, S, INV>(v, t, tw);
+        row_from<C, LG, S + 1, INV>(buf, v, t, tw);
     }
 }
 
 template <typename T, int LG>
-__global__ void __launch_bounds__(1 << LG) k_ix_s(DevPlan p) {
+__global__ void __launch_bounds__(ROW_THREADS(LG)) k_fx_r(DevPlan p) {
     typedef typename VecT<T>::T2 C;
-    typedef ColShape<LG> Sh;
+    typedef RowShape<LG> Sh;
+    constexpr int L = Sh::L, TPB = Sh::TPB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *buf = (C *)smem_raw;
-    C *tw = buf + Sh::L * (CB + 1);
-    for (int i = threadIdx.x; i < Sh::L; i += blockDim.x) tw[i] = ((const C *)p.tw[0])[i];
-    constexpr int TPB = Sh::L / 8;
+    C *tw = (C *)smem_raw;  // [L - 8], then one buffer [L] per pair
     const int b = threadIdx.x / TPB, t = threadIdx.x - b * TPB;
+    C *buf = tw + L + b * L;
+    RowTwiddles<C, LG> mytw;
+    mytw.load((const C *)p.tw[0]);
     const int Ly = p.L[1], Kx = p.Kx;
     const int lgHy = __ffs(Ly) - 2;
-    const int pr = blockIdx.x * CB + b;
+    const int pr = blockIdx.x * Sh::PB + b;
     const bool on = pr < p.n_row_pairs;
+    const int rp = on ? p.row_pairs[pr] : 0;
+    const int64_t row = (int64_t)(rp >> lgHy) * Ly + 2 * (rp & ((Ly >> 1) - 1));
     pdl_wait();
     pdl_trigger();
-    int64_t r0 = 0;
-    if (on) {
-        const int rp = p.row_pairs[pr];
-        r0 = ((int64_t)(rp >> lgHy) * Ly + 2 * (rp & ((Ly >> 1) - 1))) * Sh::L;
+    T *A = (T *)p.gridA + blockIdx.y * p.st_grid + row * L;
+    C v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const int x = t + r * TPB;
+        v[r] = on ? cmk(A[x], A[L + x]) : cmk(T(0), T(0));
     }
+    mytw.store(tw);
+    __syncthreads();  // twiddles; all of the pair's loads
+    if (on) {
+        typedef typename VecW<T>::V V;
+#pragma unroll
+        for (int i = 0; i < 8 / VecW<T>::W; ++i) {
+            ((V *)A)[t + i * TPB] = VecW<T>::zero();
+            ((V *)(A + L))[t + i * TPB] = VecW<T>::zero();
+        }
+    }
+    row_stage<C, LG, 0, false>(v, t, tw);
+    row_from<C, LG, 1, false>(buf, v, t, tw);
+    row_sync<TPB>();
+    // the split into the two rows' spectra pairs k with L - k
+    constexpr int LS = Sh::NS - 1, R = 1 << Sh::template lgr<LS>();
+#pragma unroll
+    for (int u = 0; u < 8 / R; ++u)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int o = t + row_out<LG, LS>(0, u, r);  // the last stage's outputs are in order
+            if (o < Kx || o > L - Kx) buf[row_at<T>(t) ^ row_at<T>(o - t)] = v[u * R + r];
+        }
+    row_sync<TPB>();
+    if (!on) return;
+    C *S1 = (C *)p.S1 + blockIdx.y * p.st_s1 + row * Kx;
+    for (int k = t; k < Kx; k += TPB) {
+        const C Z = buf[row_at<T>(k)];
+        const C Zc = cconj(buf[row_at<T>((L - k) & (L - 1))]);
+        S1[k] = cscale(cadd(Z, Zc), T(0.5));
+        S1[Kx + k] = cscale(cmul_mi(csub(Z, Zc)), T(0.5));  // (Z - Zc) / (2i)
+    }
+}
+
+template <typename T, int LG>
+__global__ void __launch_bounds__(ROW_THREADS(LG)) k_ix_r(DevPlan p) {
+    typedef typename VecT<T>::T2 C;
+    typedef RowShape<LG> Sh;
+    constexpr int L = Sh::L, TPB = Sh::TPB;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = (C *)smem_raw;
+    const int b = threadIdx.x / TPB, t = threadIdx.x - b * TPB;
+    C *buf = tw + L + b * L;
+    RowTwiddles<C, LG> mytw;
+    mytw.load((const C *)p.tw[0]);
+    const int Ly = p.L[1], Kx = p.Kx;
+    const int lgHy = __ffs(Ly) - 2;
+    const int pr = blockIdx.x * Sh::PB + b;
+    const bool on = pr < p.n_row_pairs;
+    const int rp = on ? p.row_pairs[pr] : 0;
+    const int64_t row = (int64_t)(rp >> lgHy) * Ly + 2 * (rp & ((Ly >> 1) - 1));
+    pdl_wait();
+    pdl_trigger();
     // stage 0 reads frequencies t + r L / 8 of the pair's complex spectrum
     // Y(k) = xa(k) + i xb(k), Y(L - k) = conj(xa(k)) + i conj(xb(k))
-    const C *S1 = (const C *)p.S1 + blockIdx.y * p.st_s1 + r0 / Sh::L * Kx;
+    const C *S1 = (const C *)p.S1 + blockIdx.y * p.st_s1 + row * Kx;
     C v[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -898,26 +1049,28 @@ __global__ void __launch_bounds__(1 << LG) k_ix_s(DevPlan p) {
             } else if (k < Kx) {
                 const C xa = S1[k], xb = S1[Kx + k];
                 y = cmk(xa.x - xb.y, xa.y + xb.x);
-            } else if (k > Sh::L - Kx) {
-                const C xa = S1[Sh::L - k], xb = S1[Kx + Sh::L - k];
+            } else if (k > L - Kx) {
+                const C xa = S1[L - k], xb = S1[Kx + L - k];
                 y = cmk(xa.x + xb.y, xb.x - xa.y);
             }
         }
         v[r] = y;
     }
+    mytw.store(tw);
     __syncthreads();  // twiddles
-    stk_compute_store<C, LG, 0, true>(buf, v, t, b, tw);
-    __syncthreads();
-    stk_from<C, LG, 1, true>(buf, t, b, tw);
+    row_stage<C, LG, 0, true>(v, t, tw);
+    row_from<C, LG, 1, true>(buf, v, t, tw);
     if (!on) return;
-    T *G = (T *)p.gridB + blockIdx.y * p.st_grid + r0;
+    T *G = (T *)p.gridB + blockIdx.y * p.st_grid + row * L;
+    constexpr int LS = Sh::NS - 1, R = 1 << Sh::template lgr<LS>();
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int x = t + r * TPB;
-        const C y = buf[x * (CB + 1) + b];
-        G[x] = y.x;
-        G[Sh::L + x] = y.y;
-    }
+    for (int u = 0; u < 8 / R; ++u)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int x = t + row_out<LG, LS>(0, u, r);
+            G[x] = v[u * R + r].x;
+            G[L + x] = v[u * R + r].y;
+        }
 }
 
 // ---------------------------------------------------------------- fused plane passes
@@ -1128,8 +1281,8 @@ __global__ void __launch_bounds__(512) k_yzy(DevPlan p, int ZC, int ZP) {
     const int col = g * CB + b;
     C *P = (C *)smem_raw;                 // [ny][ZP]
     C *tw = P + (size_t)ny * ZP;          // [L]
-    C *buf = tw + L + (size_t)g * L * (CB + 1);  // this group's exchange buffer
-    for (int i = threadIdx.x; i < L; i += blockDim.x) tw[i] = ((const C *)p.tw[1])[i];
+    C *buf = tw + L + (size_t)g * L * CB;  // this group's exchange buffer
+    col_twiddles<C, LG>(tw, (const C *)p.tw[1]);
     const int z0 = p.z0, nza = p.nz_act;
 
     // step 1 / 3 column: active plane zi of this CTA
@@ -1293,7 +1446,27 @@ template <typename K> static cudaError_t prep(K kern, size_t sm) {
 // the engine applies for 32 <= L <= 1024 and at least 8 stored x frequencies
 static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024 && p.Kx >= CB; }
 
+// row engine launch, 128 <= L <= 1024 (shorter rows share a wavefront between
+// pairs and are transformed by the fused plane passes anyway; at 1024 a pair is
+// 128 threads)
+static bool row_engine_ok(const DevPlan &p) { return p.L[0] >= 128 && p.L[0] <= 1024; }
+template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
+    typedef RowShape<LG> Sh;
+    if (p.n_row_pairs == 0) return cudaSuccess;
+    const size_t sm = (size_t)(Sh::PB + 1) * Sh::L * 2 * sizeof(T);
+    const cudaError_t e = prep(kern, sm);
+    if (e != cudaSuccess) return e;
+    const dim3 nb((unsigned)((p.n_row_pairs + Sh::PB - 1) / Sh::PB), (unsigned)p.ks);
+    const cudaError_t le = launch_k(kern, nb, Sh::NT, sm, s, p);
+    return le != cudaSuccess ? le : cudaGetLastError();
+}
 template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) {
+    if (row_engine_ok(p)) switch (__builtin_ctz(p.L[0])) {
+        case 7: return launch_rows<T, 7>(k_fx_r<T, 7>, p, s);
+        case 8: return launch_rows<T, 8>(k_fx_r<T, 8>, p, s);
+        case 9: return launch_rows<T, 9>(k_fx_r<T, 9>, p, s);
+        case 10: return launch_rows<T, 10>(k_fx_r<T, 10>, p, s);
+    }
     const size_t ce = 2 * sizeof(T);
     const int PB = row_batch(p.L[0], ce);
     const size_t sm = (2 * (size_t)p.L[0] * (PB + 1) + p.L[0]) * ce;
@@ -1304,13 +1477,11 @@ template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) 
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) {
-    // the compile-time inverse pays off for long rows (measured at 1024);
-    // short, latency-bound rows keep the runtime kernel
-    if (col_engine_ok(p, p.L[0]) && p.L[0] >= 512) {
-        if (p.n_row_pairs == 0) return cudaSuccess;
-        const size_t sm = ((size_t)p.L[0] * (CB + 1) + p.L[0]) * 2 * sizeof(T);
-        const dim3 nb((unsigned)((p.n_row_pairs + CB - 1) / CB), (unsigned)p.ks);
-        SLP_COL_DISPATCH(k_ix_s, T, __builtin_ctz(p.L[0]), nb, sm, s)
+    if (row_engine_ok(p)) switch (__builtin_ctz(p.L[0])) {
+        case 7: return launch_rows<T, 7>(k_ix_r<T, 7>, p, s);
+        case 8: return launch_rows<T, 8>(k_ix_r<T, 8>, p, s);
+        case 9: return launch_rows<T, 9>(k_ix_r<T, 9>, p, s);
+        case 10: return launch_rows<T, 10>(k_ix_r<T, 10>, p, s);
     }
     const size_t ce = 2 * sizeof(T);
     const int PB = row_batch(p.L[0], ce);
@@ -1324,7 +1495,7 @@ template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) 
 template <typename T> static cudaError_t fy_t(const DevPlan &p, cudaStream_t s) {
     if (col_engine_ok(p, p.L[1])) {
         if (p.nz_act == 0) return cudaSuccess;
-        const size_t sm = ((size_t)p.L[1] * (CB + 1) + p.L[1]) * 2 * sizeof(T);
+        const size_t sm = ((size_t)p.L[1] * CB + p.L[1]) * 2 * sizeof(T);
         const dim3 nb((unsigned)(p.nz_act * (p.Kx / CB)), (unsigned)p.ks);
         SLP_COL_DISPATCH2(k_fy_c, k_fy_c_long, T, __builtin_ctz(p.L[1]), nb, sm, s)
     }
@@ -1340,7 +1511,7 @@ template <typename T> static cudaError_t fy_t(const DevPlan &p, cudaStream_t s) 
 template <typename T> static cudaError_t iy_t(const DevPlan &p, cudaStream_t s) {
     if (col_engine_ok(p, p.L[1])) {
         if (p.nz_act == 0) return cudaSuccess;
-        const size_t sm = ((size_t)p.L[1] * (CB + 1) + p.L[1]) * 2 * sizeof(T);
+        const size_t sm = ((size_t)p.L[1] * CB + p.L[1]) * 2 * sizeof(T);
         const dim3 nb((unsigned)(p.nz_act * (p.Kx / CB)), (unsigned)p.ks);
         SLP_COL_DISPATCH2(k_iy_c, k_iy_c_long, T, __builtin_ctz(p.L[1]), nb, sm, s)
     }
@@ -1356,7 +1527,7 @@ template <typename T> static cudaError_t iy_t(const DevPlan &p, cudaStream_t s) 
 template <typename T> static cudaError_t fz_t(const DevPlan &p, cudaStream_t s) {
     if (col_engine_ok(p, p.L[2])) {
         if (p.nz_act == 0) return cudaSuccess;
-        const size_t sm = ((size_t)p.L[2] * (CB + 1) + p.L[2]) * 2 * sizeof(T);
+        const size_t sm = ((size_t)p.L[2] * CB + p.L[2]) * 2 * sizeof(T);
         const dim3 nb((unsigned)(p.n[1] * (p.Kx / CB)), (unsigned)p.ks);
         SLP_COL_DISPATCH(k_fz_c, T, __builtin_ctz(p.L[2]), nb, sm, s)
     }
@@ -1404,10 +1575,10 @@ template <typename T> static cudaError_t iyx_t(const DevPlan &p, cudaStream_t s)
 }
 
 // shared memory of one CTA of the fused column passes: P [ny][ZP], the
-// twiddles, G exchange buffers [L][CB + 1]
+// twiddles, G exchange buffers [L][CB]
 static size_t yzy_cta_smem(const DevPlan &p, int G, int ZP, size_t ce) {
     const size_t L = (size_t)p.L[1];
-    return ((size_t)p.n[1] * ZP + L + (size_t)G * L * (CB + 1)) * ce;
+    return ((size_t)p.n[1] * ZP + L + (size_t)G * L * CB) * ce;
 }
 template <typename K> static cudaError_t launch_yzy_cluster(K kern, const DevPlan &p, size_t sm, cudaStream_t s) {
     cudaError_t e = prep(kern, sm);
