@@ -50,18 +50,26 @@ template <> struct VecW<double> {
 };
 
 // ---------------------------------------------------------------- small DFTs
+// sums of complex numbers whose parts stay in place: one paired instruction in
+// FP32 (same rounding), since the passes are short of issue slots
+template <typename C> __device__ __forceinline__ C padd(C a, C b) { return cadd(a, b); }
+template <typename C> __device__ __forceinline__ C psub(C a, C b) { return csub(a, b); }
+template <> __device__ __forceinline__ float2 padd<float2>(float2 a, float2 b) { return __fadd2_rn(a, b); }
+template <> __device__ __forceinline__ float2 psub<float2>(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
 template <typename C> __device__ __forceinline__ void dft2(C &a, C &b) {
     const C t = a;
-    a = cadd(t, b);
-    b = csub(t, b);
+    a = padd(t, b);
+    b = psub(t, b);
 }
 
 template <typename C, bool INV> __device__ __forceinline__ void dft4(C &a, C &b, C &c, C &d) {
-    const C s0 = cadd(a, c), d0 = csub(a, c);
-    const C s1 = cadd(b, d), d1 = csub(b, d);
+    const C s0 = padd(a, c), d0 = psub(a, c);
+    const C s1 = padd(b, d), d1 = psub(b, d);
     const C r1 = INV ? cmul_pi(d1) : cmul_mi(d1);
-    a = cadd(s0, s1);
-    c = csub(s0, s1);
+    a = padd(s0, s1);
+    c = psub(s0, s1);
     b = cadd(d0, r1);
     d = csub(d0, r1);
 }
@@ -77,14 +85,14 @@ template <typename C, bool INV> __device__ __forceinline__ void dft8(C *v) {
     const C t1 = INV ? cmk(h * (o1.x - o1.y), h * (o1.x + o1.y)) : cmk(h * (o1.x + o1.y), h * (o1.y - o1.x));
     const C t2 = INV ? cmul_pi(o2) : cmul_mi(o2);
     const C t3 = INV ? cmk(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : cmk(h * (o3.y - o3.x), -h * (o3.x + o3.y));
-    v[0] = cadd(e0, o0);
-    v[4] = csub(e0, o0);
-    v[1] = cadd(e1, t1);
-    v[5] = csub(e1, t1);
+    v[0] = padd(e0, o0);
+    v[4] = psub(e0, o0);
+    v[1] = padd(e1, t1);
+    v[5] = psub(e1, t1);
     v[2] = cadd(e2, t2);
     v[6] = csub(e2, t2);
-    v[3] = cadd(e3, t3);
-    v[7] = csub(e3, t3);
+    v[3] = padd(e3, t3);
+    v[7] = psub(e3, t3);
 }
 
 template <typename C, int R, bool INV> __device__ __forceinline__ void dftR(C *v) {
@@ -701,7 +709,7 @@ __device__ __forceinline__ void k_fy_c_body(const DevPlan &p) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int y = col_idx<LG, 0>(t, r);
-        v[r] = ((y - iv.x) & (Sh::L - 1)) < iv.y ? S1[(int64_t)y * Kx] : cmk(T(0), T(0));
+        v[r] = ((y - iv.x) & (Sh::L - 1)) < iv.y ? S1[(unsigned)(y * Kx)] : cmk(T(0), T(0));
     }
     __syncthreads();  // twiddles
     col_stage<C, LG, 0, false>(v, t, tw);
@@ -710,10 +718,8 @@ __device__ __forceinline__ void k_fy_c_body(const DevPlan &p) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int k = col_freq<LG>(col_idx<LG, Sh::NS - 1>(t, r));
-        if (k < ny / 2)
-            S2[(int64_t)k * Kx] = v[r];
-        else if (k > Sh::L - ny / 2)
-            S2[(int64_t)(k - Sh::L + ny) * Kx] = v[r];
+        const int ky = k < Sh::L / 2 ? k : k - Sh::L;
+        if (abs(ky) < ny / 2) S2[(unsigned)((ky < 0 ? ky + ny : ky) * Kx)] = v[r];
     }
 }
 // at L <= 256 a block asks for 1024 / L blocks per SM (at most 64 registers);
@@ -807,12 +813,8 @@ __device__ __forceinline__ void k_iy_c_body(const DevPlan &p) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int k = col_freq<LG>(col_idx<LG, Sh::NS - 1>(t, r));
-        C x = cmk(T(0), T(0));
-        if (k < ny / 2)
-            x = S2[(int64_t)k * Kx];
-        else if (k > Sh::L - ny / 2)
-            x = S2[(int64_t)(k - Sh::L + ny) * Kx];
-        v[r] = x;
+        const int ky = k < Sh::L / 2 ? k : k - Sh::L;
+        v[r] = abs(ky) < ny / 2 ? S2[(unsigned)((ky < 0 ? ky + ny : ky) * Kx)] : cmk(T(0), T(0));
     }
     __syncthreads();  // twiddles
     col_stage<C, LG, Sh::NS - 1, true>(v, t, tw);
@@ -821,7 +823,7 @@ __device__ __forceinline__ void k_iy_c_body(const DevPlan &p) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int y = col_idx<LG, 0>(t, r);
-        if (((y - iv.x) & (Sh::L - 1)) < iv.y) S1[(int64_t)y * Kx] = v[r];
+        if (((y - iv.x) & (Sh::L - 1)) < iv.y) S1[(unsigned)(y * Kx)] = v[r];
     }
 }
 // at L <= 256 a block asks for 1024 / L blocks per SM (at most 64 registers);
