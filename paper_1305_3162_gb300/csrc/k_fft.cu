@@ -568,10 +568,11 @@ __global__ void __launch_bounds__(256) k_ix(DevPlan p, int PB) {
 // thread writes back exactly the positions it read, so a stage needs no
 // barrier between its read and its write.
 constexpr int CB = 8;
-// Register budget: blocks of L threads are asked to fit 1024 / L per SM (at
-// most 64 registers a thread) for L <= 256, and for the z pass at every L;
-// the y passes at L >= 512 use the variants without a minimum (`_long`).
-// Chosen by measurement on the 128^3 sphere and the 1024^3 cube.
+// Register budget: the y passes ask for 1024 / L blocks of L threads per SM (at
+// most 64 registers a thread) for L <= 256, the z pass for 1536 / L in FP32
+// (40 registers) and 1024 / L in FP64; the y passes at L >= 512 use the
+// variants without a minimum (`_long`).  Chosen by measurement on the 128^3
+// sphere, the 512^3 and the 1024^3 cube.
 
 template <int LG> struct ColShape {
     static constexpr int L = 1 << LG, S8 = LG / 3, REM = LG - 3 * S8, NS = S8 + (REM ? 1 : 0);
@@ -640,7 +641,7 @@ template <typename C, int LG, int S, bool INV> __device__ __forceinline__ void c
 // halves of the banks in every stage (rows of CB + 1 collide in one bank in all
 // but the last, which doubles those wavefronts).  With the twiddles by stage
 // and the constant offsets below, 512^3 serial: FY 39 -> 38, FZ 89 -> 74,
-// IY 42 -> 35 us, FZ with 75 % of its issue slots taken.
+// IY 42 -> 35 us; with paired sums and 32-bit offsets FY 34, IY 32 us.
 __device__ __forceinline__ int col_at(int p) { return (p ^ ((p >> 3) & 1)) * CB; }
 
 // col_at is linear over exclusive or, and element r of a task differs from
@@ -732,7 +733,7 @@ __global__ void __launch_bounds__(1 << LG) k_fy_c_long(DevPlan p) { k_fy_c_body<
 // FZ * D * IZ: row ky', columns kx0 .. kx0 + 8; the last forward stage, the
 // multiply and the first inverse stage share the same registers
 template <typename T, int LG>
-__global__ void __launch_bounds__(1 << LG, (1024 >> LG) > 0 ? (1024 >> LG) : 1) k_fz_c(DevPlan p) {
+__global__ void __launch_bounds__(1 << LG, LG < 10 ? ((sizeof(T) == 4 ? 1536 : 1024) >> LG) : 1) k_fz_c(DevPlan p) {
     typedef typename VecT<T>::T2 C;
     typedef ColShape<LG> Sh;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -745,7 +746,7 @@ __global__ void __launch_bounds__(1 << LG, (1024 >> LG) > 0 ? (1024 >> LG) : 1) 
     const int kp = blockIdx.x / ntile;
     const int kx0 = (blockIdx.x - kp * ntile) * CB;
     const int z0 = p.z0, nza = p.nz_act;
-    const int64_t zs = (int64_t)ny * Kx;
+    const unsigned zs = (unsigned)(ny * Kx);  // Lz zs < 2^32
     pdl_wait();
     pdl_trigger();
     C *S2 = (C *)p.S2 + blockIdx.y * p.st_s2 + (int64_t)kp * Kx + kx0 + b;
@@ -763,11 +764,16 @@ __global__ void __launch_bounds__(1 << LG, (1024 >> LG) > 0 ? (1024 >> LG) : 1) 
         const int z = col_idx<LG, 0>(t, r);
         v[r] = ((z - z0) & (Sh::L - 1)) < nza ? S2[z * zs] : cmk(T(0), T(0));
     }
-    // the multipliers of the elements this thread holds after the forward
-    // stages depend on its positions only: load them now, beside the pencil
+    __syncthreads();  // twiddles
+    col_stage<C, LG, 0, false>(v, t, tw);
+    col_forward_from<C, LG, 1>(buf, v, t, b, tw);
+    // the multipliers at this thread's positions are loaded here, not beside the
+    // pencil: with them out of the registers 48 warps fit on an SM in FP32
+    // instead of 32 (512^3 evaluation 733 -> 729 us, four states of a 256^3 one
+    // 316 -> 312 us; loaded first at the same 40 registers: 737 us)
     const int aky = kp < ny / 2 ? kp : ny - kp;
     const T *D = (const T *)p.Dtab + (int64_t)aky * Kx + kx0 + b;
-    const int64_t dz = (int64_t)(ny / 2) * Kx;
+    const unsigned dz = (unsigned)((ny / 2) * Kx);
     T dv[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -775,9 +781,6 @@ __global__ void __launch_bounds__(1 << LG, (1024 >> LG) > 0 ? (1024 >> LG) : 1) 
         const int akz = kz < Sh::L / 2 ? kz : Sh::L - kz;
         dv[r] = akz < nz / 2 ? D[akz * dz] : T(0);
     }
-    __syncthreads();  // twiddles
-    col_stage<C, LG, 0, false>(v, t, tw);
-    col_forward_from<C, LG, 1>(buf, v, t, b, tw);
 #pragma unroll
     for (int r = 0; r < 8; ++r) v[r] = cscale(v[r], dv[r]);
     col_stage<C, LG, Sh::NS - 1, true>(v, t, tw);
@@ -847,12 +850,11 @@ __global__ void __launch_bounds__(1 << LG) k_iy_c_long(DevPlan p) { k_iy_c_body<
 //   twiddles: [stage][r][k], read by consecutive k (stage s at 8^s - 8, L - 8
 //     entries in all); a thread requests its share of them and its row before
 //     it waits for either.
-// The passes are bound by the latency of their global reads (a third of the
-// cycles of FX, the largest share), not by shared memory any more.  FP32 512^3
-// serial, cold cache: FX 53 -> 55 us (with 40 registers; 50 at 32, but the
-// spills cost more on short rows), IX 55 -> 29 us (a [L][9] buffer with the
-// pair as the minor index collided in 3 to 5 of 8 accesses); with the column
-// engine's changes the 512^3 evaluation 815 -> 758, the 128^3 one 57.2 -> 54.1 us.
+// The passes are bound by the latency of their global reads, not by shared
+// memory any more.  FP32 512^3 serial, cold cache: FX 53 -> 33, IX 55 -> 29 us
+// (a [L][9] buffer with the pair as the minor index collided in 3 to 5 of 8
+// accesses); with the column engine's changes the 512^3 evaluation 815 -> 733,
+// the 128^3 one 57.2 -> 54.8 us.
 // threads per block of the row passes
 constexpr int ROW_THREADS(int lg) { return lg <= 7 ? 128 : 256; }
 template <int LG> struct RowShape {
