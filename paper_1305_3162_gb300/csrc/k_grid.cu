@@ -12,6 +12,8 @@
 // (smooth_phi) evaluated by NFFT): phi_i = sum_r g_r prod_q psi(u_{i,q} - r_q).
 // One CTA loads a tile plus halo of the grid into shared memory; one warp
 // per target.
+#include <type_traits>
+
 #include "dev_common.cuh"
 
 namespace slp {
@@ -742,24 +744,53 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
     constexpr int XE = G::XE;
     const int gxs = gx0 - XO;  // a multiple of 4 when TS is
     if (sizeof(T) == 4 && TS % 4 == 0 && gxs >= 0 && gxs + XE <= Lx) {
-        // rows of XE/4 aligned 16-byte vectors (the tile's x extent widened to XE)
-        constexpr int NV = XE / 4;
-        pipelined_copy<float4>(
-            TE * TE * NV,
-            [&](int i) {
-                const int v = i % NV, r = i / NV;
-                const int gy = (gy0 + r % TE) & (Ly - 1);
-                const int gz = (gz0 + r / TE) & (Lz - 1);
-                return ((const float4 *)((const float *)grid + ((int64_t)gz * Ly + gy) * Lx + gxs))[v];
-            },
-            [&](int i, float4 v) {
-                const int vv = i % NV, r = i / NV;
-                float *d = (float *)tile + (r / TE) * PS + (r % TE) * RS + 4 * vv;
-                d[0] = v.x;
-                d[1] = v.y;
-                d[2] = v.z;
-                d[3] = v.w;
-            });
+        // rows of XE/4 aligned 16-byte vectors (the tile's x extent widened to
+        // XE).  A thread keeps its vector of the row and steps RT rows at a time,
+        // so (y, z) follow by an addition and a carry.  The kernel is bound by
+        // issue slots and shared-memory wavefronts (512^3 cube, 240k targets: 69 us
+        // with divisions for each vector's load and store, 56M warp instructions
+        // and 61 registers; 62 us so, 50M and 32; the evaluation 729.6 -> 720.6,
+        // and 715.5 with the x values and the stores below)
+        constexpr int NV = XE / 4, RT = 256 / NV, STEPS = (TE * TE + RT - 1) / RT, BATCH = 4;
+        const int v = threadIdx.x % NV, r0 = threadIdx.x / NV;
+        int y = r0 % TE, z = r0 / TE;
+        const float *from = (const float *)grid + gxs + 4 * v;
+        float *to = (float *)tile + 4 * v;
+        if (r0 < RT) {
+#pragma unroll
+            for (int s0 = 0; s0 < STEPS; s0 += BATCH) {
+                float4 c[BATCH];
+                int at[BATCH];
+#pragma unroll
+                for (int e = 0; e < BATCH; ++e) {
+                    const bool in = s0 + e < STEPS && z < TE;
+                    at[e] = in ? z * PS + y * RS : -1;
+                    if (in) {
+                        const int gy = (gy0 + y) & (Ly - 1), gz = (gz0 + z) & (Lz - 1);
+                        c[e] = *(const float4 *)(from + (unsigned)((gz * Ly + gy) * Lx));  // at most 2^30 points
+                    }
+                    y += RT % TE;
+                    z += RT / TE;
+                    if (y >= TE) {
+                        y -= TE;
+                        ++z;
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < BATCH; ++e)
+                    if (at[e] >= 0) {
+                        // four rows' vectors share a bank group: each starts at
+                        // another element
+                        float *d = to + at[e];
+                        const float q0 = v & 1 ? c[e].y : c[e].x, q1 = v & 1 ? c[e].z : c[e].y;
+                        const float q2 = v & 1 ? c[e].w : c[e].z, q3 = v & 1 ? c[e].x : c[e].w;
+                        d[v & 3] = v & 2 ? q2 : q0;
+                        d[(v + 1) & 3] = v & 2 ? q3 : q1;
+                        d[(v + 2) & 3] = v & 2 ? q0 : q2;
+                        d[(v + 3) & 3] = v & 2 ? q1 : q3;
+                    }
+            }
+        }
     } else {
         pipelined_copy<T>(
             TE * TE * TE,
@@ -793,6 +824,19 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
         if (!ok) set_error(p.err, DEV_ERR_BAD_ITEM);
         const T *w = wv + t * GW;
         const T *base = tile + (ok ? lz * PS + ly * RS + lx : 0) + XO;
+        // the x values, the same for every lane: two or four per load in FP32 (in
+        // FP64 held values cost more: the 8x8 cube 78.6 us with loads, 81 without)
+        T wx[W];
+        if constexpr (sizeof(T) == 4) {
+            typedef typename std::conditional<W % 4 == 0, float4, float2>::type WV;
+            constexpr int WN = sizeof(WV) / sizeof(float);
+#pragma unroll
+            for (int ix = 0; ix < W; ix += WN) {
+                const WV v = *(const WV *)(w + ix);
+#pragma unroll
+                for (int e = 0; e < WN; ++e) wx[ix + e] = ((const float *)&v)[e];
+            }
+        }
         T acc = T(0);
 #pragma unroll
         for (int rep = 0; rep < (W * W + 31) / 32; ++rep) {
@@ -802,7 +846,7 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
                 const T *row = base + iz * PS + iy * RS;
                 T s = T(0);
 #pragma unroll
-                for (int ix = 0; ix < W; ++ix) s += row[ix] * w[ix];
+                for (int ix = 0; ix < W; ++ix) s += row[ix] * (sizeof(T) == 4 ? wx[ix] : w[ix]);
                 acc += s * w[2 * W + iz] * w[W + iy];
             }
         }
