@@ -505,11 +505,11 @@ def _potential_config(slp, args, flush, n, steps, warmup, prec=32, tol=1e-5, n_s
                 "tolerance": tol, "rel_l2": rel, "rel_l2_phi1": rel1,
                 "parity_nodes": int(sel.size), "parity_ok": ok,
                 "hedgehog_l2": l2, "hedgehog_h1_semi": h1, "setup_s": round(t_setup, 2),
-                "roofline": {"kernel": "phi_1 solve (k_cg_step, k_fem_residual, k_fem_load)",
+                "roofline": {"kernel": "phi_1 solve (k_cg_solve, or k_cg_step and k_fem_residual; k_fem_load)",
                              "bound": "hbm", "achieved": achieved, "peak": float(peaks["hbm_gbs"]),
                              "unit": "GB/s", "frac": achieved / float(peaks["hbm_gbs"]), "traffic": None,
                              "bytes_per_inner_step": it_bytes, "peak_source": peak_src,
-                             "note": "working set L2-resident at this size"}}
+                             "note": "working set on chip at this size (rows in registers, the matrix in L2): a step is bound by the exchange between blocks"}}
     finally:
         slp.slp_potential_destroy(pot)
 

@@ -747,10 +747,10 @@ __global__ void __launch_bounds__(256) k_gather(DevPlan p, T *__restrict__ phi) 
         // rows of XE/4 aligned 16-byte vectors (the tile's x extent widened to
         // XE).  A thread keeps its vector of the row and steps RT rows at a time,
         // so (y, z) follow by an addition and a carry.  The kernel is bound by
-        // issue slots and shared-memory wavefronts (512^3 cube, 240k targets: 69 us
+        // issue slots and shared-memory wavefronts (512^3 cube, 240k targets: 68 us
         // with divisions for each vector's load and store, 56M warp instructions
-        // and 61 registers; 62 us so, 50M and 32; the evaluation 729.6 -> 720.6,
-        // and 715.5 with the x values and the stores below)
+        // and 61 registers; 62 us so, 50M and 32, and 54 us with the x values and
+        // the stores below; the evaluation 729.6 -> 720.6 -> 715.5)
         constexpr int NV = XE / 4, RT = 256 / NV, STEPS = (TE * TE + RT - 1) / RT, BATCH = 4;
         const int v = threadIdx.x % NV, r0 = threadIdx.x / NV;
         int y = r0 % TE, z = r0 / TE;
