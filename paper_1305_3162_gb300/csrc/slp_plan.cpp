@@ -715,6 +715,19 @@ void tile_items(const std::vector<double> &grid, const std::vector<uint64_t> &ke
     }
 }
 
+// FP64 probes over the volume that leave fewer than four in a tile of 4^3 cells
+// are gathered from tiles of 2^3: a halo is staged for so few of them, and it is
+// the larger at 4^3 (17^3 against 15^3 points at m = 7).  500 probes in the
+// level-2 sphere at 128^3: 197 -> 176 us, in the level-3 one 220 -> 198.  (For the
+// vertices of coarse meshes neither is the better one: level-3 sphere 141 and
+// 147 us, cube7 122 and 113.)
+bool sparse_tiles(const slp_plan_s &p, const std::vector<double> &grid, const std::vector<uint64_t> &keys, int64_t n, int ts) {
+    if (p.prec != 64 || ts != 4) return false;
+    std::vector<slp::TileItem> tiles;
+    tile_items(grid, keys, n, ts, (int)std::min<int64_t>(n, 1 << 30), tiles);
+    return n < 4 * (int64_t)tiles.size();
+}
+
 // Cell groups of each spread item (runs of one cell, at most SPREAD_GMAX
 // sources; the sort makes a cell's sources contiguous), dealt largest first to
 // SPREAD_WARPS lists, each group to the list with the least work so far (work
@@ -2135,7 +2148,9 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
     std::vector<int32_t> perm;
     std::vector<double> grid;
     std::vector<uint64_t> keys;
-    sort_points(p, pts, n, p.TSg, perm, grid, keys);
+    int ts = p.TSg;
+    sort_points(p, pts, n, ts, perm, grid, keys);
+    if (sparse_tiles(p, grid, keys, n, ts)) sort_points(p, pts, n, ts = 2, perm, grid, keys);
     // every probe's window rows must lie in the region the transforms compute
     {
         const int Ly = p.L[1], Lz = p.L[2], m = p.m;
@@ -2155,7 +2170,7 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
         }
     }
     std::vector<slp::TileItem> items;
-    tile_items(grid, keys, n, p.TSg, p.gather_chunk, items);
+    tile_items(grid, keys, n, ts, p.gather_chunk, items);
     std::stable_sort(items.begin(), items.end(),
                      [](const slp::TileItem &a, const slp::TileItem &b) { return a.end - a.begin > b.end - b.begin; });
     auto alloc_up = [&](void **dst, const void *src, size_t bytes) -> slp_status {
@@ -2172,6 +2187,7 @@ template <typename T> slp_status probe_build(slp_plan_s &p, const double *pts, i
     slp::DevPlan v = p.dp;
     v.N = n;
     v.ks = 1;
+    v.TSg = ts;
     v.wtab64_tgt = nullptr;  // the plan's target window table does not cover the probes
     std::vector<T4> tg(n);
     for (int64_t i = 0; i < n; ++i) {
