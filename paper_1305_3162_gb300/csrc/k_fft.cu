@@ -1453,7 +1453,14 @@ static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024
 // row engine launch, 128 <= L <= 1024 (shorter rows share a wavefront between
 // pairs and are transformed by the fused plane passes anyway; at 1024 a pair is
 // 128 threads)
-static bool row_engine_ok(const DevPlan &p) { return p.L[0] >= 128 && p.L[0] <= 1024; }
+// FP64 rows of 128 behind a gridding product (triangle integrals, deterministic
+// spread) keep the staged kernels: level-3 sphere at 128^3, deterministic, 178 us
+// an evaluation against 261, cube7 with triangles 130 against 193; behind the
+// spread kernels the row engine is the better one (157 against 133 us).
+static bool row_engine_ok(const DevPlan &p) {
+    if (p.prec == 64 && p.L[0] == 128 && p.am_rowptr) return false;
+    return p.L[0] >= 128 && p.L[0] <= 1024;
+}
 template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
     typedef RowShape<LG> Sh;
     if (p.n_row_pairs == 0) return cudaSuccess;
