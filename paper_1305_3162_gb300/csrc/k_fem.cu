@@ -957,8 +957,10 @@ cudaError_t solve_blocks(const FemDev &d, int *blocks) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    // the limit belongs to the kernel, which every potential of the process that
+    // runs it shares: always the same one, whatever this potential needs
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute((const void *)solve_kernel(d), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem(d));
+        e = cudaFuncSetAttribute((const void *)solve_kernel(d), cudaFuncAttributeMaxDynamicSharedMemorySize, SOLVE_SMEM);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, solve_kernel(d), SNT, solve_smem(d));
     *blocks = coop ? sms * per : 0;

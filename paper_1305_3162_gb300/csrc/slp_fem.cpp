@@ -584,7 +584,7 @@ slp_status build_parts(slp_potential_s &P, const FemHost &H, const std::vector<d
     d.near_max = near_max;
     d.solve_reg = rpt <= 2 && wmax <= slp::SOLVE_REG_W;
     int fit = 0;
-    if (slp::solve_smem(d) > 200 * 1024 || slp::solve_blocks(d, &fit) != cudaSuccess || fit < parts) {
+    if (slp::solve_smem(d) > slp::SOLVE_SMEM || slp::solve_blocks(d, &fit) != cudaSuccess || fit < parts) {
         cudaGetLastError();
         d.parts = 0;
         return SLP_OK;
