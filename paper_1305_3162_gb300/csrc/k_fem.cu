@@ -532,8 +532,9 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
 // e + 1, which that block wrote after it had read its records of e, so two
 // copies suffice.  All blocks add the sums in one order and hold the same
 // scalars.  The launch is cooperative (all blocks resident); every wait is
-// bounded, and a block that gives up sets `stalled` and leaves, after which the
-// others' waits run out as well.
+// bounded, a thread whose wait has run out starts no other, and a block that
+// gives up sets `stalled` and leaves, after which the others' waits run out as
+// well.
 //
 // The system is scaled by its diagonal (S_ij / sqrt(S_ii S_jj), unit
 // diagonal).  The preconditioner adds to Jacobi's (the identity here) a coarse
@@ -694,7 +695,7 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
             if (tid < P) lost = !wait_record((e & 1 ? in1 : in0) + tid, e, sums);
 #pragma unroll
             for (int i = 0; i < HB; ++i)
-                if (i * SNT + hid < nh) lost = !wait_record(mine + i * SNT + hid, e, v[i]) || lost;
+                if (i * SNT + hid < nh) lost = lost || !wait_record(mine + i * SNT + hid, e, v[i]);
             float sum[2] = {0.f, 0.f}, wc = 0.f;
             if (tid < P) {
                 sum[0] = __uint_as_float(sums.x);
@@ -757,7 +758,10 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
             }
             for (int h = HB * SNT + hid; h < nh; h += SNT) {
                 uint4 vh;
-                lost = !wait_record(mine + h, e, vh) || lost;
+                if (lost || !wait_record(mine + h, e, vh)) {
+                    lost = true;
+                    break;
+                }
                 s_u[d.rp + h] = __uint_as_float(vh.x) -
                                 alpha * (__uint_as_float(vh.y) + beta * __uint_as_float(vh.z)) +
                                 d.halo_z[h0 + h] * s_ec[d.halo_near[h0 + h]];
@@ -811,7 +815,10 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
         bool lost = false;
         for (int h = tid; h < nh; h += SNT) {
             uint4 vh;
-            lost = !wait_record((e & 1 ? rec1 : rec0) + h, e, vh) || lost;
+            if (!wait_record((e & 1 ? rec1 : rec0) + h, e, vh)) {
+                lost = true;
+                break;
+            }
             s_x[d.rp + h] = __longlong_as_double((long long)((unsigned long long)vh.x | (unsigned long long)vh.y << 32));
         }
         __syncthreads();
