@@ -295,7 +295,7 @@ slp_status slp_probe_destroy(slp_probe_t probe);
  * of the free nodes.
  * Computation (slp_potential_eval): b = B m (in the plan's precision);
  * phi_1 by iterative refinement on the device: preconditioned conjugate
- * gradients in FP32 (Jacobi and, up to about 0.9M free nodes, one coarse
+ * gradients in FP32 (Jacobi and, up to about 0.78M free nodes, one coarse
  * unknown per block of rows) cut the residual of the current correction
  * equation by 1e-4, the correction joins the FP64 solution and the residual
  * b - S x is recomputed in FP64, until |b - S x| <= cg_tolerance |b|;

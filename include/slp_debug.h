@@ -130,6 +130,18 @@ slp_status slp_debug_fem_assemble(const double *nodes, int64_t n_nodes, const in
                                   int64_t *s_ptr, int32_t *s_col, double *s_val, int64_t *b_ptr, int32_t *b_col,
                                   double *b_val);
 
+/* slp_potential_create with a choice of the phi_1 solver: most_parts < 0 as
+ * there; 0 the solve graph (a launch per inner step), which otherwise only
+ * systems too large for one launch take; n > 0 the one-launch solve with at
+ * most n blocks, so that a moderate mesh reaches the variants with many rows per
+ * thread (the graph where n blocks cannot hold the system). */
+slp_status slp_debug_potential_create(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
+                                      double tolerance, const slp_plan_opts *opts, double cg_tolerance,
+                                      int cg_max_iterations, int most_parts, slp_potential_t *out);
+/* The solver a potential got: the one-launch solve's blocks and rows per
+ * thread, both 0 for the solve graph. */
+slp_status slp_debug_potential_solver(slp_potential_t pot, int *parts, int *rows_per_thread);
+
 #ifdef __cplusplus
 }
 #endif

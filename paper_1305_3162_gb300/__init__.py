@@ -153,7 +153,7 @@ EXPORTED = ["slp_default_opts", "slp_plan", "slp_eval", "slp_eval_states", "slp_
             "slp_check", "slp_destroy", "slp_status_string", "slp_last_error",
             "slp_debug_run", "slp_debug_copy", "slp_debug_buffer_bytes", "slp_debug_host_count",
             "slp_debug_host_array", "slp_debug_window", "slp_debug_window_hat", "slp_debug_profile",
-            "slp_debug_timeline", "slp_debug_fem_assemble",
+            "slp_debug_timeline", "slp_debug_fem_assemble", "slp_debug_potential_create", "slp_debug_potential_solver",
             "slp_debug_stage_name", "slp_eval_direct_static", "slp_batch_create", "slp_batch_run",
             "slp_batch_query", "slp_batch_destroy", "slp_eval_batched", "slp_plan_autotune", "slp_server_default_opts",
             "slp_server_create", "slp_server_submit", "slp_server_status", "slp_server_wait", "slp_server_cancel",
@@ -191,6 +191,10 @@ def load():
         "slp_potential_create": ([ctypes.POINTER(ctypes.c_double), I64, ctypes.POINTER(ctypes.c_int32), I64,
                                   ctypes.c_double, ctypes.POINTER(slp_plan_opts), ctypes.c_double, ctypes.c_int,
                                   ctypes.POINTER(vp)], St),
+        "slp_debug_potential_create": ([ctypes.POINTER(ctypes.c_double), I64, ctypes.POINTER(ctypes.c_int32), I64,
+                                        ctypes.c_double, ctypes.POINTER(slp_plan_opts), ctypes.c_double, ctypes.c_int,
+                                        ctypes.c_int, ctypes.POINTER(vp)], St),
+        "slp_debug_potential_solver": ([vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)], St),
         "slp_potential_eval": ([vp, vp, vp, vp, vp], St),
         "slp_potential_query": ([vp, ctypes.POINTER(slp_potential_info)], St),
         "slp_potential_destroy": ([vp], St),
@@ -369,6 +373,28 @@ def slp_potential_create(nodes, tets, tolerance: float, opts: slp_plan_opts | No
                                        float(tolerance), ctypes.byref(o), float(cg_tolerance), int(cg_max_iterations),
                                        ctypes.byref(out)), "slp_potential_create")
     return out
+
+
+def slp_debug_potential_create(nodes, tets, tolerance: float, most_parts: int, opts: slp_plan_opts | None = None,
+                               cg_tolerance: float = 0.0, cg_max_iterations: int = 0):
+    """slp_potential_create with a choice of the phi_1 solver (include/slp_debug.h)."""
+    X = np.ascontiguousarray(nodes, dtype=np.float64)
+    K = np.ascontiguousarray(tets, dtype=np.int32)
+    out = ctypes.c_void_p()
+    o = opts if opts is not None else slp_default_opts()
+    _check(load().slp_debug_potential_create(X.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), X.shape[0],
+                                             K.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), K.shape[0],
+                                             float(tolerance), ctypes.byref(o), float(cg_tolerance),
+                                             int(cg_max_iterations), int(most_parts), ctypes.byref(out)),
+           "slp_debug_potential_create")
+    return out
+
+
+def slp_debug_potential_solver(pot) -> tuple:
+    """(blocks, rows per thread) of the one-launch solve, (0, 0) for the solve graph."""
+    a, b = ctypes.c_int(), ctypes.c_int()
+    _check(load().slp_debug_potential_solver(pot, ctypes.byref(a), ctypes.byref(b)), "slp_debug_potential_solver")
+    return a.value, b.value
 
 
 def slp_debug_fem_assemble(nodes, tets) -> dict:

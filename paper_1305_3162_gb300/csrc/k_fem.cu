@@ -20,7 +20,7 @@
 //   beta_{k+1} = gamma_{k+1} / gamma_k,
 //   alpha_{k+1} = gamma_{k+1} / (delta_{k+1} - beta_{k+1} gamma_{k+1} / alpha_k),
 // which needs both dot products at one point of the step.  Systems of up to
-// SOLVE_THREADS 12 rows a block (0.9M free nodes) are solved in one launch
+// SOLVE_THREADS 10 rows a block (0.78M free nodes) are solved in one launch
 // (k_cg_solve, further down, with a better preconditioner); for larger ones a
 // launch does a step: every vector update is per row, and u_{k+1} at the columns the
 // product gathers is formed there from r_k, w_k and s_{k-1}, which a row
@@ -551,7 +551,13 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
 // Measured, phi_1 (load, solve and all corrections): ball n = 16 672 -> 319 us,
 // n = 32 2155 -> 760 us (5.2 us a step: about 2.2 exchange, 0.9 product, the
 // rest the coarse correction, sums and barriers), n = 48 7600 -> 5600 us (its
-// matrix no longer fits the registers).
+// matrix no longer fits the registers).  The line to the launch chain: a step is
+// the slower here from n = 44 on (its matrix comes from L2 to half as many warps),
+// but half as many steps are needed.  Chain and one launch, ms: n = 48 (436k
+// rows) 8.2 and 5.8, n = 52 (555k) 10.0 and 7.9, n = 56 (693k, ten rows a
+// thread) 15.1 and 13.4 to 14.3, n = 58 (771k) 16.2 and 14.0; with twelve rows a
+// thread, which spill twice as much, 15 to 16.3 and 15.8 to 18.0, and 19.9 and
+// 23.5 at n = 60 (853k).
 constexpr int SNT = SOLVE_THREADS;
 constexpr int SNW = SNT / 32;
 constexpr int HB = 2;                  // halo records a thread reads at once
@@ -950,7 +956,7 @@ SolveKernel solve_kernel(const FemDev &d) {
         case 2: return k_cg_solve<2, false>;
         case 4: return k_cg_solve<4, false>;
         case 8: return k_cg_solve<8, false>;
-        default: return k_cg_solve<12, false>;
+        default: return k_cg_solve<10, false>;
     }
 }
 }  // namespace

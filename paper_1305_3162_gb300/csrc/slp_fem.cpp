@@ -51,6 +51,7 @@ struct slp_potential_s {
     double cg_tol = 0.0;
     int64_t last_iter = -1, last_outer = 0;
     double last_res = 0.0;
+    int most_parts = -1;  // of the one-launch solve: -1 automatic, 0 none (the solve graph)
     std::vector<void *> allocs;
 };
 
@@ -478,7 +479,9 @@ slp_status build_parts(slp_potential_s &P, const FemHost &H, const std::vector<d
     int sms = 0;
     FTRY(cu(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P.device), "device"));
     // a block per SM; small systems fewer, at least 128 rows each
-    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, slp::SOLVE_PARTS), (nf + 127) / 128));
+    int parts = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, slp::SOLVE_PARTS), (nf + 127) / 128));
+    if (P.most_parts >= 0) parts = std::min(parts, P.most_parts);
+    if (parts == 0) return SLP_OK;
     const int64_t most = (nf + parts - 1) / parts;
     int rpt = 0;
     for (int k : slp::SOLVE_RPT)
@@ -779,9 +782,9 @@ slp_status build(slp_potential_s &P, const double *X, int64_t N, const int32_t *
 
 extern "C" {
 
-slp_status slp_potential_create(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
-                                double tolerance, const slp_plan_opts *opts, double cg_tolerance,
-                                int cg_max_iterations, slp_potential_t *out) {
+slp_status slp_debug_potential_create(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
+                                      double tolerance, const slp_plan_opts *opts, double cg_tolerance,
+                                      int cg_max_iterations, int most_parts, slp_potential_t *out) {
     if (!out) return slp_fail(SLP_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     if (!nodes || !tets || n_nodes < 4 || n_tets < 1)
@@ -797,12 +800,27 @@ slp_status slp_potential_create(const double *nodes, int64_t n_nodes, const int3
     P->n_tets = n_tets;
     P->cg_tol = cg_tolerance > 0.0 ? cg_tolerance : std::max(1e-2 * tolerance, 1e-14);
     P->d.max_iter = cg_max_iterations > 0 ? cg_max_iterations : 10000;
+    P->most_parts = most_parts;
     const slp_status st = build(*P, nodes, n_nodes, tets, n_tets, tolerance, opts);
     if (st != SLP_OK) {
         release(P);
         return st;
     }
     *out = P;
+    return SLP_OK;
+}
+
+slp_status slp_potential_create(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
+                                double tolerance, const slp_plan_opts *opts, double cg_tolerance,
+                                int cg_max_iterations, slp_potential_t *out) {
+    return slp_debug_potential_create(nodes, n_nodes, tets, n_tets, tolerance, opts, cg_tolerance, cg_max_iterations,
+                                      -1, out);
+}
+
+slp_status slp_debug_potential_solver(slp_potential_t P, int *parts, int *rows_per_thread) {
+    if (!P) return slp_fail(SLP_ERR_INVALID_ARG, "potential is NULL");
+    if (parts) *parts = P->d.parts;
+    if (rows_per_thread) *rows_per_thread = P->d.parts > 0 ? P->d.rpt : 0;
     return SLP_OK;
 }
 

@@ -127,7 +127,7 @@ struct FemDev {
 constexpr int FEM_THREADS = 256;
 constexpr int SOLVE_THREADS = 512;  // threads of a block of the one-launch solve
 constexpr int SOLVE_PARTS = 256;    // blocks at most (a thread reads one block's sums)
-constexpr int SOLVE_RPT[] = {1, 2, 4, 8, 12};  // rows per thread it is compiled for
+constexpr int SOLVE_RPT[] = {1, 2, 4, 8, 10};  // rows per thread it is compiled for
 constexpr int SOLVE_SMEM = 200 * 1024;  // bytes of dynamic shared memory at most
 constexpr int SOLVE_REG_W = 16;     // most off-diagonal entries of a row kept in registers (rpt <= 2)
 constexpr int FEM_CHUNK = 16;       // inner launches per pass of the inner loop (even: parities repeat)
