@@ -113,7 +113,14 @@ typedef struct {
 
 typedef struct {
     int precision;        /* 32 (FP32 spread/FFT/gather/near field) or 64 */
-    int grid[3];          /* oversampled FFT grid per axis (power of two, 8..1024); 0 = auto */
+    int grid[3];          /* oversampled FFT grid per axis (power of two, 8..1024); 0 = auto: about
+                             2 sqrt(sources + targets) cells across the body, except that a point plan
+                             with all three 0 and kernel_mode AUTO or RADIAL takes the grid whose
+                             evaluation is estimated cheapest, and its kernel split then spends 0.3 of
+                             the tolerance.  Where the grid by points cannot carry the radial kernel,
+                             allow_grid_raise = 0 refuses the plan as for a given grid, and with AUTO
+                             an FP64 mesh of at most 2^24 pairs and a tolerance below 1e-9 stays on
+                             that grid with the separable kernel. */
     int m;                /* Kaiser-Bessel half-width in grid cells; 0 = from the tolerance */
     int kernel_mode;      /* SLP_KERNEL_* */
     int near_mode;        /* SLP_NEAR_* */

@@ -456,6 +456,25 @@ bool cheapest_grid(const slp_plan_s &p, double c, int out[3]) {
     return best < 1e300;
 }
 
+// The automatic axes (L < 0) by the number of points: equal spacing at about
+// (Q + N)^(1/2) cells across the body.
+void grid_by_points(const slp_plan_s &p, int L[3]) {
+    const double target_cells = std::max(16.0, 2.0 * std::sqrt((double)(p.Q + p.N)));
+    const double dmax = std::max(p.D[0], std::max(p.D[1], p.D[2]));
+    for (int d = 0; d < 3; ++d) {
+        if (L[d] > 0) continue;
+        // cells of the oversampled grid across the period ~ 2.3x the body
+        double want = target_cells * (p.D[d] + p.diam) / (dmax + p.diam) * 1.0;
+        int v = 16;
+        while (v < want && v < 1024) v <<= 1;
+        L[d] = v;
+    }
+}
+
+// Tolerance below which AUTO keeps a small FP64 mesh on the separable kernel
+// (choose_parameters).
+constexpr double SEPARABLE_TOL = 1e-9;
+
 slp_status choose_parameters(slp_plan_s &p) {
     // bounding box and enclosing-ball diameter of targets (sources are convex
     // combinations of targets, so they lie inside both)
@@ -497,10 +516,28 @@ slp_status choose_parameters(slp_plan_s &p) {
             return fail(SLP_ERR_INVALID_ARG, "grid[%d] = %d must be a power of two in [8, 1024]", d, L[d]);
     }
     int mode = p.opts.kernel_mode;
+    const bool separable_size = p.prec == 64 && (double)p.Q * (double)p.N <= (double)(1 << 24);
     // an automatic grid for the radial kernel (point plans): sized by cost, with
     // a smaller share of the tolerance for the kernel split (AUTO_SPLIT)
-    const bool by_cost = L[0] < 0 && L[1] < 0 && L[2] < 0 && !p.opts.integration &&
-                         (mode == SLP_KERNEL_AUTO || mode == SLP_KERNEL_RADIAL);
+    bool by_cost = L[0] < 0 && L[1] < 0 && L[2] < 0 && !p.opts.integration &&
+                   (mode == SLP_KERNEL_AUTO || mode == SLP_KERNEL_RADIAL);
+    if (by_cost) {
+        // Where the grid by points cannot carry the radial kernel: a plan that may
+        // not raise its grid stays refused, and a small FP64 mesh whose tolerance is
+        // below SEPARABLE_TOL stays on that grid with the separable kernel, which has
+        // no split error (1e-16 where the radial kernel spends its share of the
+        // tolerance) and transforms a grid of half or a quarter of the points per
+        // axis.  Evaluations with one point a triangle, us, radial and separable:
+        // 42 vertices 68 and 51, 56 of a cube 67 and 51, 252 of a plate 73 and 61,
+        // 119 of a torus 83 and 60 at 1e-10; 119 and 52, 119 and 52, 170 and 66, 253
+        // and 62 at 1e-13.  Looser tolerances take the radial kernel
+        // at every size (the torus 82 at 1e-9).
+        int Lp[3] = {-1, -1, -1};
+        grid_by_points(p, Lp);
+        const int np[3] = {Lp[0] / 2, Lp[1] / 2, Lp[2] / 2};
+        if (!radial_feasible(p, np, std::sqrt(2.0 * std::log(1.0 / std::min(0.1, p.tol * KFAC)))))
+            by_cost = mode == SLP_KERNEL_AUTO && separable_size ? p.tol >= SEPARABLE_TOL : p.opts.allow_grid_raise != 0;
+    }
     p.split_share = by_cost ? AUTO_SPLIT : 1.0;
     double tk = std::min(0.1, p.tol * p.split_share * KFAC);
     double c = std::sqrt(2.0 * std::log(1.0 / tk));
@@ -510,25 +547,13 @@ slp_status choose_parameters(slp_plan_s &p) {
         c = std::sqrt(2.0 * std::log(1.0 / tk));
     }
     p.c_band = c;
-    if (L[0] < 0 || L[1] < 0 || L[2] < 0) {
-        // automatic: equal spacing at about (Q + N)^(1/2) cells across the body
-        const double target_cells = std::max(16.0, 2.0 * std::sqrt((double)(p.Q + p.N)));
-        const double dmax = std::max(p.D[0], std::max(p.D[1], p.D[2]));
-        for (int d = 0; d < 3; ++d) {
-            if (L[d] > 0) continue;
-            // cells of the oversampled grid across the period ~ 2.3x the body
-            double want = target_cells * (p.D[d] + p.diam) / (dmax + p.diam) * 1.0;
-            int v = 16;
-            while (v < want && v < 1024) v <<= 1;
-            L[d] = v;
-        }
-    }
+    grid_by_points(p, L);
     int nreq[3] = {L[0] / 2, L[1] / 2, L[2] / 2};
 
     if (mode == SLP_KERNEL_AUTO) {
         if (radial_feasible(p, nreq, c))
             mode = SLP_KERNEL_RADIAL;
-        else if (p.prec == 64 && (double)p.Q * (double)p.N <= (double)(1 << 24))
+        else if (separable_size)
             mode = SLP_KERNEL_SEPARABLE;  // FP64 only: in FP32 the all-pairs difference loses digits
         else if (p.opts.allow_grid_raise)
             mode = -SLP_KERNEL_RADIAL;  // radial after raising the grid
