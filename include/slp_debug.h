@@ -37,7 +37,8 @@ enum {
     SLP_BUF_GRID_B = 2,   /* [Lz][Ly][Lx] */
     SLP_BUF_S1 = 3,       /* complex [Lz][Ly][n_x/2] */
     SLP_BUF_S2 = 4,       /* complex [Lz][n_y][n_x/2] */
-    SLP_BUF_DTAB = 5      /* [n_z/2][n_y/2][n_x/2] */
+    SLP_BUF_DTAB = 5,     /* [n_z/2][n_y/2][n_x/2] */
+    SLP_BUF_NEAR = 6      /* [8][N]: near-field parts of the last evaluation's states, sorted targets */
 };
 
 /* Plan-time host arrays that slp_debug_host_array can copy out. */

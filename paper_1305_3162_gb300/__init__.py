@@ -38,7 +38,7 @@ SLP_NEAR_AUTO, SLP_NEAR_ON_THE_FLY, SLP_NEAR_PRECOMPUTED = 0, 1, 2
 
 SLP_STAGE_CHARGES, SLP_STAGE_SPREAD, SLP_STAGE_FFT_X, SLP_STAGE_FFT_Y, SLP_STAGE_FFT_Z = 0, 1, 2, 3, 4
 SLP_STAGE_IFFT_Y, SLP_STAGE_IFFT_X, SLP_STAGE_GATHER, SLP_STAGE_NEAR = 5, 6, 7, 8
-SLP_BUF_QBUF, SLP_BUF_GRID_A, SLP_BUF_GRID_B, SLP_BUF_S1, SLP_BUF_S2, SLP_BUF_DTAB = 0, 1, 2, 3, 4, 5
+SLP_BUF_QBUF, SLP_BUF_GRID_A, SLP_BUF_GRID_B, SLP_BUF_S1, SLP_BUF_S2, SLP_BUF_DTAB, SLP_BUF_NEAR = 0, 1, 2, 3, 4, 5, 6
 (SLP_HOST_SRC_PERM, SLP_HOST_TGT_PERM, SLP_HOST_SRC_GRID, SLP_HOST_TGT_GRID, SLP_HOST_SPREAD_ITEMS,
  SLP_HOST_GATHER_ITEMS, SLP_HOST_NEAR_ITEMS, SLP_HOST_NEAR_RANGES, SLP_HOST_DTAB, SLP_HOST_SRC_POINTS,
  SLP_HOST_TGT_POINTS, SLP_HOST_PLANE_ROWS, SLP_HOST_ACTIVE_Z, SLP_HOST_SPREAD_GROUPS,

@@ -3241,6 +3241,7 @@ slp_status slp_debug_buffer_bytes(slp_plan_t p, int buf, int64_t *bytes) {
         case SLP_BUF_S1: *bytes = 2 * es * p->L[2] * p->L[1] * Kx; break;
         case SLP_BUF_S2: *bytes = 2 * es * p->L[2] * p->n[1] * Kx; break;
         case SLP_BUF_DTAB: *bytes = es * (int64_t)p->Dtab.size(); break;
+        case SLP_BUF_NEAR: *bytes = es * p->N * slp::NEAR_STATES; break;
         default: return fail(SLP_ERR_INVALID_ARG, "unknown buffer %d", buf);
     }
     return SLP_OK;
@@ -3260,6 +3261,7 @@ slp_status slp_debug_copy(slp_plan_t p, int buf, void *host, int64_t bytes) {
         case SLP_BUF_S1: src = p->dp.S1; break;
         case SLP_BUF_S2: src = p->dp.S2; break;
         case SLP_BUF_DTAB: src = p->dp.Dtab; break;
+        case SLP_BUF_NEAR: src = p->dp.phi_part; break;
     }
     DeviceGuard g(p->device);
     TRY(cuda_status(cudaDeviceSynchronize(), "synchronize"));
