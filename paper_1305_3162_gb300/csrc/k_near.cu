@@ -21,6 +21,9 @@
 // E being smooth on [0, (a eps)^2]: one polynomial in r^2 in FP32, a table of
 // short ones in FP64.  The general kernel k_near takes the other modes, and
 // RADIAL plans whose a eps lies outside the fits' range.
+#include <algorithm>
+#include <climits>
+
 #include "dev_common.cuh"
 
 namespace slp {
@@ -451,19 +454,23 @@ __device__ __forceinline__ double nm_kernel(const NMBuild &b, const double *tab,
     return erfc(r2 * ri * b.inv_s_sqrt2) * ri * 0.079577471545947667884;
 }
 
-// One warp per group of NM_ROWS consecutive sorted targets, a candidate vertex
-// per lane.  An entry is a vertex with a quadrature point of an adjacent
+// b.parts warps per group of NM_ROWS consecutive sorted targets, which share its
+// candidate vertices by consecutive batches of 32 (`batches`), a candidate per
+// lane; counts and offsets are per part.  An entry is a vertex with a quadrature point of an adjacent
 // triangle within eps of some target of the group; its weights are zero for the
-// others.  pass 0: count the group's entries, its (target, vertex) pairs with a
+// others.  pass 0: count the part's entries, its (target, vertex) pairs with a
 // point inside and the near pairs; pass 1: fill.  The kernel is evaluated in
 // FP64, three times per pair (once per vertex of the triangle), so the FP64 pipe
 // bounds the fill: the table's 25 operations where erfc and rsqrt took over 100,
 // no evaluation in the count, and vertices out of every target's reach passed
 // over.  Plan of plate400 (319M pairs) 2.56 -> 0.83 s, of sphere5 at 128^3 (6M)
-// 0.23 -> 0.09 s.
+// 0.23 -> 0.09 s.  With one warp a group the 97 groups of the 8x8 cube are 13
+// blocks, each with four rows' series to add up: plans with every pair near,
+// FP64, 13.6 -> 2.9 ms (8x8 cube), 14.0 -> 2.7 (level-2 sphere, 7 points), 47.2 ->
+// 10.3 (level 3); a radial one of the level-3 sphere 10.7 -> 7.0.
 template <typename T4>
 __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, NMCount *__restrict__ counts,
-                                                  const int64_t *__restrict__ gptr, int *__restrict__ col,
+                                                  const int64_t *__restrict__ offset, int *__restrict__ col,
                                                   T4 *__restrict__ val, int64_t stride) {
     constexpr int R = NM_ROWS;
     __shared__ double tab[(NEAR_DEG64 + 1) * NEAR_INT64];
@@ -472,18 +479,27 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, NMCount *
         for (int i = threadIdx.x; i < (NEAR_DEG64 + 1) * b.ni; i += blockDim.x) tab[i] = b.tab[i];
         __syncthreads();
     }
-    const int64_t g = (int64_t)blockIdx.x * 8 + warp;
+    const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp, g = w / b.parts;
+    const int part = (int)(w - g * b.parts);
     if (R * g >= b.N) return;
     const int nr = (int)min((int64_t)R, b.N - R * g);
     double4 x[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = b.tgt[R * g + min(r, nr - 1)];
     const int blk = b.grp_block[g];
-    int64_t out = pass == 1 ? gptr[g] : 0;
+    int64_t out = pass == 1 ? offset[w] : 0;
     int64_t cnt = 0, npairs = 0, nnz = 0;
-    for (int rr = b.blk_r0[blk]; rr < b.blk_r0[blk + 1]; ++rr) {
+    int first = 0, last = INT_MAX, batch = 0;  // the part's batches of the group's candidates
+    if (b.parts > 1) {
+        int all = 0;
+        for (int rr = b.blk_r0[blk]; rr < b.blk_r0[blk + 1]; ++rr) all += (b.ranges[rr].y - b.ranges[rr].x + 31) / 32;
+        first = (int)((int64_t)all * part / b.parts);
+        last = (int)((int64_t)all * (part + 1) / b.parts);
+    }
+    for (int rr = b.blk_r0[blk]; rr < b.blk_r0[blk + 1] && batch < last; ++rr) {
         const int2 rg = b.ranges[rr];
-        for (int u0 = rg.x; u0 < rg.y; u0 += 32) {
+        for (int u0 = rg.x; u0 < rg.y; u0 += 32, ++batch) {
+            if (batch < first || batch >= last) continue;
             const int u = u0 + lane;
             double wx[R], wy[R], wz[R];
 #pragma unroll
@@ -546,17 +562,26 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, NMCount *
     }
     npairs = warp_sum((long long)npairs);
     nnz = warp_sum((long long)nnz);
-    if (pass == 0 && lane == 0) counts[g] = {cnt, nnz, npairs};
+    if (pass == 0 && lane == 0) counts[w] = {cnt, nnz, npairs};
 }
 
-cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *gptr, int *col,
+// Warps per group: as many as give each of 152 SMs 16 warps (what it holds of
+// this kernel), at most 32 (a candidate list is rarely longer than 32 batches
+// where groups are so few).
+int nm_build_parts(int64_t N) {
+    const int64_t groups = (N + NM_ROWS - 1) / NM_ROWS;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(32, (152 * 16 + groups - 1) / groups));
+}
+
+cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *offset, int *col,
                             void *val, int64_t stride, cudaStream_t s) {
-    const int64_t groups = (b.N + NM_ROWS - 1) / NM_ROWS;
-    const unsigned nb = (unsigned)((groups + 7) / 8);
+    const int64_t warps = (b.N + NM_ROWS - 1) / NM_ROWS * b.parts;
+    const int wpb = warps >= 152 * 32 ? 8 : 2;  // few warps: small blocks, over all SMs
+    const unsigned nb = (unsigned)((warps + wpb - 1) / wpb);
     if (prec == 64)
-        k_nm_build<double4><<<nb, 256, 0, s>>>(b, pass, counts, gptr, col, (double4 *)val, stride);
+        k_nm_build<double4><<<nb, 32 * wpb, 0, s>>>(b, pass, counts, offset, col, (double4 *)val, stride);
     else
-        k_nm_build<float4><<<nb, 256, 0, s>>>(b, pass, counts, gptr, col, (float4 *)val, stride);
+        k_nm_build<float4><<<nb, 32 * wpb, 0, s>>>(b, pass, counts, offset, col, (float4 *)val, stride);
     return cudaGetLastError();
 }
 

@@ -296,13 +296,14 @@ cudaError_t launch_zero(void *ptr, size_t bytes, cudaStream_t s);
 // assembly of W (FP64, temporary device arrays).
 constexpr int NM_ROWS = 4;  // rows of a group (the entries' 4-vectors)
 struct NMCount {
-    int64_t entries, nnz, pairs;  // of a group; (target, vertex) and (target, source) pairs with a source within eps
+    int64_t entries, nnz, pairs;  // of a part of a group; (target, vertex) and (target, source) pairs with a source within eps
 };
 struct NMBuild {
     const double4 *vpos;     // sorted vertices, like tgt
     double reach2;           // squared distance a vertex with a point within eps can have
     const double4 *tgt;      // [N] sorted targets, physical coordinates relative to the torus centre
     const int *tgt_perm;     // [N] sorted -> user vertex
+    int parts;               // warps that share a group (nm_build_parts)
     const int *grp_block;    // [groups] candidate list of each group
     const int *blk_r0;       // [lists + 1]
     const int2 *ranges;      // candidate vertex ranges (sorted target order)
@@ -328,7 +329,9 @@ struct NMBuild {
     int ni;
     double iw, sqrt_iw;
 };
-cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *gptr, int *col,
+int nm_build_parts(int64_t N);
+// counts (pass 0) and offset of the first entry (pass 1): [groups][parts]
+cudaError_t launch_nm_build(const NMBuild &b, int pass, int prec, NMCount *counts, const int64_t *offset, int *col,
                             void *val, int64_t stride, cudaStream_t s);
 // phi_part = W m (overwrites)
 cudaError_t launch_near_matrix(const DevPlan &p, const void *d_m, cudaStream_t s);

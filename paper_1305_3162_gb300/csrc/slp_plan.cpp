@@ -1725,23 +1725,26 @@ void run_candidates(NearCandidates &c, int64_t N, int run) {
 // The operator's two assembly passes: group pointers, columns and weights
 // allocated by alloc(bytes, &ptr), which may refuse (ptr NULL: left unbuilt).
 template <typename Alloc>
-slp_status build_operator(const slp_plan_s &p, const slp::NMBuild &nb, Alloc alloc, slp::DevPlan &v, int64_t &nnz,
-                          int64_t &pairs) {
+slp_status build_operator(const slp_plan_s &p, slp::NMBuild nb, Alloc alloc, slp::DevPlan &v, int64_t &nnz, int64_t &pairs) {
     const int64_t groups = (nb.N + slp::NM_ROWS - 1) / slp::NM_ROWS;
-    TmpBuf b_cnt;
-    std::vector<slp::NMCount> cnt(groups);
+    nb.parts = slp::nm_build_parts(nb.N);
+    TmpBuf b_cnt, b_off;
+    std::vector<slp::NMCount> cnt(groups * nb.parts);
     TRY(tmp_upload(b_cnt, cnt.data(), cnt.size()));
     TRY(cuda_status(slp::launch_nm_build(nb, 0, p.prec, (slp::NMCount *)b_cnt.p, nullptr, nullptr, nullptr, 0, 0),
                     "near matrix count"));
-    TRY(cuda_status(cudaMemcpy(cnt.data(), b_cnt.p, sizeof(slp::NMCount) * groups, cudaMemcpyDeviceToHost), "count copy"));
-    std::vector<int64_t> gptr(groups + 1, 0);
+    TRY(cuda_status(cudaMemcpy(cnt.data(), b_cnt.p, sizeof(slp::NMCount) * cnt.size(), cudaMemcpyDeviceToHost), "count copy"));
+    std::vector<int64_t> gptr(groups + 1, 0), offset(cnt.size());
+    int64_t entries = 0;
     nnz = pairs = 0;
-    for (int64_t g = 0; g < groups; ++g) {
-        gptr[g + 1] = gptr[g] + cnt[g].entries;
-        nnz += cnt[g].nnz;
-        pairs += cnt[g].pairs;
+    for (size_t k = 0; k < cnt.size(); ++k) {
+        offset[k] = entries;
+        entries += cnt[k].entries;
+        nnz += cnt[k].nnz;
+        pairs += cnt[k].pairs;
+        gptr[k / nb.parts + 1] = entries;
     }
-    const int64_t entries = std::max<int64_t>(gptr[groups], 1);
+    entries = std::max<int64_t>(entries, 1);
     void *d_val = nullptr, *d_col = nullptr, *d_gptr = nullptr;
     TRY(alloc(3 * 4 * (size_t)(p.prec / 8) * entries, &d_val));
     if (!d_val) return SLP_OK;
@@ -1749,13 +1752,14 @@ slp_status build_operator(const slp_plan_s &p, const slp::NMBuild &nb, Alloc all
     TRY(alloc(sizeof(int64_t) * (groups + 1), &d_gptr));
     if (!d_col || !d_gptr) return fail(SLP_ERR_OOM, "near-field operator");
     TRY(cuda_status(cudaMemcpy(d_gptr, gptr.data(), sizeof(int64_t) * (groups + 1), cudaMemcpyHostToDevice), "upload"));
+    TRY(tmp_upload(b_off, offset.data(), offset.size()));
     v.nm_gptr = (const int64_t *)d_gptr;
     v.nm_col = (const int *)d_col;
     v.nm_val = d_val;
     v.nm_stride = entries;
-    TRY(cuda_status(slp::launch_nm_build(nb, 1, p.prec, nullptr, v.nm_gptr, (int *)d_col, d_val, entries, 0),
+    TRY(cuda_status(slp::launch_nm_build(nb, 1, p.prec, nullptr, (const int64_t *)b_off.p, (int *)d_col, d_val, entries, 0),
                     "near matrix fill"));
-    return SLP_OK;
+    return cuda_status(cudaDeviceSynchronize(), "near matrix build");
 }
 
 slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) {
