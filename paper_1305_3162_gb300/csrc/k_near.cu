@@ -565,9 +565,8 @@ __global__ void __launch_bounds__(256) k_nm_build(NMBuild b, int pass, NMCount *
     if (pass == 0 && lane == 0) counts[w] = {cnt, nnz, npairs};
 }
 
-// Warps per group: as many as give each of 152 SMs 16 warps (what it holds of
-// this kernel), at most 32 (a candidate list is rarely longer than 32 batches
-// where groups are so few).
+// Warps per group: as many as give each of 152 SMs 16 warps, at most 32 (a
+// candidate list is rarely longer than 32 batches where groups are so few).
 int nm_build_parts(int64_t N) {
     const int64_t groups = (N + NM_ROWS - 1) / NM_ROWS;
     return (int)std::max<int64_t>(1, std::min<int64_t>(32, (152 * 16 + groups - 1) / groups));
@@ -597,7 +596,10 @@ __device__ __forceinline__ double4 ld_stream(const double4 *p) {
 // entry is a column and 4 x 3 weights, in three streams of 4-vectors (the x, y
 // and z weights of the four rows), and a gathered m serves four rows.  Bounds:
 // HBM (52 bytes an entry against four of 16; 83 % of the weights are non-zero
-// on the level-5 sphere at 128^3, 93 % on plate400) and, with several states,
+// on the level-5 sphere at 128^3, 93 % on plate400, and 25 to 45 % for probes so
+// scattered that neighbours share few vertices, where the product is no slower
+// for it: level-6 sphere at 256^3 with 200, 2000 and 8000 probes 137.7, 142.0 and
+// 149.5 us an evaluation, 143.7, 145.8 and 151.9 with a warp per row) and, with several states,
 // the gathers through L1, which fall to a quarter.  Against one row per warp
 // and 16-byte entries of their own: plate400 725 -> 650 us, cube200 371 -> 345,
 // cube400 1392 -> 1240; evaluations with it beside the far field: sphere5 52.0

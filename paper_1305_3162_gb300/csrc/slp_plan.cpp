@@ -1844,12 +1844,19 @@ slp_status build_near_matrix(slp_plan_s &p, const std::vector<uint64_t> &tkeys) 
         nb.es_g = (const double *)b_esg.p;
         nb.es_n = (int)w.size();
     }
-    bool refused = false;
+    // Budget, decided at the first allocation (the weights): 24 GB and half of the
+    // free memory for 4 values a (target, vertex) pair, whatever the groups' unions
+    // add or save (0.8 of that where the weights are 93 % full, 1.0 at 75 %), as long
+    // as they fit; else the near field stays per pair.
+    bool refused = false, decided = false;
     auto alloc = [&](size_t bytes, void **ptr) -> slp_status {
-        size_t freeb = 0, totb = 0;
-        cudaMemGetInfo(&freeb, &totb);
-        // budget (the weights come first): else keep the near field per pair
-        refused = refused || bytes > ((size_t)24 << 30) || bytes > freeb / 2;
+        if (!decided) {
+            size_t freeb = 0, totb = 0;
+            cudaMemGetInfo(&freeb, &totb);
+            const double want = 4.0 * (p.prec / 8) * (double)p.nm_nnz;
+            refused = want > 24.0 * (1 << 30) || want > 0.5 * (double)freeb || (double)bytes > 0.9 * (double)freeb;
+            decided = true;
+        }
         return refused ? SLP_OK : dalloc(p, ptr, bytes);
     };
     TRY(build_operator(p, nb, alloc, p.dp, p.nm_nnz, p.near_pairs_within));
