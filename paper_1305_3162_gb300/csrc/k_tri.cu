@@ -445,7 +445,12 @@ __global__ void __launch_bounds__(256) k_p0_charges(DevPlan p, const T *__restri
 // are short (185 entries in the level-5 sphere's gridding matrix), by latency: a
 // lane has four (rows of 32 lanes: eight) entries in flight, then their gathers.
 // Against one at a time, evaluations: sphere5 triangles 84.9 -> 84.2 us, cube40
-// 62.1 -> 60.6, sphere5 deterministic 102.1 -> 99.4.
+// 62.1 -> 60.6, sphere5 deterministic 102.1 -> 99.4.  In FP64 only whole batches
+// are taken so: on fine grids the rows are of a few entries, and a batch's unused
+// places cost the FP64 pipe as much as used ones (deterministic level-3 sphere
+// at 512^3 4849 us with the loop alone, 4930 with all rests in batches, 4844 so;
+// cube7 at 256^3 512, 526, 515; triangles of the level-3 sphere at 256^3 651,
+// 656, 638).
 template <typename T, int LPR>
 __global__ void __launch_bounds__(256) k_csr_apply(int64_t nrows, const int64_t *__restrict__ rowptr,
                                                    const int64_t *__restrict__ row_idx, const int *__restrict__ col,
@@ -478,7 +483,9 @@ __global__ void __launch_bounds__(256) k_csr_apply(int64_t nrows, const int64_t 
 #pragma unroll
             for (int u = 0; u < U; ++u) acc += w[u] * g[u];
         }
-        if (k < n) {
+        if constexpr (sizeof(T) == 8) {
+            for (; k + sub < n; k += LPR) acc += __ldcs(v + k) * x[__ldcs(c + k)];
+        } else if (k < n) {
             T w[U];
             int ci[U];
 #pragma unroll
