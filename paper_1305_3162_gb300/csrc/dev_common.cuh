@@ -111,10 +111,10 @@ template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch with programmatic stream serialization allowed (see pdl_wait).
+// Launch with programmatic stream serialization allowed (`early`; see pdl_wait).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
-                            Args... args) {
+inline cudaError_t launch_when(bool early, void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                               Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
@@ -124,8 +124,13 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, unsigned block, s
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                            Args... args) {
+    return launch_when(true, kern, grid, block, smem, s, args...);
 }
 
 __device__ __forceinline__ void set_error(int *err, int code) {

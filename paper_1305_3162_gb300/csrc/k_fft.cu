@@ -1416,36 +1416,57 @@ template <typename K> static cudaError_t prep(K kern, size_t sm) {
     return cudaSuccess;
 }
 
+// Launch of one transform pass.  Blocks launched early take whatever room the
+// pass before has left on each SM, so they are not spread evenly: at 128^3 the
+// 147 blocks of the x pass put 4 on one SM (108 blocks: 8) where 1 would be even,
+// the 256 of the z pass 3 or 4 where 2 would be.  An FP64 pass is bound by its
+// SMs' FP64 pipes (2 lanes each), so the fullest SM sets its time: where the y
+// pass has 64 to 304 blocks (up to two per SM), passes with blocks of at least
+// 128 threads are launched when the pass before has ended.  FP64 evaluations at
+// 128^3: level-2 sphere with one point a triangle 132 -> 109 us, level-3 sphere
+// 229 -> 185, level-4 454 -> 417, level-3 deterministic 220 -> 196, 7x7 cube with
+// triangles 129 -> 120.  More blocks even out by themselves (256^3, 500 to 1000:
+// 655 us an evaluation, 672 so), and fewer leave SMs free for each other (a plate
+// at 128^3, 25 and 60 blocks in the x and y passes, 101 and 105; at 128x64x64 84
+// and 97): both keep the early launch.
+template <typename T, typename... KArgs, typename... Args>
+static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigned threads, size_t sm, cudaStream_t s,
+                               const DevPlan &p, Args... args) {
+    const int yb = p.nz_act * (p.Kx / CB) * p.ks;
+    const bool even = sizeof(T) == 8 && threads >= 128 && yb >= 64 && yb <= 2 * 152;
+    return launch_when(!even, kern, nb, threads, sm, s, p, args...);
+}
+
 // column engine launch: L = 2^lg threads, 8 columns per block
 #define SLP_COL_DISPATCH(KERN, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
         case 5: { cudaError_t e_ = prep(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
+                  return launch_pass<T>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
         case 6: { cudaError_t e_ = prep(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
+                  return launch_pass<T>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
         case 7: { cudaError_t e_ = prep(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
+                  return launch_pass<T>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
         case 8: { cudaError_t e_ = prep(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
+                  return launch_pass<T>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
         case 9: { cudaError_t e_ = prep(KERN<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 9>, NBLK, 512, SM, S, p); }                                    \
+                  return launch_pass<T>(KERN<T, 9>, NBLK, 512, SM, S, p); }                                    \
         case 10: { cudaError_t e_ = prep(KERN<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
-                   return launch_k(KERN<T, 10>, NBLK, 1024, SM, S, p); }                                 \
+                   return launch_pass<T>(KERN<T, 10>, NBLK, 1024, SM, S, p); }                                 \
     }
 #define SLP_COL_DISPATCH2(KERN, KERNL, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
         case 5: { cudaError_t e_ = prep(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
+                  return launch_pass<T>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
         case 6: { cudaError_t e_ = prep(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
+                  return launch_pass<T>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
         case 7: { cudaError_t e_ = prep(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
+                  return launch_pass<T>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
         case 8: { cudaError_t e_ = prep(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
+                  return launch_pass<T>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
         case 9: { cudaError_t e_ = prep(KERNL<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_k(KERNL<T, 9>, NBLK, 512, SM, S, p); }                                    \
+                  return launch_pass<T>(KERNL<T, 9>, NBLK, 512, SM, S, p); }                                    \
         case 10: { cudaError_t e_ = prep(KERNL<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
-                   return launch_k(KERNL<T, 10>, NBLK, 1024, SM, S, p); }                                 \
+                   return launch_pass<T>(KERNL<T, 10>, NBLK, 1024, SM, S, p); }                                 \
     }
 // the engine applies for 32 <= L <= 1024 and at least 8 stored x frequencies
 static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024 && p.Kx >= CB; }
@@ -1453,14 +1474,7 @@ static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024
 // row engine launch, 128 <= L <= 1024 (shorter rows share a wavefront between
 // pairs and are transformed by the fused plane passes anyway; at 1024 a pair is
 // 128 threads)
-// FP64 rows of 128 behind a gridding product (triangle integrals, deterministic
-// spread) keep the staged kernels: level-3 sphere at 128^3, deterministic, 178 us
-// an evaluation against 261, cube7 with triangles 130 against 193; behind the
-// spread kernels the row engine is the better one (157 against 133 us).
-static bool row_engine_ok(const DevPlan &p) {
-    if (p.prec == 64 && p.L[0] == 128 && p.am_rowptr) return false;
-    return p.L[0] >= 128 && p.L[0] <= 1024;
-}
+static bool row_engine_ok(const DevPlan &p) { return p.L[0] >= 128 && p.L[0] <= 1024; }
 template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
     typedef RowShape<LG> Sh;
     if (p.n_row_pairs == 0) return cudaSuccess;
@@ -1468,7 +1482,7 @@ template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPla
     const cudaError_t e = prep(kern, sm);
     if (e != cudaSuccess) return e;
     const dim3 nb((unsigned)((p.n_row_pairs + Sh::PB - 1) / Sh::PB), (unsigned)p.ks);
-    const cudaError_t le = launch_k(kern, nb, Sh::NT, sm, s, p);
+    const cudaError_t le = launch_pass<T>(kern, nb, Sh::NT, sm, s, p);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) {
@@ -1484,7 +1498,7 @@ template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = prep(k_fx<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.n_row_pairs == 0) return cudaSuccess;
-    { const cudaError_t le = launch_k(k_fx<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T>(k_fx<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) {
@@ -1500,7 +1514,7 @@ template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = prep(k_ix<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.n_row_pairs == 0) return cudaSuccess;
-    { const cudaError_t le = launch_k(k_ix<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T>(k_ix<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t fy_t(const DevPlan &p, cudaStream_t s) {
@@ -1516,7 +1530,7 @@ template <typename T> static cudaError_t fy_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = prep(k_fy<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
-    { const cudaError_t le = launch_k(k_fy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T>(k_fy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t iy_t(const DevPlan &p, cudaStream_t s) {
@@ -1532,7 +1546,7 @@ template <typename T> static cudaError_t iy_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = prep(k_iy<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
-    { const cudaError_t le = launch_k(k_iy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T>(k_iy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t fz_t(const DevPlan &p, cudaStream_t s) {
@@ -1548,7 +1562,7 @@ template <typename T> static cudaError_t fz_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = prep(k_fz<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
-    { const cudaError_t le = launch_k(k_fz<T>, dim3(p.n[1] * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T>(k_fz<T>, dim3(p.n[1] * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 
