@@ -98,6 +98,13 @@ slp_status slp_debug_profile(slp_plan_t plan, int input_kind, const void *d_in, 
                              float *ms, int n);
 const char *slp_debug_stage_name(int i);
 
+/* 1 where the near field per pair (charges at the quadrature points) runs the
+ * kernels with the fitted erf, 0 where it runs the general one: EXPSUM and
+ * SEPARABLE plans, and RADIAL ones whose radius the fits do not cover
+ * (tolerances below about 3e-7 in FP32, 4e-20 in FP64).  NO_DEVICE for a
+ * host-only plan. */
+slp_status slp_debug_near_fit(slp_plan_t plan, int *fit);
+
 /* The normalised Kaiser-Bessel window psi(d) in grid units (Sec. 3.2,
  * Eq. (KBfct) scaled to psi(0) = 1) and its continuous Fourier transform at
  * frequency index l of an L-point grid, both in FP64 on the host. */

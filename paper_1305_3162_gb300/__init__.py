@@ -154,6 +154,7 @@ EXPORTED = ["slp_default_opts", "slp_plan", "slp_eval", "slp_eval_states", "slp_
             "slp_debug_run", "slp_debug_copy", "slp_debug_buffer_bytes", "slp_debug_host_count",
             "slp_debug_host_array", "slp_debug_window", "slp_debug_window_hat", "slp_debug_profile",
             "slp_debug_timeline", "slp_debug_fem_assemble", "slp_debug_potential_create", "slp_debug_potential_solver",
+            "slp_debug_near_fit",
             "slp_debug_stage_name", "slp_eval_direct_static", "slp_batch_create", "slp_batch_run",
             "slp_batch_query", "slp_batch_destroy", "slp_eval_batched", "slp_plan_autotune", "slp_server_default_opts",
             "slp_server_create", "slp_server_submit", "slp_server_status", "slp_server_wait", "slp_server_cancel",
@@ -214,6 +215,7 @@ def load():
         "slp_debug_window_hat": ([ctypes.c_int, ctypes.c_int, ctypes.c_double], ctypes.c_double),
         "slp_debug_profile": ([vp, ctypes.c_int, vp, vp, vp, ctypes.POINTER(ctypes.c_float), ctypes.c_int], St),
         "slp_debug_timeline": ([vp, ctypes.c_int, vp, vp, vp, ctypes.POINTER(ctypes.c_float)], St),
+        "slp_debug_near_fit": ([vp, ctypes.POINTER(ctypes.c_int)], St),
         "slp_debug_stage_name": ([ctypes.c_int], ctypes.c_char_p),
         "slp_debug_fem_assemble": ([ctypes.POINTER(ctypes.c_double), I64, ctypes.POINTER(ctypes.c_int32), I64,
                                     ctypes.POINTER(I64), vp, vp, vp, vp, vp, vp, vp, vp, vp], St),
@@ -642,6 +644,13 @@ def slp_debug_profile(plan, input_kind, d_in, d_phi, stream=None) -> dict:
     _check(load().slp_debug_profile(plan, int(input_kind), _ptr(d_in), _ptr(d_phi), _stream(stream), ms, n),
            "slp_debug_profile")
     return {load().slp_debug_stage_name(i).decode(): float(ms[i]) for i in range(n) if ms[i] >= 0.0}
+
+
+def slp_debug_near_fit(plan) -> bool:
+    """Whether the near field per pair runs the kernels with the fitted erf."""
+    v = ctypes.c_int()
+    _check(load().slp_debug_near_fit(plan, ctypes.byref(v)), "slp_debug_near_fit")
+    return bool(v.value)
 
 
 def slp_debug_window(m: int, d: float) -> float:

@@ -3390,6 +3390,13 @@ slp_status slp_debug_timeline(slp_plan_t p, int kind, const void *d_in, void *d_
     return st;
 }
 
+slp_status slp_debug_near_fit(slp_plan_t p, int *fit) {
+    if (!p || !fit) return fail(SLP_ERR_INVALID_ARG, "NULL argument");
+    if (p->device < 0) return fail(SLP_ERR_NO_DEVICE, "host-only plan");
+    *fit = p->dp.near_fit;
+    return SLP_OK;
+}
+
 const char *slp_debug_stage_name(int i) { return (i >= 0 && i < SLP_PROFILE_SLOTS) ? STAGE_NAMES[i] : ""; }
 
 double slp_debug_window(int m, double d) { return kb_window_host(m, d); }
