@@ -175,7 +175,7 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 // FP32: a lane takes two sources per step in paired operations.  Per pair: 9 subtractions
 // (integer and fractional parts), 5 operations for r^2, one reciprocal square
 // root, the degree-14 polynomial of a E (15 multiply-adds, its argument's map
-// included), 2 for the sum: 31 lane operations where erfcf, the integer
+// included), 2 for the sum: 32 lane operations where erfcf, the integer
 // conversions and the cell arithmetic per pair took about 180.  Level-5 sphere
 // at 128^3 (118M lane pairs after the cull, 73M inside eps): 670 -> 164 us.
 __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_radial32(DevPlan p) {

@@ -397,7 +397,11 @@ slp_status expsum_params(slp_plan_s &p) {
 // Sized by the number of points alone (2 sqrt(Q + N) cells), a level-5 sphere
 // of 143360 sources got 1024^3 cells and 4035 us an evaluation; here 128^3 and
 // 52 us (256^3: 93).  cube131 (618k sources) 1024^3, 3385 us; here 256^3, 404 us
-// (512^3: 502).  level-3 sphere 256^3, 69 us; here 64^3, 31 us.
+// (512^3: 502), as the passes then ran.  The rates predate the row engine and
+// today's column exchanges (512^3 passes a third faster); with those, of twenty
+// meshes in both precisions none is more than 20 % above the best of the grids
+// with half, as many and twice the cells (torus60 30.8 us, at half 25.7; cube131
+// at 512^3 now 379 to 390, at 256^3 361).  level-3 sphere 256^3, 69 us; here 64^3, 31 us.
 // A coarser grid carries more of the kernel's split error (the level-5 sphere:
 // 3.7e-7 at 1024^3, 9.8e-7 at 128^3), so automatic grids split with AUTO_SPLIT
 // of the tolerance: cube40 at 128^3 1.35e-6 -> 3.7e-7 (5.3e-7 at 1024^3 before),
@@ -2480,18 +2484,22 @@ enum {
 // beside the far field?  Beside it, it fills the latency-bound passes' idle
 // SMs; but its short blocks also keep the larger blocks of the other stream
 // waiting for room, and where both are bound by HBM there is nothing to fill.
-// So first in line where the operator is large (the far field is a small part
-// of the evaluation; with several states, which share one pass over it, the
-// pass is longer still) or the grids exceed L2.  Measured, beside -> first:
-// cube200 at 512^3 (2.4 GB) 1002 -> 844 us, plate400 (5.1 GB) 884 -> 852,
-// cube400 at 1024^3 (9 GB) 5660 -> 5232, cube131 at 512^3 (0.5 GB) 506 -> 487;
-// cube131 at 256^3 (1.9 GB) 404 -> 410, sphere6 at 256^3 (0.3 GB) 147 -> 163,
-// sphere5 at 128^3 52 -> 64.  Eight states: torus400 (1.1 GB) 811 -> 790 us,
-// cube74 at 256^3 (0.2 GB) 693 -> 694, plate90 104 -> 129.
+// So first in line where the operator is so large that the far field is a small
+// part of the evaluation, or is large and the grids exceed L2; with several
+// states, which share one pass over it, sooner.  The operator's size is taken
+// as four values a pair, 4 es nnz (stored are 3.3 to 4 with the groups' padding).
+// Measured, beside and first, us: 5.1 GB (plate400) 763 and 752, 4.2 GB
+// (cube160 at 256^3) 705 and 703, 3.1 GB (plate250) 444 and 453, 2.9 GB (cube145
+// at 256^3) 509 and 514, 1.9 GB (cube131 at 256^3) 365 and 377, 0.3 GB (sphere6 at
+// 256^3) 140 and 159; with grids of 144 MB (512^3) 2.4 GB (cube200) 726 and 713,
+// 0.5 GB (cube131) 379 and 384, 0.2 GB (cube100) 313 and 320.  Eight states:
+// 1.4 GB (cube120 at 256^3) 1029 and 978, 1.1 GB (torus400) 657 and 639, 0.4 GB
+// (torus300) 352 and 359, 0.07 GB (plate90) 99 and 109.
 bool near_product_first(const slp_plan_s &p, int states) {
     const double es = p.prec == 64 ? 8 : 4;
     const double op = 4 * es * (double)p.nm_nnz, grids = 2 * es * 2.0 * p.row_pairs.size() * p.L[0];
-    return op >= (states > 1 ? 0.8e9 : 2.1e9) || grids >= 96e6;
+    if (states > 1) return op >= 0.8e9 || grids >= 96e6;
+    return op >= 4e9 || (op >= 1.5e9 && grids >= 96e6);
 }
 
 // Enqueue the evaluation up to stage `last`.
