@@ -108,6 +108,16 @@ template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Before a launch with `sm` bytes of dynamic shared memory.  The limit belongs to
+// the kernel, which plans of several sizes and host threads share, so it is
+// always raised to the same bound (no kernel here asks for more), never to a
+// plan's own size.
+constexpr int SMEM_LIMIT = 200 * 1024;
+template <typename K> inline cudaError_t allow_smem(K kern, size_t sm) {
+    if (sm <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+}
+
 // Launch with programmatic stream serialization allowed (`early`; see pdl_wait).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_when(bool early, void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,

@@ -1411,11 +1411,6 @@ static int col_batch(int L, int Kx, size_t celem, int64_t rows_of_blocks) {
     return b;
 }
 
-template <typename K> static cudaError_t prep(K kern, size_t sm) {
-    if (sm > 48 * 1024) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    return cudaSuccess;
-}
-
 // Launch of one transform pass.  Blocks launched early take whatever room the
 // pass before has left on each SM, so they are not spread evenly: at 128^3 the
 // 147 blocks of the x pass put 4 on one SM (108 blocks: 8) where 1 would be even,
@@ -1440,32 +1435,32 @@ static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigne
 // column engine launch: L = 2^lg threads, 8 columns per block
 #define SLP_COL_DISPATCH(KERN, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
-        case 5: { cudaError_t e_ = prep(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 5: { cudaError_t e_ = allow_smem(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
-        case 6: { cudaError_t e_ = prep(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 6: { cudaError_t e_ = allow_smem(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
-        case 7: { cudaError_t e_ = prep(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 7: { cudaError_t e_ = allow_smem(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
-        case 8: { cudaError_t e_ = prep(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 8: { cudaError_t e_ = allow_smem(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
-        case 9: { cudaError_t e_ = prep(KERN<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 9: { cudaError_t e_ = allow_smem(KERN<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 9>, NBLK, 512, SM, S, p); }                                    \
-        case 10: { cudaError_t e_ = prep(KERN<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
+        case 10: { cudaError_t e_ = allow_smem(KERN<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
                    return launch_pass<T>(KERN<T, 10>, NBLK, 1024, SM, S, p); }                                 \
     }
 #define SLP_COL_DISPATCH2(KERN, KERNL, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
-        case 5: { cudaError_t e_ = prep(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 5: { cudaError_t e_ = allow_smem(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
-        case 6: { cudaError_t e_ = prep(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 6: { cudaError_t e_ = allow_smem(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
-        case 7: { cudaError_t e_ = prep(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 7: { cudaError_t e_ = allow_smem(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
-        case 8: { cudaError_t e_ = prep(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 8: { cudaError_t e_ = allow_smem(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
-        case 9: { cudaError_t e_ = prep(KERNL<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
+        case 9: { cudaError_t e_ = allow_smem(KERNL<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
                   return launch_pass<T>(KERNL<T, 9>, NBLK, 512, SM, S, p); }                                    \
-        case 10: { cudaError_t e_ = prep(KERNL<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
+        case 10: { cudaError_t e_ = allow_smem(KERNL<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
                    return launch_pass<T>(KERNL<T, 10>, NBLK, 1024, SM, S, p); }                                 \
     }
 // the engine applies for 32 <= L <= 1024 and at least 8 stored x frequencies
@@ -1479,7 +1474,7 @@ template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPla
     typedef RowShape<LG> Sh;
     if (p.n_row_pairs == 0) return cudaSuccess;
     const size_t sm = (size_t)(Sh::PB + 1) * Sh::L * 2 * sizeof(T);
-    const cudaError_t e = prep(kern, sm);
+    const cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
     const dim3 nb((unsigned)((p.n_row_pairs + Sh::PB - 1) / Sh::PB), (unsigned)p.ks);
     const cudaError_t le = launch_pass<T>(kern, nb, Sh::NT, sm, s, p);
@@ -1495,7 +1490,7 @@ template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) 
     const size_t ce = 2 * sizeof(T);
     const int PB = row_batch(p.L[0], ce);
     const size_t sm = (2 * (size_t)p.L[0] * (PB + 1) + p.L[0]) * ce;
-    cudaError_t e = prep(k_fx<T>, sm);
+    cudaError_t e = allow_smem(k_fx<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.n_row_pairs == 0) return cudaSuccess;
     { const cudaError_t le = launch_pass<T>(k_fx<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
@@ -1511,7 +1506,7 @@ template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) 
     const size_t ce = 2 * sizeof(T);
     const int PB = row_batch(p.L[0], ce);
     const size_t sm = (2 * (size_t)p.L[0] * (PB + 1) + p.L[0]) * ce;
-    cudaError_t e = prep(k_ix<T>, sm);
+    cudaError_t e = allow_smem(k_ix<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.n_row_pairs == 0) return cudaSuccess;
     { const cudaError_t le = launch_pass<T>(k_ix<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
@@ -1527,7 +1522,7 @@ template <typename T> static cudaError_t fy_t(const DevPlan &p, cudaStream_t s) 
     const size_t ce = 2 * sizeof(T);
     const int B = col_batch(p.L[1], p.Kx, ce, p.nz_act);
     const size_t sm = ((size_t)p.L[1] * (B + 1) + p.L[1]) * ce;
-    cudaError_t e = prep(k_fy<T>, sm);
+    cudaError_t e = allow_smem(k_fy<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
     { const cudaError_t le = launch_pass<T>(k_fy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
@@ -1543,7 +1538,7 @@ template <typename T> static cudaError_t iy_t(const DevPlan &p, cudaStream_t s) 
     const size_t ce = 2 * sizeof(T);
     const int B = col_batch(p.L[1], p.Kx, ce, p.nz_act);
     const size_t sm = ((size_t)p.L[1] * (B + 1) + p.L[1]) * ce;
-    cudaError_t e = prep(k_iy<T>, sm);
+    cudaError_t e = allow_smem(k_iy<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
     { const cudaError_t le = launch_pass<T>(k_iy<T>, dim3(p.nz_act * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
@@ -1559,7 +1554,7 @@ template <typename T> static cudaError_t fz_t(const DevPlan &p, cudaStream_t s) 
     const size_t ce = 2 * sizeof(T);
     const int B = col_batch(p.L[2], p.Kx, ce, p.n[1]);
     const size_t sm = ((size_t)p.L[2] * (B + 1) + p.L[2]) * ce;
-    cudaError_t e = prep(k_fz<T>, sm);
+    cudaError_t e = allow_smem(k_fz<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
     { const cudaError_t le = launch_pass<T>(k_fz<T>, dim3(p.n[1] * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
@@ -1573,7 +1568,7 @@ static size_t fused_cta_smem(const DevPlan &p, int PB, size_t ce) {
 }
 
 template <typename K> static cudaError_t launch_cluster(K kern, const DevPlan &p, size_t sm, cudaStream_t s) {
-    cudaError_t e = prep(kern, sm);
+    cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
@@ -1606,7 +1601,7 @@ static size_t yzy_cta_smem(const DevPlan &p, int G, int ZP, size_t ce) {
     return ((size_t)p.n[1] * ZP + L + (size_t)G * L * CB) * ce;
 }
 template <typename K> static cudaError_t launch_yzy_cluster(K kern, const DevPlan &p, size_t sm, cudaStream_t s) {
-    cudaError_t e = prep(kern, sm);
+    cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.Kx * YZY_CL, p.ks);

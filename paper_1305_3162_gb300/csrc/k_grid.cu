@@ -1022,10 +1022,8 @@ static cudaError_t spread_mt(const DevPlan &p, int fused_kind, const void *in, c
         while (nw > 1 && SpreadSmem<T, M, TS>::bytes(nw, p.spread_chunk) > 100 * 1024) nw >>= 1;
         const size_t sm = SpreadSmem<T, M, TS>::bytes(nw, p.spread_chunk);
         auto go = [&](auto kern) -> cudaError_t {
-            if (sm > 48 * 1024) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e != cudaSuccess) return e;
-            }
+            const cudaError_t e = allow_smem(kern, sm);
+            if (e != cudaSuccess) return e;
             if (p.n_spread > 0) {
                 const cudaError_t le = launch_k(kern, dim3(p.n_spread, p.ks), 32 * nw, sm, s, p, fused_kind, (const T *)in);
                 if (le != cudaSuccess) return le;
@@ -1037,10 +1035,8 @@ static cudaError_t spread_mt(const DevPlan &p, int fused_kind, const void *in, c
                 typedef TileGeomG<M, TS> G;
                 const size_t smt = spread_tab_smem<M>(nw, p.spread_chunk, G::SIZE);
                 auto go_t = [&](auto kern) -> cudaError_t {
-                    if (smt > 48 * 1024) {
-                        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smt);
-                        if (e != cudaSuccess) return e;
-                    }
+                    const cudaError_t e = allow_smem(kern, smt);
+                    if (e != cudaSuccess) return e;
                     if (p.n_spread > 0) {
                         const cudaError_t le = launch_k(kern, dim3(p.n_spread, p.ks), 32 * nw, smt, s, p, fused_kind,
                                                         (const float *)in);
@@ -1060,10 +1056,8 @@ static cudaError_t spread_mt(const DevPlan &p, int fused_kind, const void *in, c
         }
     }
     const size_t sm = PlaneSmem<T, M, TS>::bytes(p.wdeg);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_spread_planes<T, M, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k_spread_planes<T, M, TS>, sm);
+    if (e != cudaSuccess) return e;
     if (p.n_spread > 0) {
         const cudaError_t le = launch_k(k_spread_planes<T, M, TS>, dim3(p.n_spread, p.ks), 32 * M, sm, s, p, fused_kind,
                                         (const T *)in);
@@ -1076,10 +1070,8 @@ template <typename T, int M, int TS> static cudaError_t gather_mt(const DevPlan 
     typedef TileGeom<M, TS> G;
     const size_t GC = (size_t)p.gather_chunk;
     const size_t sm = ((size_t)((G::SIZE + 3) & ~3) + GC * (3 * 2 * M + 4) + 8 * GATHER_SPLIT) * sizeof(T) + 2 * GC * sizeof(int);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_gather<T, M, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k_gather<T, M, TS>, sm);
+    if (e != cudaSuccess) return e;
     // FP64: bound by the SMs' FP64 pipes, so its blocks are launched when the pass
     // before has ended and spread evenly (beside blocks of it they are not: probes
     // of a torus at 128^3 166 -> 154 us, four states of a 10x10 cube 470 -> 399,
