@@ -609,24 +609,22 @@ __device__ __forceinline__ double4 ld_stream(const double4 *p) {
 // before the gathered m; FULL batches need no predicates, the tail batch reads
 // zero weights past the end.  The K sorted magnetisations are m4[k N + column];
 // lane l adds its entries in order, and warps that share a group take chunks of
-// 64 entries in turn whatever K (a batch of four takes two chunks, `gap` other
-// warps' entries apart), so a row's sums do not depend on K.
-constexpr int CHUNK = 64;
+// 128 entries in turn whatever K, so a row's sums do not depend on K.
+constexpr int CHUNK = 128;
 template <typename T, int K, int U, bool FULL>
 __device__ __forceinline__ void near_batch(const int *__restrict__ col, const typename VecT<T>::T4 *__restrict__ val,
-                                           int64_t stride, int j, int gap, int n, int lane,
+                                           int64_t stride, int j, int n, int lane,
                                            const typename VecT<T>::T4 *__restrict__ m4, int64_t N, T (&acc)[K][NM_ROWS]) {
     typedef typename VecT<T>::T4 T4;
     T4 wx[U], wy[U], wz[U];
     int c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const int jj = 32 * u < CHUNK ? j : j + gap;
-        if (FULL || jj + lane + 32 * u < n) {
-            c[u] = __ldcs(col + jj + 32 * u);
-            wx[u] = ld_stream(val + jj + 32 * u);
-            wy[u] = ld_stream(val + stride + jj + 32 * u);
-            wz[u] = ld_stream(val + 2 * stride + jj + 32 * u);
+        if (FULL || j + lane + 32 * u < n) {
+            c[u] = __ldcs(col + j + 32 * u);
+            wx[u] = ld_stream(val + j + 32 * u);
+            wy[u] = ld_stream(val + stride + j + 32 * u);
+            wz[u] = ld_stream(val + 2 * stride + j + 32 * u);
         } else {
             c[u] = 0;
             wx[u].x = wx[u].y = wx[u].z = wx[u].w = T(0);
@@ -648,11 +646,13 @@ __device__ __forceinline__ void near_batch(const int *__restrict__ col, const ty
 // phi_part[k][t] = the rows of a group applied to K states with one pass over
 // them.  `split` (1, 2 or 4) warps share a group, taking its chunks in turn,
 // so that meshes with few groups fill the GPU; their sums are added in order.
-// SHARED false: split is 1 (for one state, whose batch of two chunks then has no
-// gap to step over: plate400 751 us an evaluation, 769 with it).
-template <typename T, int K, bool SHARED = true> __global__ void __launch_bounds__(128) k_near_matrix(DevPlan p, int split) {
+template <typename T, int K> __global__ void __launch_bounds__(128) k_near_matrix(DevPlan p, int split) {
     typedef typename VecT<T>::T4 T4;
-    constexpr int U = K == 1 ? 4 : 2;  // entries in flight per lane
+    // entries in flight per lane: a chunk in one batch, or for four and eight states
+    // (registers) and FP64 in two, unrolled in FP32.  With two a batch and a loop
+    // over batches, torus400 with 2 to 8 states 287, 328, 382, 449, 500, 573, 642 us
+    // an evaluation; so 260, 296, 365, 403, 472, 500, 570
+    constexpr int U = K == 1 || (sizeof(T) == 4 && K != 4 && K != 8) ? 4 : 2;
     __shared__ T part[4][K * NM_ROWS];
     pdl_wait();
     pdl_trigger();
@@ -670,11 +670,14 @@ template <typename T, int K, bool SHARED = true> __global__ void __launch_bounds
         const int n = (int)(p.nm_gptr[g + 1] - e0);  // a group holds < 2^31 entries
         const int *col = p.nm_col + e0 + lane;
         const T4 *val = (const T4 *)p.nm_val + e0 + lane;
-        const int gap = SHARED ? CHUNK * (split - 1) : 0;  // the other warps' chunks
         int j = CHUNK * sub;
-        for (; j + (U > 2 ? gap : 0) + 32 * U <= n; j += 32 * U * split)
-            near_batch<T, K, U, true>(col, val, p.nm_stride, j, gap, n, lane, m4, p.N, acc);
-        if (j < n) near_batch<T, K, U, false>(col, val, p.nm_stride, j, gap, n, lane, m4, p.N, acc);
+        for (; j + CHUNK <= n; j += CHUNK * split)
+#pragma unroll(sizeof(T) == 8 ? 1 : CHUNK / (32 * U))
+            for (int h = 0; h < CHUNK; h += 32 * U)
+                near_batch<T, K, U, true>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
+#pragma unroll 1
+        for (int h = 0; h < CHUNK && j + h < n; h += 32 * U)
+            near_batch<T, K, U, false>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
     }
     // lane r of the group's first warp ends up with row r
     T v[K];
@@ -716,7 +719,7 @@ template <typename T> static cudaError_t near_states_t(const DevPlan &p, int K, 
     const int split = near_split(p), rows = NM_ROWS * 4 / split;  // rows of a block
     const unsigned nb = (unsigned)((p.N + rows - 1) / rows);
     switch (K) {
-        case 1: return launch_k(split > 1 ? k_near_matrix<T, 1> : k_near_matrix<T, 1, false>, nb, 128, 0, s, p, split);
+        case 1: return launch_k(k_near_matrix<T, 1>, nb, 128, 0, s, p, split);
         case 2: return launch_k(k_near_matrix<T, 2>, nb, 128, 0, s, p, split);
         case 3: return launch_k(k_near_matrix<T, 3>, nb, 128, 0, s, p, split);
         case 4: return launch_k(k_near_matrix<T, 4>, nb, 128, 0, s, p, split);
