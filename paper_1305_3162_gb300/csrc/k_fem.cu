@@ -532,7 +532,7 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
 // e + 1, which that block wrote after it had read its records of e, so two
 // copies suffice.  All blocks add the sums in one order and hold the same
 // scalars.  The launch is cooperative (all blocks resident); every wait is
-// bounded, a thread whose wait has run out starts no other, and a block that
+// bounded, all of a thread's waits in an exchange together, and a block that
 // gives up sets `stalled` and leaves, after which the others' waits run out as
 // well.
 //
@@ -561,7 +561,7 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
 constexpr int SNT = SOLVE_THREADS;
 constexpr int SNW = SNT / 32;
 constexpr int HB = 2;                  // halo records a thread reads at once
-constexpr int WAIT_LIMIT = 1 << 21;    // polls of one exchange (about a second)
+constexpr int WAIT_LIMIT = 1 << 21;    // polls of one exchange by a thread (about a second)
 
 __device__ __forceinline__ uint4 ld_record(const uint4 *p) {
     unsigned long long lo, hi;
@@ -579,13 +579,14 @@ __device__ __forceinline__ void st_record(uint4 *p, unsigned a, unsigned b, unsi
                  : "memory");
 }
 
-// Waits until the record at q carries number e; false when the bound is reached.
-__device__ __forceinline__ bool wait_record(const uint4 *q, unsigned e, uint4 &v) {
-    for (int n = 0; n < WAIT_LIMIT; ++n) {
+// Waits until the record at q carries number e; false when `left`, the polls
+// that the thread's waits of this exchange may still miss, runs out.
+__device__ __forceinline__ bool wait_record(const uint4 *q, unsigned e, uint4 &v, int &left) {
+    while (true) {
         v = ld_record(q);
         if (v.w == e) return true;
+        if (--left <= 0) return false;
     }
-    return false;
 }
 
 // K sums over the block's first NW warps, the same in every thread: shuffles,
@@ -698,10 +699,11 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
             // threads without a record of their own poll nothing
             uint4 sums, v[HB];
             bool lost = false;
-            if (tid < P) lost = !wait_record((e & 1 ? in1 : in0) + tid, e, sums);
+            int left = WAIT_LIMIT;
+            if (tid < P) lost = !wait_record((e & 1 ? in1 : in0) + tid, e, sums, left);
 #pragma unroll
             for (int i = 0; i < HB; ++i)
-                if (i * SNT + hid < nh) lost = lost || !wait_record(mine + i * SNT + hid, e, v[i]);
+                if (i * SNT + hid < nh) lost = !wait_record(mine + i * SNT + hid, e, v[i], left) || lost;
             float sum[2] = {0.f, 0.f}, wc = 0.f;
             if (tid < P) {
                 sum[0] = __uint_as_float(sums.x);
@@ -764,10 +766,7 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
             }
             for (int h = HB * SNT + hid; h < nh; h += SNT) {
                 uint4 vh;
-                if (lost || !wait_record(mine + h, e, vh)) {
-                    lost = true;
-                    break;
-                }
+                lost = !wait_record(mine + h, e, vh, left) || lost;
                 s_u[d.rp + h] = __uint_as_float(vh.x) -
                                 alpha * (__uint_as_float(vh.y) + beta * __uint_as_float(vh.z)) +
                                 d.halo_z[h0 + h] * s_ec[d.halo_near[h0 + h]];
@@ -819,12 +818,10 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
             for (int o = out0[j]; o < out1[j]; ++o) st_record(rec + d.dst[o], (unsigned)b, (unsigned)(b >> 32), 0u, e);
         }
         bool lost = false;
+        int left = WAIT_LIMIT;
         for (int h = tid; h < nh; h += SNT) {
             uint4 vh;
-            if (!wait_record((e & 1 ? rec1 : rec0) + h, e, vh)) {
-                lost = true;
-                break;
-            }
+            lost = !wait_record((e & 1 ? rec1 : rec0) + h, e, vh, left) || lost;
             s_x[d.rp + h] = __longlong_as_double((long long)((unsigned long long)vh.x | (unsigned long long)vh.y << 32));
         }
         __syncthreads();
@@ -854,7 +851,7 @@ template <int RPT, bool REG> __global__ void __launch_bounds__(SNT, 1) k_cg_solv
         lost = false;
         if (tid < P) {
             uint4 vt;
-            lost = !wait_record((e & 1 ? in1 : in0) + tid, e, vt);
+            lost = !wait_record((e & 1 ? in1 : in0) + tid, e, vt, left);
             tot[0] = __longlong_as_double((long long)((unsigned long long)vt.x | (unsigned long long)vt.y << 32));
         }
         if (solve_sum<SNW>(tot, sh_e, lost)) {
