@@ -445,13 +445,14 @@ __global__ void __launch_bounds__(256) k_p0_charges(DevPlan p, const T *__restri
 // are short (185 entries in the level-5 sphere's gridding matrix), by latency: a
 // lane has four (rows of 32 lanes: eight) entries in flight, then their gathers.
 // Against one at a time, evaluations: sphere5 triangles 84.9 -> 84.2 us, cube40
-// 62.1 -> 60.6, sphere5 deterministic 102.1 -> 99.4.  In FP64 only whole batches
-// are taken so: on fine grids the rows are of a few entries, and a batch's unused
-// places cost the FP64 pipe as much as used ones (deterministic level-3 sphere
-// at 512^3 4849 us with the loop alone, 4930 with all rests in batches, 4844 so;
-// cube7 at 256^3 512, 526, 515; triangles of the level-3 sphere at 256^3 651,
-// 656, 638).
-template <typename T, int LPR>
+// 62.1 -> 60.6, sphere5 deterministic 102.1 -> 99.4.  FP64 products of fewer than 16
+// entries a row (FEW: gridding matrices on fine grids) take them one by one: a
+// batch's unused places cost the FP64 pipe as much as used ones.  Deterministic,
+// one by one and in batches: level-3 sphere at 512^3 (8 entries a row) 4842 and
+// 4935 us, cube7 at 256^3 (10) 518 and 532, triangles of the level-3 sphere at
+// 256^3 (12) 639 and 657; the level-3 sphere at 256^3 (38) 679 and 674, cube13 at
+// 64^3 (hundreds) 159 and 138.
+template <typename T, int LPR, bool FEW>
 __global__ void __launch_bounds__(256) k_csr_apply(int64_t nrows, const int64_t *__restrict__ rowptr,
                                                    const int64_t *__restrict__ row_idx, const int *__restrict__ col,
                                                    const T *__restrict__ val, const T *__restrict__ x,
@@ -470,20 +471,21 @@ __global__ void __launch_bounds__(256) k_csr_apply(int64_t nrows, const int64_t 
         const int *c = col + a + sub;
         constexpr int U = LPR == 32 ? 8 : 4;
         int k = 0;
-        for (; k + LPR * U <= n; k += LPR * U) {
-            T w[U], g[U];
-            int ci[U];
+        if constexpr (!FEW)
+            for (; k + LPR * U <= n; k += LPR * U) {
+                T w[U], g[U];
+                int ci[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                ci[u] = __ldcs(c + k + LPR * u);
-                w[u] = __ldcs(v + k + LPR * u);
+                for (int u = 0; u < U; ++u) {
+                    ci[u] = __ldcs(c + k + LPR * u);
+                    w[u] = __ldcs(v + k + LPR * u);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) g[u] = x[ci[u]];
+#pragma unroll
+                for (int u = 0; u < U; ++u) acc += w[u] * g[u];
             }
-#pragma unroll
-            for (int u = 0; u < U; ++u) g[u] = x[ci[u]];
-#pragma unroll
-            for (int u = 0; u < U; ++u) acc += w[u] * g[u];
-        }
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (FEW) {
             for (; k + sub < n; k += LPR) acc += __ldcs(v + k) * x[__ldcs(c + k)];
         } else if (k < n) {
             T w[U];
@@ -553,21 +555,23 @@ cudaError_t launch_p0_charges(const DevPlan &p, const void *d_in, cudaStream_t s
     return cudaGetLastError();
 }
 
-template <typename T, int LPR>
+template <typename T, int LPR, bool FEW = false>
 static cudaError_t csr_go(int64_t nrows, const int64_t *rowptr, const int64_t *row_idx, const int *col, const void *val,
                           const void *x, void *y, cudaStream_t s) {
     const int64_t threads = nrows * LPR;
     const unsigned nb = (unsigned)((threads + 255) / 256);
-    return launch_k(k_csr_apply<T, LPR>, nb, 256, 0, s, nrows, rowptr, row_idx, col, (const T *)val, (const T *)x,
+    return launch_k(k_csr_apply<T, LPR, FEW>, nb, 256, 0, s, nrows, rowptr, row_idx, col, (const T *)val, (const T *)x,
                     (T *)y);
 }
 
-cudaError_t launch_csr_apply(int prec, int lanes_per_row, int64_t nrows, const int64_t *rowptr, const int64_t *row_idx,
-                             const int *col, const void *val, const void *x, void *y, cudaStream_t s) {
+cudaError_t launch_csr_apply(int prec, int lanes_per_row, int64_t nrows, int64_t nnz, const int64_t *rowptr,
+                             const int64_t *row_idx, const int *col, const void *val, const void *x, void *y,
+                             cudaStream_t s) {
     if (nrows == 0) return cudaSuccess;
     cudaError_t e;
     if (prec == 64)
         e = lanes_per_row >= 32 ? csr_go<double, 32>(nrows, rowptr, row_idx, col, val, x, y, s)
+            : nnz < 16 * nrows  ? csr_go<double, 8, true>(nrows, rowptr, row_idx, col, val, x, y, s)
                                 : csr_go<double, 8>(nrows, rowptr, row_idx, col, val, x, y, s);
     else
         e = lanes_per_row >= 32 ? csr_go<float, 32>(nrows, rowptr, row_idx, col, val, x, y, s)

@@ -254,7 +254,7 @@ cudaError_t launch_nmt_build(const TriBuildN &b, int pass, int prec, int64_t *co
 // element charges of NODAL_MAG input into gbuf
 cudaError_t launch_p0_charges(const DevPlan &p, const void *d_in, cudaStream_t s);
 // y[row_idx ? row_idx[i] : i] = sum over CSR row i of val * x[col]
-cudaError_t launch_csr_apply(int prec, int lanes_per_row, int64_t nrows, const int64_t *rowptr, const int64_t *row_idx,
+cudaError_t launch_csr_apply(int prec, int lanes_per_row, int64_t nrows, int64_t nnz, const int64_t *rowptr, const int64_t *row_idx,
                              const int *col, const void *val, const void *x, void *y, cudaStream_t s);
 
 // Kernel launchers (return the launch error, if any).

@@ -2542,7 +2542,7 @@ slp_status run_pipeline(slp_plan_s &p, const slp::DevPlan &d, int kind, const vo
     auto near_branch = [&](cudaStream_t t) -> slp_status {
         if (tri) {
             TRY(timed(SLOT_NEAR, t, [&] {
-                return slp::launch_csr_apply(p.prec, 32, p.N, d.nt_rowptr, nullptr, d.nt_col, d.nt_val, gch,
+                return slp::launch_csr_apply(p.prec, 32, p.N, p.nt_nnz, d.nt_rowptr, nullptr, d.nt_col, d.nt_val, gch,
                                              d.phi_part, t);
             }, "near-field matrix"));
             return SLP_OK;
@@ -2585,7 +2585,7 @@ slp_status run_pipeline(slp_plan_s &p, const slp::DevPlan &d, int kind, const vo
     }
     if (tri || det)
         TRY(timed(SLOT_SPREAD, s, [&] {
-            return slp::launch_csr_apply(p.prec, 8, d.am_rows, d.am_rowptr, d.am_row, d.am_col, d.am_val,
+            return slp::launch_csr_apply(p.prec, 8, d.am_rows, p.am_nnz, d.am_rowptr, d.am_row, d.am_col, d.am_val,
                                          tri ? gch : d.qbuf, d.gridA, s);
         }, "gridding matrix"));
     else
@@ -3106,7 +3106,7 @@ slp_status slp_eval_probe(slp_plan_t p, slp_probe_t pr, int kind, const void *d_
     const slp::DevPlan &v = pr->view;
     if (p->opts.integration) {
         const void *gch = kind == SLP_INPUT_ELEMENT ? d_in : p->dp.gbuf;
-        TRY(cuda_status(slp::launch_csr_apply(p->prec, 32, pr->n, v.nt_rowptr, nullptr, v.nt_col, v.nt_val, gch,
+        TRY(cuda_status(slp::launch_csr_apply(p->prec, 32, pr->n, pr->near_nnz, v.nt_rowptr, nullptr, v.nt_col, v.nt_val, gch,
                                               v.phi_part, s), "probe near field"));
     } else {
         TRY(cuda_status(slp::launch_near_matrix(v, nullptr, s), "probe near field"));
