@@ -1423,12 +1423,16 @@ static int col_batch(int L, int Kx, size_t celem, int64_t rows_of_blocks) {
 // triangles 129 -> 120.  More blocks even out by themselves (256^3, 500 to 1000:
 // 655 us an evaluation, 672 so), and fewer leave SMs free for each other (a plate
 // at 128^3, 25 and 60 blocks in the x and y passes, 101 and 105; at 128x64x64 84
-// and 97): both keep the early launch.
-template <typename T, typename... KArgs, typename... Args>
+// and 97): both keep the early launch, but for the forward x pass and the z pass
+// (FZ) of such plates behind a gridding product, which fills every SM to its end
+// (deterministic plate at 128x64x64 113 us, 152 with them launched early; at
+// 128^3 118, 151).
+template <typename T, bool FZ = false, typename... KArgs, typename... Args>
 static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigned threads, size_t sm, cudaStream_t s,
                                const DevPlan &p, Args... args) {
     const int yb = p.nz_act * (p.Kx / CB) * p.ks;
-    const bool even = sizeof(T) == 8 && threads >= 128 && yb >= 64 && yb <= 2 * 152;
+    const bool after_product = FZ && p.am_rowptr;
+    const bool even = sizeof(T) == 8 && threads >= 128 && (yb >= 64 || after_product) && yb <= 2 * 152;
     return launch_when(!even, kern, nb, threads, sm, s, p, args...);
 }
 
@@ -1436,17 +1440,17 @@ static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigne
 #define SLP_COL_DISPATCH(KERN, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
         case 5: { cudaError_t e_ = allow_smem(KERN<T, 5>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_pass<T>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
+                  return launch_pass<T, true>(KERN<T, 5>, NBLK, 32, SM, S, p); }                                     \
         case 6: { cudaError_t e_ = allow_smem(KERN<T, 6>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_pass<T>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
+                  return launch_pass<T, true>(KERN<T, 6>, NBLK, 64, SM, S, p); }                                     \
         case 7: { cudaError_t e_ = allow_smem(KERN<T, 7>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_pass<T>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
+                  return launch_pass<T, true>(KERN<T, 7>, NBLK, 128, SM, S, p); }                                    \
         case 8: { cudaError_t e_ = allow_smem(KERN<T, 8>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_pass<T>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
+                  return launch_pass<T, true>(KERN<T, 8>, NBLK, 256, SM, S, p); }                                    \
         case 9: { cudaError_t e_ = allow_smem(KERN<T, 9>, SM); if (e_ != cudaSuccess) return e_;               \
-                  return launch_pass<T>(KERN<T, 9>, NBLK, 512, SM, S, p); }                                    \
+                  return launch_pass<T, true>(KERN<T, 9>, NBLK, 512, SM, S, p); }                                    \
         case 10: { cudaError_t e_ = allow_smem(KERN<T, 10>, SM); if (e_ != cudaSuccess) return e_;             \
-                   return launch_pass<T>(KERN<T, 10>, NBLK, 1024, SM, S, p); }                                 \
+                   return launch_pass<T, true>(KERN<T, 10>, NBLK, 1024, SM, S, p); }                                 \
     }
 #define SLP_COL_DISPATCH2(KERN, KERNL, T, LGV, NBLK, SM, S)                                                      \
     switch (LGV) {                                                                                       \
@@ -1470,22 +1474,22 @@ static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024
 // pairs and are transformed by the fused plane passes anyway; at 1024 a pair is
 // 128 threads)
 static bool row_engine_ok(const DevPlan &p) { return p.L[0] >= 128 && p.L[0] <= 1024; }
-template <typename T, int LG> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
+template <typename T, int LG, bool FZ = false> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
     typedef RowShape<LG> Sh;
     if (p.n_row_pairs == 0) return cudaSuccess;
     const size_t sm = (size_t)(Sh::PB + 1) * Sh::L * 2 * sizeof(T);
     const cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
     const dim3 nb((unsigned)((p.n_row_pairs + Sh::PB - 1) / Sh::PB), (unsigned)p.ks);
-    const cudaError_t le = launch_pass<T>(kern, nb, Sh::NT, sm, s, p);
+    const cudaError_t le = launch_pass<T, FZ>(kern, nb, Sh::NT, sm, s, p);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) {
     if (row_engine_ok(p)) switch (__builtin_ctz(p.L[0])) {
-        case 7: return launch_rows<T, 7>(k_fx_r<T, 7>, p, s);
-        case 8: return launch_rows<T, 8>(k_fx_r<T, 8>, p, s);
-        case 9: return launch_rows<T, 9>(k_fx_r<T, 9>, p, s);
-        case 10: return launch_rows<T, 10>(k_fx_r<T, 10>, p, s);
+        case 7: return launch_rows<T, 7, true>(k_fx_r<T, 7>, p, s);
+        case 8: return launch_rows<T, 8, true>(k_fx_r<T, 8>, p, s);
+        case 9: return launch_rows<T, 9, true>(k_fx_r<T, 9>, p, s);
+        case 10: return launch_rows<T, 10, true>(k_fx_r<T, 10>, p, s);
     }
     const size_t ce = 2 * sizeof(T);
     const int PB = row_batch(p.L[0], ce);
@@ -1493,7 +1497,7 @@ template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = allow_smem(k_fx<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.n_row_pairs == 0) return cudaSuccess;
-    { const cudaError_t le = launch_pass<T>(k_fx<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T, true>(k_fx<T>, dim3((p.n_row_pairs + PB - 1) / PB, p.ks), 256, sm, s, p, PB); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 template <typename T> static cudaError_t ix_t(const DevPlan &p, cudaStream_t s) {
@@ -1557,7 +1561,7 @@ template <typename T> static cudaError_t fz_t(const DevPlan &p, cudaStream_t s) 
     cudaError_t e = allow_smem(k_fz<T>, sm);
     if (e != cudaSuccess) return e;
     if (p.nz_act == 0) return cudaSuccess;
-    { const cudaError_t le = launch_pass<T>(k_fz<T>, dim3(p.n[1] * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
+    { const cudaError_t le = launch_pass<T, true>(k_fz<T>, dim3(p.n[1] * (p.Kx / B), p.ks), 256, sm, s, p, B); if (le != cudaSuccess) return le; }
     return cudaGetLastError();
 }
 
