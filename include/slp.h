@@ -120,7 +120,7 @@ typedef struct {
                              the tolerance.  Where the grid by points cannot carry the radial kernel,
                              allow_grid_raise = 0 refuses the plan as for a given grid, and with AUTO
                              an FP64 mesh of at most 2^24 pairs and a tolerance below 1e-9 stays on
-                             that grid with the separable kernel. */
+                             that grid with the separable kernel where that is estimated cheaper. */
     int m;                /* Kaiser-Bessel half-width in grid cells; 0 = from the tolerance */
     int kernel_mode;      /* SLP_KERNEL_* */
     int near_mode;        /* SLP_NEAR_* */

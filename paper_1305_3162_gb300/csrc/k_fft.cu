@@ -1424,14 +1424,14 @@ static int col_batch(int L, int Kx, size_t celem, int64_t rows_of_blocks) {
 // 655 us an evaluation, 672 so), and fewer leave SMs free for each other (a plate
 // at 128^3, 25 and 60 blocks in the x and y passes, 101 and 105; at 128x64x64 84
 // and 97): both keep the early launch, but for the forward x pass and the z pass
-// (FZ) of such plates behind a gridding product, which fills every SM to its end
+// (XZ) of such plates behind a gridding product, which fills every SM to its end
 // (deterministic plate at 128x64x64 113 us, 152 with them launched early; at
 // 128^3 118, 151).
-template <typename T, bool FZ = false, typename... KArgs, typename... Args>
+template <typename T, bool XZ = false, typename... KArgs, typename... Args>
 static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigned threads, size_t sm, cudaStream_t s,
                                const DevPlan &p, Args... args) {
     const int yb = p.nz_act * (p.Kx / CB) * p.ks;
-    const bool after_product = FZ && p.am_rowptr;
+    const bool after_product = XZ && p.am_rowptr;
     const bool even = sizeof(T) == 8 && threads >= 128 && (yb >= 64 || after_product) && yb <= 2 * 152;
     return launch_when(!even, kern, nb, threads, sm, s, p, args...);
 }
@@ -1474,14 +1474,14 @@ static bool col_engine_ok(const DevPlan &p, int L) { return L >= 32 && L <= 1024
 // pairs and are transformed by the fused plane passes anyway; at 1024 a pair is
 // 128 threads)
 static bool row_engine_ok(const DevPlan &p) { return p.L[0] >= 128 && p.L[0] <= 1024; }
-template <typename T, int LG, bool FZ = false> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
+template <typename T, int LG, bool XZ = false> static cudaError_t launch_rows(void (*kern)(DevPlan), const DevPlan &p, cudaStream_t s) {
     typedef RowShape<LG> Sh;
     if (p.n_row_pairs == 0) return cudaSuccess;
     const size_t sm = (size_t)(Sh::PB + 1) * Sh::L * 2 * sizeof(T);
     const cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
     const dim3 nb((unsigned)((p.n_row_pairs + Sh::PB - 1) / Sh::PB), (unsigned)p.ks);
-    const cudaError_t le = launch_pass<T, FZ>(kern, nb, Sh::NT, sm, s, p);
+    const cudaError_t le = launch_pass<T, XZ>(kern, nb, Sh::NT, sm, s, p);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 template <typename T> static cudaError_t fx_t(const DevPlan &p, cudaStream_t s) {

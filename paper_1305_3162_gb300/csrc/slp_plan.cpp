@@ -408,7 +408,16 @@ slp_status expsum_params(slp_plan_s &p) {
 // sphere4 at 64^3 1.3e-6 -> 2.6e-7, plate100 1.4e-6 -> 4.0e-7, for 1 to 4 us.
 constexpr double AUTO_SPLIT = 0.3;
 
-bool cheapest_grid(const slp_plan_s &p, double c, int out[3]) {
+// An evaluation's estimated far field, us: grid points of the passes' active
+// regions (act per axis) at the rates above.
+double far_cost(const slp_plan_s &p, const int L[3], const double act[3]) {
+    const double kx = 0.25 * L[0];
+    const double fx = act[1] * act[2] * L[0], fy = act[2] * kx * L[1], fz = 0.5 * L[1] * kx * L[2];
+    return p.prec == 64 ? 120.0 + 4e-5 * fx + 1.2e-4 * fy + 9e-5 * fz : 32.0 + 6.6e-6 * fx + 7.4e-6 * fy + 5.4e-6 * fz;
+}
+
+// cost: the chosen grid's estimate, us
+bool cheapest_grid(const slp_plan_s &p, double c, int out[3], double &cost) {
     const bool f64 = p.prec == 64;
     const double dmax = std::max(p.D[0], std::max(p.D[1], p.D[2]));
     // distances from up to 32 vertices to up to 32768
@@ -442,9 +451,7 @@ bool cheapest_grid(const slp_plan_s &p, double c, int out[3]) {
         radial_params(q, c);
         double act[3];  // grid points the body and its window span
         for (int d = 0; d < 3; ++d) act[d] = std::min<double>(L[d], p.D[d] / q.P[d] * L[d] + 2 * p.m);
-        const double kx = 0.25 * L[0];
-        const double fx = act[1] * act[2] * L[0], fy = act[2] * kx * L[1], fz = n[1] * kx * L[2];
-        const double far = f64 ? 120.0 + 4e-5 * fx + 1.2e-4 * fy + 9e-5 * fz : 32.0 + 6.6e-6 * fx + 7.4e-6 * fy + 5.4e-6 * fz;
+        const double far = far_cost(p, L, act);
         int64_t in = 0;
         for (double d2 : dist) in += d2 < q.eps * q.eps;
         const double share = (double)in / ((double)nt * nv);
@@ -457,7 +464,18 @@ bool cheapest_grid(const slp_plan_s &p, double c, int out[3]) {
             for (int d = 0; d < 3; ++d) out[d] = L[d];
         }
     }
+    cost = best;
     return best < 1e300;
+}
+
+// The same estimate for the separable kernel on grid L (FP64): a dense nodal
+// operator, and for charges at the points, at a tenth, every pair's series (0.07
+// ns a pair and term: plate of 22 cells, 151k pairs of 40 terms, 416 us).
+double separable_cost(const slp_plan_s &p, const int L[3]) {
+    const double act[3] = {(double)L[0], (double)L[1], (double)L[2]};
+    const double terms = 0.25 * (L[0] + L[1] + L[2]), n = (double)p.N, q = (double)p.Q;
+    const bool fly = p.opts.near_mode == SLP_NEAR_ON_THE_FLY;
+    return far_cost(p, L, act) + (fly ? 0.0 : n * n * 32.0 / 6.5e6) + (fly ? 1.0 : 0.1) * n * q * 7e-5 * terms;
 }
 
 // The automatic axes (L < 0) by the number of points: equal spacing at about
@@ -526,26 +544,36 @@ slp_status choose_parameters(slp_plan_s &p) {
     bool by_cost = L[0] < 0 && L[1] < 0 && L[2] < 0 && !p.opts.integration &&
                    (mode == SLP_KERNEL_AUTO || mode == SLP_KERNEL_RADIAL);
     if (by_cost) {
-        // Where the grid by points cannot carry the radial kernel: a plan that may
-        // not raise its grid stays refused, and a small FP64 mesh whose tolerance is
-        // below SEPARABLE_TOL stays on that grid with the separable kernel, which has
-        // no split error (1e-16 where the radial kernel spends its share of the
-        // tolerance) and transforms a grid of half or a quarter of the points per
-        // axis.  Evaluations with one point a triangle, us, radial and separable:
-        // 42 vertices 68 and 51, 56 of a cube 67 and 51, 252 of a plate 73 and 61,
-        // 119 of a torus 83 and 60 at 1e-10; 119 and 52, 119 and 52, 170 and 66, 253
-        // and 62 at 1e-13.  Looser tolerances take the radial kernel
-        // at every size (the torus 82 at 1e-9).
-        int Lp[3] = {-1, -1, -1};
+        // Where the grid by points cannot carry the radial kernel, a plan that may not
+        // raise its grid stays refused.  A small FP64 mesh whose tolerance is below
+        // SEPARABLE_TOL stays on that grid with the separable kernel where that is
+        // estimated cheaper than the cheapest radial one: it has no split error (1e-16
+        // where the radial kernel spends its share of the tolerance) and transforms a
+        // grid of half or a quarter of the points per axis, but sums every pair.
+        // Nodal evaluations with one point a triangle, us, radial and separable:
+        // 42 vertices 68 and 51, 56 of a cube 67 and 51, 119 of a torus 83 and 60 at
+        // 1e-10; 119 and 52, 119 and 52, 253 and 62 at 1e-13.  Charges at the points of
+        // a plate of 276 vertices, 1e-10: 98 and 477, so that one stays radial.  Looser
+        // tolerances take the radial kernel at every size (the torus 82 at 1e-9).
+        int Lp[3] = {-1, -1, -1}, Lr[3];
         grid_by_points(p, Lp);
         const int np[3] = {Lp[0] / 2, Lp[1] / 2, Lp[2] / 2};
-        if (!radial_feasible(p, np, std::sqrt(2.0 * std::log(1.0 / std::min(0.1, p.tol * KFAC)))))
-            by_cost = mode == SLP_KERNEL_AUTO && separable_size ? p.tol >= SEPARABLE_TOL : p.opts.allow_grid_raise != 0;
+        if (!radial_feasible(p, np, std::sqrt(2.0 * std::log(1.0 / std::min(0.1, p.tol * KFAC))))) {
+            if (mode != SLP_KERNEL_AUTO || !separable_size) {
+                by_cost = p.opts.allow_grid_raise != 0;
+            } else if (p.tol < SEPARABLE_TOL) {
+                p.split_share = AUTO_SPLIT;
+                const double ca = std::sqrt(2.0 * std::log(1.0 / std::min(0.1, p.tol * AUTO_SPLIT * KFAC)));
+                double cost = 0.0;
+                by_cost = cheapest_grid(p, ca, Lr, cost) && cost < separable_cost(p, Lp);
+            }
+        }
     }
     p.split_share = by_cost ? AUTO_SPLIT : 1.0;
     double tk = std::min(0.1, p.tol * p.split_share * KFAC);
     double c = std::sqrt(2.0 * std::log(1.0 / tk));
-    if (by_cost && !cheapest_grid(p, c, L)) {
+    double cost = 0.0;
+    if (by_cost && !cheapest_grid(p, c, L, cost)) {
         p.split_share = 1.0;
         tk = std::min(0.1, p.tol * KFAC);
         c = std::sqrt(2.0 * std::log(1.0 / tk));
