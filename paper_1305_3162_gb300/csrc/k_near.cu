@@ -675,9 +675,10 @@ template <typename T, int K> __global__ void __launch_bounds__(128) k_near_matri
 #pragma unroll(sizeof(T) == 8 ? 1 : CHUNK / (32 * U))
             for (int h = 0; h < CHUNK; h += 32 * U)
                 near_batch<T, K, U, true>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
+        constexpr int UT = K == 2 ? 2 : U;  // two states, small meshes: 126 us in batches of two, 128 of four
 #pragma unroll 1
-        for (int h = 0; h < CHUNK && j + h < n; h += 32 * U)
-            near_batch<T, K, U, false>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
+        for (int h = 0; h < CHUNK && j + h < n; h += 32 * UT)
+            near_batch<T, K, UT, false>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
     }
     // lane r of the group's first warp ends up with row r
     T v[K];
