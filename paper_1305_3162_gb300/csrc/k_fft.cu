@@ -1430,9 +1430,9 @@ static int col_batch(int L, int Kx, size_t celem, int64_t rows_of_blocks) {
 template <typename T, bool XZ = false, typename... KArgs, typename... Args>
 static cudaError_t launch_pass(void (*kern)(DevPlan, KArgs...), dim3 nb, unsigned threads, size_t sm, cudaStream_t s,
                                const DevPlan &p, Args... args) {
-    const int yb = p.nz_act * (p.Kx / CB) * p.ks;
+    const int yb = p.nz_act * (p.Kx / CB);  // of a state
     const bool after_product = XZ && p.am_rowptr;
-    const bool even = sizeof(T) == 8 && threads >= 128 && (yb >= 64 || after_product) && yb <= 2 * 152;
+    const bool even = sizeof(T) == 8 && threads >= 128 && (yb >= 64 || after_product) && yb * p.ks <= 2 * 152;
     return launch_when(!even, kern, nb, threads, sm, s, p, args...);
 }
 

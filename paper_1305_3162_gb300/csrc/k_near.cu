@@ -649,10 +649,12 @@ __device__ __forceinline__ void near_batch(const int *__restrict__ col, const ty
 template <typename T, int K> __global__ void __launch_bounds__(128) k_near_matrix(DevPlan p, int split) {
     typedef typename VecT<T>::T4 T4;
     // entries in flight per lane: a chunk in one batch, or for four and eight states
-    // (registers) and FP64 in two, unrolled in FP32.  With two a batch and a loop
-    // over batches, torus400 with 2 to 8 states 287, 328, 382, 449, 500, 573, 642 us
-    // an evaluation; so 260, 296, 365, 403, 472, 500, 570
-    constexpr int U = K == 1 || (sizeof(T) == 4 && K != 4 && K != 8) ? 4 : 2;
+    // (registers) in two, unrolled.  With two a batch and a loop over batches,
+    // torus400 with 2 to 8 states 287, 328, 382, 449, 500, 573, 642 us an evaluation;
+    // so 260, 296, 365, 403, 472, 500, 570.  FP64, whose pipe the far field beside it
+    // needs: two, or one from seven states on (a 10x10 cube with 4, 7 and 8 states
+    // 469, 645 and 740 us with two, 486, 628 and 731 with one).
+    constexpr int U = K == 1 ? 4 : sizeof(T) == 8 ? (K < 7 ? 2 : 1) : K == 4 || K == 8 ? 2 : 4;
     __shared__ T part[4][K * NM_ROWS];
     pdl_wait();
     pdl_trigger();
@@ -672,10 +674,10 @@ template <typename T, int K> __global__ void __launch_bounds__(128) k_near_matri
         const T4 *val = (const T4 *)p.nm_val + e0 + lane;
         int j = CHUNK * sub;
         for (; j + CHUNK <= n; j += CHUNK * split)
-#pragma unroll(sizeof(T) == 8 ? 1 : CHUNK / (32 * U))
+#pragma unroll(sizeof(T) == 8 ? 1 : 2)
             for (int h = 0; h < CHUNK; h += 32 * U)
                 near_batch<T, K, U, true>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
-        constexpr int UT = K == 2 ? 2 : U;  // two states, small meshes: 126 us in batches of two, 128 of four
+        constexpr int UT = sizeof(T) == 4 && K == 2 ? 2 : U;  // two states, small meshes: 126 us in batches of two, 128 of four
 #pragma unroll 1
         for (int h = 0; h < CHUNK && j + h < n; h += 32 * UT)
             near_batch<T, K, UT, false>(col, val, p.nm_stride, j + h, n, lane, m4, p.N, acc);
