@@ -548,9 +548,9 @@ __global__ void k_loop_inner_next(FemDev d, cudaGraphConditionalHandle h, int bo
 // parts.  The inner iteration stops when r . u has fallen by 1e-8 (the
 // residual by 1e-4 in the preconditioner's norm).
 //
-// Measured, phi_1 (load, solve and all corrections): ball n = 16 672 -> 319 us,
+// Measured, phi_1 (load, solve and all corrections): ball n = 16 672 -> 281 us,
 // n = 32 2155 -> 760 us (5.2 us a step: about 2.2 exchange, 0.9 product, the
-// rest the coarse correction, sums and barriers), n = 48 7600 -> 5600 us (its
+// rest the coarse correction, sums and barriers), n = 48 7600 -> 5460 us (its
 // matrix no longer fits the registers).  The line to the launch chain: a step is
 // the slower here from n = 44 on (its matrix comes from L2 to half as many warps),
 // but half as many steps are needed.  Chain and one launch, ms: n = 48 (436k
